@@ -14,16 +14,11 @@
 //      not depend on scheduling).
 //   2. chol_kernel: semi-definite Cholesky in shared memory; a pivot at or
 //      below d_head * eps * max(diag) leaves a zero column (rank deficiency).
-//   3. er_kernel: A = L_K^T L_Q, then one-sided (Hestenes) Jacobi: pairs of
-//      columns are rotated until every pair is orthogonal to d_head * eps,
-//      with the round-robin ordering so the d_head / 2 pairs of a round
-//      are disjoint; the singular values are the column norms. Values at or
-//      below sigma_max * d_model * eps are the zeros of a rank-deficient
-//      M_h and are dropped (Eq. 4 sums over nonzero values); ER (Eq. 4) is
-//      exp of the entropy of the normalised singular values. FP64 is slow
-//      on this part, so a pair costs one fp64 dot product and the column
-//      update: squared norms are carried in shared memory (exact again at
-//      each sweep), and the angle is formed in fp32 (any angle is exact).
+//   3. bidiag_kernel: A = L_K^T L_Q and its bidiagonal form; svals_kernel:
+//      its singular values. Values at or below sigma_max * d_model * eps are
+//      the zeros of a rank-deficient M_h and are dropped (Eq. 4 sums over
+//      nonzero values); ER (Eq. 4) is exp of the entropy of the normalised
+//      singular values.
 //   4. classify_kernel: per layer, group score = mean ER of the group's
 //      query heads; the k = ceil((100 - s) * groups / 100) lowest groups
 //      (stable order, ties to the lower index) are retrieval, the rest
@@ -47,7 +42,6 @@ constexpr int kGT = 64;              // Gram output tile
 constexpr int kGK = 32;              // d_model columns per step
 constexpr int kGramThreads = 256;
 constexpr int kMatThreads = 256;
-constexpr int kMaxSweeps = 40;
 
 // Matrices are numbered layer-major: layer l's query projections, then its
 // key projections (nmat = Hq + Hkv per layer).
@@ -160,109 +154,239 @@ __global__ void __launch_bounds__(kMatThreads) chol_kernel(const double* part, i
   }
 }
 
-// Round-robin tournament: pair k of round r among n (even) columns.
-__device__ __forceinline__ void rr_pair(int n, int r, int k, int& p, int& q) {
-  if (k == 0) {
-    p = n - 1;
-    q = r;
-  } else {
-    p = (r + k) % (n - 1);
-    q = (r - k + n - 1) % (n - 1);
-  }
-}
-
 // Warp sum of a double (every lane gets it).
 __device__ __forceinline__ double warp_sum(double v) {
   for (int o = 16; o >= 1; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
   return v;
 }
 
-// One query head per CTA (blockIdx.x = layer * Hq + head): A = L_K^T L_Q,
-// one-sided Jacobi, ER.
-__global__ void __launch_bounds__(kMatThreads) er_kernel(const double* L, int Hq, int Hkv, int dh, int dm,
-                                                         double* er, int* sweeps_out) {
-  extern __shared__ double A[];  // column-major: column c at A + c * dh; then dh squared norms
-  __shared__ double red[32];
-  __shared__ int rotated;
+// Singular values of one query head's A = L_K^T L_Q need no vectors, so A is
+// reduced to bidiagonal form by Householder reflections (Golub & Kahan 1965;
+// 8/3 n^3 flops) and svals_kernel finds the n values of the bidiagonal. The
+// one-sided Jacobi iteration that stood here spent about 10 sweeps of 10 n^3
+// flops each: 240 ms for 784 heads of 128. The reduction now takes 9.7 ms (its
+// 4.4 GFLOP and the product's 1.5 cost 5 ms at the 1.2 TFLOP/s the fp64 pipe
+// gives; the rest is the chain of 256 reflectors a head and the sixth, mostly
+// empty, wave of heads) and the values 22 ms.
+//
+// One CTA per head, 4 N threads, A row-major in shared memory with N + 1
+// doubles a row, so that neither a row nor a column walk meets a bank
+// conflict; lanes lie along the columns for the left reflections and along
+// the rows for the right ones, the four thread groups split the other index,
+// and a product's four partial sums meet in shared memory (a warp shuffle
+// reduction would cost as many fp64 adds as the product itself). The pipe
+// issues two fp64 FMAs a clock, so shared memory (one load per FMA) keeps up.
+// A reflector H = I - c v v^T, c = 1 / (beta (beta - alpha)), keeps v in place
+// of the eliminated entries with only its first entry stored apart.
+template <int N>
+struct BidiagCfg {
+  static constexpr int LD = N + 1;
+  static constexpr int THREADS = 4 * N;
+  static constexpr int SMEM = (N * LD + 4 * N) * 8;
+};
+
+// The reflector that maps x = (alpha, rest), |rest|^2 = sig, to (beta, 0):
+// head[0] = beta, head[1] = first entry of v, head[2] = c (0: nothing to do).
+__device__ __forceinline__ void make_reflector(double alpha, double sig, double* head) {
+  if (sig == 0.0) {
+    head[0] = alpha;
+    head[1] = 0.0;
+    head[2] = 0.0;
+  } else {
+    const double mu = sqrt(fma(alpha, alpha, sig));
+    const double beta = alpha > 0.0 ? -mu : mu;
+    head[0] = beta;
+    head[1] = alpha - beta;
+    head[2] = 1.0 / (beta * (beta - alpha));
+  }
+}
+
+template <int N>
+__global__ void __launch_bounds__(4 * N) bidiag_kernel(const double* L, int Hq, int Hkv, double* diag, double* sup) {
+  using C = BidiagCfg<N>;
+  constexpr int LD = C::LD, R = N / 4;
+  extern __shared__ double A[];  // row i, column j at A[i * LD + j]
+  double* part = A + N * LD;     // [4][N] partial products
+  __shared__ double head[2][3];  // the left and the right reflector
   const int hg = blockIdx.x, l = hg / Hq, h = hg % Hq, kv = h / (Hq / Hkv);
-  const size_t n2 = (size_t)dh * dh;
+  const size_t n2 = (size_t)N * N;
   const double* Lq = L + ((size_t)l * (Hq + Hkv) + h) * n2;
   const double* Lk = L + ((size_t)l * (Hq + Hkv) + Hq + kv) * n2;
-  double* nrm2 = A + n2;
-  for (int e = threadIdx.x; e < dh * dh; e += kMatThreads) {
-    const int i = e % dh, j = e / dh;  // A[i][j] = sum_m Lk[m][i] Lq[m][j] over m >= max(i, j)
-    double s = 0.0;
-    for (int mm = max(i, j); mm < dh; ++mm) s = fma(Lk[(size_t)mm * dh + i], Lq[(size_t)mm * dh + j], s);
-    A[(size_t)j * dh + i] = s;
+  const int x = threadIdx.x % N, g = threadIdx.x / N, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+
+  {
+    // column x, rows R g .. R g + R - 1 of A = L_K^T L_Q; both factors are
+    // lower triangular, so the sum starts at the larger of the two blocks
+    double acc[R];
+#pragma unroll
+    for (int i = 0; i < R; ++i) acc[i] = 0.0;
+    for (int m = max(R * g, x & ~31); m < N; ++m) {
+      const double b = Lq[(size_t)m * N + x];
+      const double2* a = reinterpret_cast<const double2*>(Lk + (size_t)m * N + R * g);
+#pragma unroll
+      for (int i = 0; i < R / 2; ++i) {
+        const double2 v = a[i];
+        acc[2 * i] = fma(v.x, b, acc[2 * i]);
+        acc[2 * i + 1] = fma(v.y, b, acc[2 * i + 1]);
+      }
+    }
+#pragma unroll
+    for (int i = 0; i < R; ++i) A[(R * g + i) * LD + x] = acc[i];
   }
   __syncthreads();
 
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  constexpr int kWarps = kMatThreads / 32;
-  // a pair counts as orthogonal once |a_p . a_q| <= d_head * eps * |a_p| |a_q|
-  // (the rounding level of a length-d_head dot product), tested squared
-  const double rot_tol2 = (dh * DBL_EPSILON) * (dh * DBL_EPSILON);
-  int sweep = 0;
-  for (; sweep < kMaxSweeps; ++sweep) {
-    // squared column norms, exact at the start of each sweep and carried
-    // through its rotations
-    for (int c = threadIdx.x; c < dh; c += kMatThreads) {
-      const double* a = A + (size_t)c * dh;
-      double s2 = 0.0;
-      for (int i = 0; i < dh; ++i) s2 = fma(a[i], a[i], s2);
-      nrm2[c] = s2;
+  for (int k = 0; k < N; ++k) {
+    // left: column k, rows k .. N - 1
+    if (warp == 0) {
+      double s = 0.0;
+      for (int i = k + 1 + lane; i < N; i += 32) s = fma(A[i * LD + k], A[i * LD + k], s);
+      s = warp_sum(s);
+      if (lane == 0) {
+        make_reflector(A[k * LD + k], s, head[0]);
+        diag[(size_t)hg * N + k] = head[0][0];
+      }
     }
-    if (threadIdx.x == 0) rotated = 0;
     __syncthreads();
-    for (int r = 0; r < dh - 1; ++r) {
-      for (int k = warp; k < dh / 2; k += kWarps) {
-        int p, q;
-        rr_pair(dh, r, k, p, q);
-        double* ap = A + (size_t)p * dh;
-        double* aq = A + (size_t)q * dh;
-        const double al = nrm2[p], be = nrm2[q];
-        double ga = 0.0;
-        for (int i = lane; i < dh; i += 32) ga = fma(ap[i], aq[i], ga);
-        ga = warp_sum(ga);
-        if (ga != 0.0 && ga * ga > rot_tol2 * al * be) {
-          // The angle only steers convergence: any (c, s) with c^2 + s^2 = 1
-          // to fp64 precision is an exact orthogonal transform, so tan is
-          // formed in fp32 and c, s from it in fp64.
-          const float zeta = (float)(be - al) / (2.0f * (float)ga);
-          const float tf = fabsf(zeta) > 1e18f ? 0.5f / zeta
-                                               : copysignf(1.0f, zeta) / (fabsf(zeta) + sqrtf(1.0f + zeta * zeta));
-          const double t = tf;
-          const double c = rsqrt(1.0 + t * t), s = c * t;
-          for (int i = lane; i < dh; i += 32) {
-            const double x = ap[i], y = aq[i];
-            ap[i] = fma(c, x, -s * y);
-            aq[i] = fma(s, x, c * y);
-          }
-          if (lane == 0) {
-            const double cc = c * c, ss = s * s, cs2 = 2.0 * c * s * ga;
-            nrm2[p] = fmax(fma(cc, al, fma(ss, be, -cs2)), 0.0);
-            nrm2[q] = fmax(fma(ss, al, fma(cc, be, cs2)), 0.0);
-            rotated = 1;
-          }
-        }
+    const int j = k + 1 + x;  // the column this thread updates
+    double c = head[0][2], v0 = head[0][1];
+    if (c != 0.0) {
+      if (j < N) {
+        double s = g == 0 ? v0 * A[k * LD + j] : 0.0;
+        for (int i = k + 1 + g; i < N; i += 4) s = fma(A[i * LD + k], A[i * LD + j], s);
+        part[g * N + x] = s;
+      }
+      __syncthreads();
+      if (j < N) {
+        const double w = -c * ((part[x] + part[N + x]) + (part[2 * N + x] + part[3 * N + x]));
+        if (g == 0) A[k * LD + j] = fma(v0, w, A[k * LD + j]);
+        for (int i = k + 1 + g; i < N; i += 4) A[i * LD + j] = fma(A[i * LD + k], w, A[i * LD + j]);
       }
       __syncthreads();
     }
-    const int any = rotated;
+    if (k + 1 >= N) break;
+    // right: row k, columns k + 1 .. N - 1
+    if (warp == 0) {
+      double s = 0.0;
+      for (int i = k + 2 + lane; i < N; i += 32) s = fma(A[k * LD + i], A[k * LD + i], s);
+      s = warp_sum(s);
+      if (lane == 0) {
+        make_reflector(A[k * LD + k + 1], s, head[1]);
+        sup[(size_t)hg * N + k] = head[1][0];
+      }
+    }
     __syncthreads();
-    if (!any) break;
+    c = head[1][2];
+    v0 = head[1][1];
+    if (c != 0.0) {
+      const int r = k + 1 + x;  // the row this thread updates
+      const double* u = A + k * LD;
+      if (r < N) {
+        double s = g == 0 ? v0 * A[r * LD + k + 1] : 0.0;
+        for (int i = k + 2 + g; i < N; i += 4) s = fma(u[i], A[r * LD + i], s);
+        part[g * N + x] = s;
+      }
+      __syncthreads();
+      if (r < N) {
+        const double w = -c * ((part[x] + part[N + x]) + (part[2 * N + x] + part[3 * N + x]));
+        if (g == 0) A[r * LD + k + 1] = fma(v0, w, A[r * LD + k + 1]);
+        for (int i = k + 2 + g; i < N; i += 4) A[r * LD + i] = fma(u[i], w, A[r * LD + i]);
+      }
+    }
+    __syncthreads();
   }
+}
 
-  // singular values = column norms; ER over the nonzero ones (Eq. 4)
-  double nrm = 0.0;
-  if (threadIdx.x < dh) {
-    const double* a = A + (size_t)threadIdx.x * dh;
-    for (int i = 0; i < dh; ++i) nrm = fma(a[i], a[i], nrm);
-    nrm = sqrt(nrm);
+// Singular values of each head's bidiagonal matrix B and its ER; one CTA of N
+// threads per head, thread j finds the j-th smallest value. With q_i = d_i^2
+// and f_i = e_i^2, the stationary qd transform (Fernando & Parlett 1994)
+//   delta_i = q_i + t_i, t_0 = -s, t_{i+1} = t_i f_i / delta_i - s
+// has as many negative delta_i as B^T B has eigenvalues below s, to high
+// relative accuracy, and sum_i delta_i' / delta_i is p'(s) / p(s) of its
+// characteristic polynomial. The N threads first count at N points spread
+// over [0, bound], which brackets every value to a part in N, then each
+// thread bisects until its bracket holds one value and takes Newton steps
+// inside the bracket, which the count that each evaluation gives keeps
+// shrinking. The values are wanted to absolute accuracy (ER weights them by
+// their share of the sum): a bracket of 2^-53 of the bound ends the search.
+template <int N>
+__global__ void __launch_bounds__(N) svals_kernel(const double* diag, const double* sup, int dm, double* er) {
+  __shared__ double2 qf[N];  // (q_i, f_i)
+  __shared__ double red[32];
+  __shared__ int cnt[N];
+  const int hg = blockIdx.x, j = threadIdx.x;
+  const double d = fabs(diag[(size_t)hg * N + j]);
+  const double e = j + 1 < N ? fabs(sup[(size_t)hg * N + j]) : 0.0;
+  const double ep = j > 0 ? fabs(sup[(size_t)hg * N + j - 1]) : 0.0;
+  // sigma_max <= sqrt(|B|_1 |B|_inf) <= bound
+  const double bound = block_max(fmax(d + e, d + ep), red);
+  if (!(bound > 0.0)) {
+    if (j == 0) er[hg] = 1.0;  // exp of an empty sum
+    return;
   }
-  const double smax = block_max(threadIdx.x < dh ? nrm : 0.0, red);
-  const double tol = smax * (double)max(dm, dh) * DBL_EPSILON;
-  const bool keep = threadIdx.x < dh && nrm > tol;
+  const double inv_b = 1.0 / bound;
+  qf[j] = make_double2((d * inv_b) * (d * inv_b), (e * inv_b) * (e * inv_b));
+  __syncthreads();
+  double g;  // p'(s) / p(s) at the last point
+  auto count = [&](double s) {
+    int c = 0;
+    double t = -s, tp = -1.0;
+    g = 0.0;
+#pragma unroll 4
+    for (int i = 0; i < N; ++i) {
+      const double2 v = qf[i];
+      double del = v.x + t;
+      if (fabs(del) < 1e-280) del = -1e-280;
+      c += del < 0.0;
+      const double inv = 1.0 / del;
+      const double r = v.y * inv, u = tp * inv;
+      g += u;
+      t = fma(r, t, -s);
+      tp = fma(r * v.x, u, -1.0);
+    }
+    return c;
+  };
+  double x = (double)(j + 1) / (N + 1);
+  cnt[j] = count(x * x);
+  __syncthreads();
+  double lo = 0.0, hi = 1.0 + 1e-9;
+  int nlo = 0, nhi = N;
+  for (int i = 0; i < N; ++i) {
+    const double p = (double)(i + 1) / (N + 1);
+    if (cnt[i] <= j && p > lo) {
+      lo = p;
+      nlo = cnt[i];
+    }
+  }
+  for (int i = N - 1; i >= 0; --i) {
+    const double p = (double)(i + 1) / (N + 1);
+    if (cnt[i] > j && p < hi && p > lo) {
+      hi = p;
+      nhi = cnt[i];
+    }
+  }
+  x = 0.5 * (lo + hi);
+  bool done = false;
+  for (int round = 0; round < 120 && !__syncthreads_and(done); ++round) {
+    const int c = count(x * x);  // done threads repeat their last point
+    if (done) continue;
+    if (c <= j) {
+      lo = x;
+      nlo = c;
+    } else {
+      hi = x;
+      nhi = c;
+    }
+    const double mid = 0.5 * (lo + hi);
+    const double xn = x - 1.0 / (2.0 * x * g);
+    // every fourth round halves the bracket whatever Newton says
+    const bool newton = nhi - nlo == 1 && (round & 3) != 3 && xn > lo && xn < hi;
+    done = hi - lo < 1.2e-16 || hi < 1e-15 || (newton && fabs(xn - x) < 4e-15);
+    x = newton ? xn : mid;
+  }
+  const double nrm = x * bound;
+  const double smax = block_max(nrm, red);
+  const double tol = smax * (double)max(dm, N) * DBL_EPSILON;
+  const bool keep = nrm > tol;
   const double total = block_sum(keep ? nrm : 0.0, red);
   double ent = 0.0;
   if (keep) {
@@ -270,10 +394,7 @@ __global__ void __launch_bounds__(kMatThreads) er_kernel(const double* L, int Hq
     ent = -p * log(p);
   }
   ent = block_sum(ent, red);
-  if (threadIdx.x == 0) {
-    er[hg] = exp(ent);
-    sweeps_out[hg] = sweep;
-  }
+  if (j == 0) er[hg] = exp(ent);
 }
 
 // One layer per block (blockIdx.x), one thread.
@@ -340,23 +461,24 @@ extern "C" aoh_status aoh_classify(const void* w_q, const void* w_k, int32_t n_l
   const int span = ((d_model + nsplit - 1) / nsplit + kGK - 1) / kGK * kGK;
   nsplit = (d_model + span - 1) / span;
   const size_t n2 = (size_t)dh * dh;
-  const size_t bytes = ((size_t)nsplit * nall * n2 + (size_t)nall * n2 + nq) * sizeof(double) + nq * sizeof(int) +
+  // Gram parts, factors, bidiagonals, ER; labels
+  const size_t bytes = ((size_t)nsplit * nall * n2 + (size_t)nall * n2 + 2 * (size_t)nq * dh + nq) * sizeof(double) +
                        (size_t)n_layers * n_kv_heads + 64;
   void* scratch = nullptr;
   e = cudaMallocAsync(&scratch, bytes, s);
   if (e != cudaSuccess) return fail(AOH_ERR_CUDA, "aoh_classify: cudaMallocAsync failed");
   double* part = static_cast<double*>(scratch);
   double* L = part + (size_t)nsplit * nall * n2;
-  double* er = L + (size_t)nall * n2;
-  int* sweeps = reinterpret_cast<int*>(er + nq);
-  uint8_t* labels = reinterpret_cast<uint8_t*>(sweeps + nq);
+  double* diag = L + (size_t)nall * n2;
+  double* sup = diag + (size_t)nq * dh;
+  double* er = sup + (size_t)nq * dh;
+  uint8_t* labels = reinterpret_cast<uint8_t*>(er + nq);
   const int smem = (int)(n2 * sizeof(double));
-  const int smem_er = (int)((n2 + dh) * sizeof(double));
   static bool attr_set = false;
   if (!attr_set) {
     e = cudaFuncSetAttribute(chol_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 128 * 128 * 8);
     if (e == cudaSuccess)
-      e = cudaFuncSetAttribute(er_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (128 * 128 + 128) * 8);
+      e = cudaFuncSetAttribute(bidiag_kernel<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, BidiagCfg<128>::SMEM);
     if (e != cudaSuccess) {
       cudaFreeAsync(scratch, s);
       return fail(AOH_ERR_CUDA, "aoh_classify: cudaFuncSetAttribute failed");
@@ -367,7 +489,13 @@ extern "C" aoh_status aoh_classify(const void* w_q, const void* w_k, int32_t n_l
                                                                           static_cast<const bf16*>(w_k), n_q_heads,
                                                                           n_kv_heads, nall, dh, d_model, span, part);
   chol_kernel<<<nall, kMatThreads, smem, s>>>(part, nsplit, nall, dh, L);
-  er_kernel<<<nq, kMatThreads, smem_er, s>>>(L, n_q_heads, n_kv_heads, dh, d_model, er, sweeps);
+  if (dh == 128) {
+    bidiag_kernel<128><<<nq, 512, BidiagCfg<128>::SMEM, s>>>(L, n_q_heads, n_kv_heads, diag, sup);
+    svals_kernel<128><<<nq, 128, 0, s>>>(diag, sup, d_model, er);
+  } else {
+    bidiag_kernel<64><<<nq, 256, BidiagCfg<64>::SMEM, s>>>(L, n_q_heads, n_kv_heads, diag, sup);
+    svals_kernel<64><<<nq, 64, 0, s>>>(diag, sup, d_model, er);
+  }
   classify_kernel<<<n_layers, 32, 0, s>>>(er, n_q_heads, n_kv_heads, sparsity_pct, labels);
   e = cudaGetLastError();
   if (e == cudaSuccess)

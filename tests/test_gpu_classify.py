@@ -158,3 +158,40 @@ def test_layers_in_one_call():
         want = oer.head_scores(wq[l], wk[l], Hkv)
         np.testing.assert_allclose(ers[l], want, rtol=1e-9)
         _check_labels(np.array(labels[l]), np.array(ers[l]), want, Hkv, 50)
+
+
+def _er_by_svd(wq, wk):
+    """ER of every head from a float64 SVD of M_h = W_K^T W_Q itself."""
+    Hq, g = len(wq), len(wq) // len(wk)
+    out = np.empty(Hq)
+    for h in range(Hq):
+        s = np.linalg.svd(wk[h // g].T @ wq[h], compute_uv=False)
+        s = s[s > s[0] * max(wq.shape[1:]) * np.finfo(np.float64).eps] if s[0] > 0 else s[:0]
+        p = s / s.sum() if s.size else s
+        out[h] = math.exp(-(p * np.log(p)).sum())
+    return out
+
+
+@pytest.mark.parametrize("dh", [64, 128])
+def test_spectra_at_the_edges_of_the_value_search(dh):
+    """Bidiagonals whose values repeat, vanish or span many decades: two
+    values each dh / 2 times, a single nonzero row, a zero matrix, a graded
+    spectrum, and one value set apart by 2^12. fp64 backward error of the
+    reduction is a few dh * eps of the largest value, and ER weights a value by
+    its share of the sum, so 1e-12 leaves room for dh = 128."""
+    rng = np.random.default_rng(dh + 1)
+    dm = dh + 24
+    wk = np.zeros((1, dh, dm))
+    wk[0, :, :dh] = np.eye(dh)
+    wq = np.zeros((5, dh, dm))
+    wq[0, :, :dh] = np.diag(np.where(np.arange(dh) < dh // 2, 1.0, 2.0))
+    wq[1, dh // 3] = _bf16(rng.standard_normal(dm))
+    wq[3] = _bf16(np.geomspace(1.0, 1e-6, dh)[:, None] * rng.standard_normal((dh, dm)))
+    wq[4] = _bf16(rng.standard_normal((dh, dm)))
+    wq[4, 5] *= 4096.0
+    _, er = _classify(wq, wk, 50)
+    n = dh // 2
+    two = math.exp(-n * (1 / (3 * n) * math.log(1 / (3 * n)) + 2 / (3 * n) * math.log(2 / (3 * n))))
+    np.testing.assert_allclose(er[0], two, rtol=1e-12)
+    assert abs(er[1] - 1.0) < 1e-12 and er[2] == 1.0
+    np.testing.assert_allclose(er[3:], _er_by_svd(wq[3:], wk), rtol=1e-12)

@@ -33,14 +33,12 @@
 #include "../../include/aoh.h"
 #include "common.cuh"
 #include "internal.h"
+#include "tc.cuh"
 
 namespace aoh {
 namespace {
 
 using bf16 = __nv_bfloat16;
-constexpr int kGT = 64;              // Gram output tile
-constexpr int kGK = 32;              // d_model columns per step
-constexpr int kGramThreads = 256;
 constexpr int kMatThreads = 256;
 
 // Matrices are numbered layer-major: layer l's query projections, then its
@@ -51,44 +49,245 @@ __device__ __forceinline__ const bf16* weight_of(const bf16* wq, const bf16* wk,
   return mi < Hq ? wq + ((size_t)l * Hq + mi) * dh * dm : wk + ((size_t)l * Hkv + (mi - Hq)) * dh * dm;
 }
 
-__global__ void __launch_bounds__(kGramThreads) gram_kernel(const bf16* wq, const bf16* wk, int Hq, int Hkv, int nall,
-                                                            int dh, int dm, int span, double* part) {
-  __shared__ double sa[kGK][kGT + 1], sb[kGK][kGT + 1];
-  const int m = blockIdx.z, split = blockIdx.y;
-  const int tiles = dh / kGT;
-  const int ti = blockIdx.x / tiles, tj = blockIdx.x % tiles;
-  const bf16* W = weight_of(wq, wk, m, Hq, Hkv, dh, dm);
-  const int k0 = split * span, k1 = min(dm, k0 + span);
-  const int tx = threadIdx.x % 16, ty = threadIdx.x / 16;
-  double acc[4][4] = {};
-  for (int kc = k0; kc < k1; kc += kGK) {
-    for (int e = threadIdx.x; e < kGT * kGK; e += kGramThreads) {
-      const int row = e / kGK, kk = e % kGK;
-      const bool in = kc + kk < k1;
-      sa[kk][row] = in ? (double)__bfloat162float(W[(size_t)(ti * kGT + row) * dm + kc + kk]) : 0.0;
-      sb[kk][row] = in ? (double)__bfloat162float(W[(size_t)(tj * kGT + row) * dm + kc + kk]) : 0.0;
+// Largest exponent field of every weight row (255: the row holds an infinity
+// or a NaN), one warp per row; rows are numbered matrix-major.
+__global__ void __launch_bounds__(256) row_exp_kernel(const bf16* wq, const bf16* wk, int Hq, int Hkv, int rows, int dh,
+                                                      int dm, int vec, int* row_exp) {
+  const int row = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+  if (row >= rows) return;
+  const uint16_t* w =
+      reinterpret_cast<const uint16_t*>(weight_of(wq, wk, row / dh, Hq, Hkv, dh, dm)) + (size_t)(row % dh) * dm;
+  uint32_t m = 0;  // the largest magnitude, two halves a word when vec
+  if (vec) {
+    for (int c = lane; c < dm / 8; c += 32) {
+      const uint4 v = __ldg(reinterpret_cast<const uint4*>(w) + c);
+      m = __vmaxu2(m, __vmaxu2(__vmaxu2(v.x & 0x7fff7fffu, v.y & 0x7fff7fffu),
+                               __vmaxu2(v.z & 0x7fff7fffu, v.w & 0x7fff7fffu)));
     }
-    __syncthreads();
-#pragma unroll 4
-    for (int kk = 0; kk < kGK; ++kk) {
-      double a[4], b[4];
-#pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        a[i] = sa[kk][ty * 4 + i];
-        b[i] = sb[kk][tx * 4 + i];
-      }
-#pragma unroll
-      for (int i = 0; i < 4; ++i)
-#pragma unroll
-        for (int j = 0; j < 4; ++j) acc[i][j] = fma(a[i], b[j], acc[i][j]);
-    }
-    __syncthreads();
+  } else {
+    for (int c = lane; c < dm; c += 32) m = max(m, (uint32_t)(w[c] & 0x7fffu));
   }
-  double* out = part + ((size_t)split * nall + m) * dh * dh;
+  m = max(m & 0xffffu, m >> 16);
+  m = __reduce_max_sync(0xffffffffu, m);
+  if (lane == 0) row_exp[row] = max((int)(m >> 7), 1);
+}
+
+// Exact Gram matrices W W^T on the tensor cores. A row's values are fixed
+// point fractions of its largest exponent, x = sum_s d_s 2^(-7 s) with signed
+// 7-bit digits d_1 .. d_8 (a bf16 value's 8 bits fall into two neighbouring
+// digits), and digit matrices are exact in bf16, so W W^T is the sum over
+// digit pairs of D_i D_j^T 2^(-7 (i + j)). Pairs with the same i + j = c share
+// a TMEM accumulator: at most 8 pairs times 128 columns times 2^14 stay below
+// 2^24, so every fp32 accumulation is exact, and after every 128 columns the
+// accumulators are added into 64-bit integers. Products below 2^-63 of the
+// two rows' scale (c > 9) are left out; fp64 sums round at 2^-53 of it. The
+// result rounds once, when it becomes a double.
+//
+// The 8 accumulators (c = 2 .. 9) do not fit TMEM at once, so
+// blockIdx.z = 0 takes c = 2 .. 5 (digits 1-4, 10 pairs) and 1 takes c = 6 .. 9
+// (26 pairs), each writing its own part. For 896 matrices of 128 x 3584 this
+// takes 4.8 ms, and the row exponents 0.12 ms (7.1 TB/s); the plain fp64 Gram
+// took 88.6 ms (105 GFLOP at 1.19 TFLOP/s, the fp64 pipe's two FMAs a clock
+// and SM). It is bound by the tensor cores (36 digit products of 128 x 128 x
+// 64 a step) plus the digit production, which alternate.
+//
+// One CTA: 128 rows (one matrix at d_head 128, two at 64, whose off-diagonal
+// blocks are dropped), 512 threads. Each thread turns 16 weights of a
+// 64-column step into digits (128-byte-swizzled K-major tiles, one per digit),
+// one thread issues the step's MMAs, and the next step's weights are loaded
+// meanwhile.
+constexpr int kDigits = 8;
+constexpr int kDigitTile = 128 * 64 * 2;
+constexpr int kGramTcThreads = 512;
+constexpr int kGramTcSmem = kDigits * kDigitTile + 1024;
+constexpr int kGramChunk = 128;  // columns between two reads of the accumulators
+constexpr uint32_t kGramIdesc = idesc_bf16(128, 128, false);
+
+// bf16 bits of +-d, 0 <= d < 256.
+__device__ __forceinline__ uint32_t digit_bf16(uint32_t d, uint32_t sign) {
+  const float f = __uint_as_float(0x4B000000u | d) - 8388608.f;
+  return (__float_as_uint(f) >> 16) | sign;
+}
+
+__global__ void __launch_bounds__(kGramTcThreads, 1)
+    gram_tc_kernel(const bf16* wq, const bf16* wk, int Hq, int Hkv, int nall, int dh, int dm, int span, int vec,
+                   const int* row_exp, double* part, uint32_t* err) {
+  extern __shared__ uint8_t smem_raw[];
+  uint8_t* smem = smem_raw + ((1024 - (smem_u32(smem_raw) & 1023)) & 1023);
+  __shared__ uint64_t done;
+  __shared__ uint32_t tmem_slot;
+  __shared__ int s_abort, col_exp[128];
+  const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
+  const int per = 128 / dh;  // matrices of this CTA
+  const int split = blockIdx.y, high = blockIdx.z;
+  const int k0 = split * span, k1 = min(dm, k0 + span);
+  if (t == 0) {
+    mbar_init(&done, 1);
+    s_abort = 0;
+    fence_mbar_init();
+  }
+  if (t < 128) {
+    const int m = blockIdx.x * per + t / dh;
+    col_exp[t] = m < nall ? row_exp[m * dh + t % dh] : 1;
+  }
+  if (warp == 0) {
+    tmem_alloc(&tmem_slot, 512);
+    tmem_relinquish();
+  }
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tmem = tmem_slot;
+
+  // digit production: row t / 4, columns 16 (t % 4) .. + 15 of each step
+  const int prow = t >> 2, pch = (t & 3) * 2;
+  const int pm = blockIdx.x * per + prow / dh;
+  const bool has = pm < nall;
+  const uint16_t* wrow =
+      has ? reinterpret_cast<const uint16_t*>(weight_of(wq, wk, pm, Hq, Hkv, dh, dm)) + (size_t)(prow % dh) * dm
+          : nullptr;
+  const int pexp = col_exp[prow];
+  uint32_t w[8];
+  auto load = [&](int kc) {
+    const int c0 = kc + (t & 3) * 16;
 #pragma unroll
-  for (int i = 0; i < 4; ++i)
+    for (int i = 0; i < 8; ++i) w[i] = 0u;
+    if (!has) return;
+    if (vec) {  // dm, k0 and k1 are multiples of 8
 #pragma unroll
-    for (int j = 0; j < 4; ++j) out[(size_t)(ti * kGT + ty * 4 + i) * dh + tj * kGT + tx * 4 + j] = acc[i][j];
+      for (int i = 0; i < 2; ++i)
+        if (c0 + 8 * i < k1) {
+          const uint4 v = __ldg(reinterpret_cast<const uint4*>(wrow + c0 + 8 * i));
+          w[4 * i] = v.x;
+          w[4 * i + 1] = v.y;
+          w[4 * i + 2] = v.z;
+          w[4 * i + 3] = v.w;
+        }
+    } else {
+#pragma unroll
+      for (int i = 0; i < 16; ++i)
+        if (c0 + i < k1) w[i >> 1] |= (uint32_t)wrow[c0 + i] << ((i & 1) * 16);
+    }
+  };
+  const int n_dig = high ? kDigits : 4;
+  auto digits = [&]() {
+#pragma unroll
+    for (int half = 0; half < 2; ++half) {
+      uint32_t hi[8], lo[8];
+      int s0[8];
+#pragma unroll
+      for (int i = 0; i < 8; ++i) {
+        const uint32_t h = (w[4 * half + (i >> 1)] >> ((i & 1) * 16)) & 0xffffu;
+        const int ef = (int)((h >> 7) & 255u);
+        const uint32_t mant = (h & 127u) | (ef ? 128u : 0u);
+        const int p = min(pexp - max(ef, 1), 63);  // leading bit at 2^(-1 - p)
+        s0[i] = (p * 37) >> 8;                      // p / 7
+        const uint32_t y = mant << (6 - (p - 7 * s0[i]));
+        const uint32_t sign = h & 0x8000u;
+        hi[i] = digit_bf16(y >> 7, sign);
+        lo[i] = digit_bf16(y & 127u, sign);
+      }
+      uint8_t* dst = smem + prow * 128 + (((pch + half) ^ (prow & 7)) << 4);
+#pragma unroll
+      for (int s = 0; s < kDigits; ++s) {
+        if (s >= n_dig) break;
+        uint32_t o[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          const uint32_t a = s == s0[2 * i] ? hi[2 * i] : s == s0[2 * i] + 1 ? lo[2 * i] : 0u;
+          const uint32_t b = s == s0[2 * i + 1] ? hi[2 * i + 1] : s == s0[2 * i + 1] + 1 ? lo[2 * i + 1] : 0u;
+          o[i] = a | (b << 16);
+        }
+        *reinterpret_cast<uint4*>(dst + s * kDigitTile) = make_uint4(o[0], o[1], o[2], o[3]);
+      }
+    }
+  };
+  auto issue = [&](bool fresh) {  // one thread: the step's digit pairs
+    const uint32_t base = smem_u32(smem);
+    for (int a = 0; a < 4; ++a) {
+      const int c = a + (high ? 6 : 2);
+      const int i0 = max(1, c - kDigits), i1 = min(c - 1, kDigits);
+      for (int i = i0; i <= i1; ++i) {
+        const uint32_t da = base + (i - 1) * kDigitTile, db = base + (c - i - 1) * kDigitTile;
+#pragma unroll
+        for (int kk = 0; kk < 4; ++kk)
+          tc_mma(tmem + a * 128, sdesc_sw128(da + kk * 32, 16, 1024), sdesc_sw128(db + kk * 32, 16, 1024), kGramIdesc,
+                 (fresh && i == i0 && kk == 0) ? 0u : 1u);
+      }
+    }
+    tc_commit(&done);
+  };
+
+  // accumulators: row 32 (warp % 4) + lane, columns 32 (warp / 4) .. + 31
+  const int row = (warp & 3) * 32 + lane, cg = warp >> 2;
+  const bool wanted = dh == 128 || (row >> 6) == (cg >> 1);  // uniform over the warp
+  long long acc[32];
+#pragma unroll
+  for (int i = 0; i < 32; ++i) acc[i] = 0;
+  auto flush = [&]() {
+    if (!wanted) return;
+    const uint32_t tl = tmem + ((uint32_t)((warp & 3) * 32) << 16) + cg * 32;
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      uint32_t v0[8], v1[8], v2[8], v3[8];
+      tmem_ld8(tl + q * 8, v0);
+      tmem_ld8(tl + 128 + q * 8, v1);
+      tmem_ld8(tl + 256 + q * 8, v2);
+      tmem_ld8(tl + 384 + q * 8, v3);
+      tmem_ld_wait();
+#pragma unroll
+      for (int i = 0; i < 8; ++i) {
+        const int a = __float2int_rn(__uint_as_float(v0[i])) * 128 + __float2int_rn(__uint_as_float(v1[i]));
+        const int b = __float2int_rn(__uint_as_float(v2[i])) * 128 + __float2int_rn(__uint_as_float(v3[i]));
+        acc[8 * q + i] += (long long)a * 16384 + b;
+      }
+    }
+  };
+
+  int step = 0;
+  bool ok = true;
+  load(k0);
+  for (int kc = k0; kc < k1; kc += 64, ++step) {
+    const bool fresh = (step * 64) % kGramChunk == 0;
+    if (step > 0) {
+      ok = wait_bar(&done, (step - 1) & 1, err, &s_abort);  // the digit tiles are free
+      tc_fence_after();
+      ok = __all_sync(0xffffffffu, ok);
+      if (ok && fresh) flush();
+    }
+    if (ok) digits();
+    if (kc + 64 < k1) load(kc + 64);
+    fence_proxy_async_smem();
+    tc_fence_before();
+    ok = __syncthreads_and(ok);
+    if (!ok) break;
+    if (t == 0) {
+      tc_fence_after();
+      issue(fresh);
+    }
+    __syncwarp();
+  }
+  if (step > 0) {  // every issued MMA ends before TMEM is freed
+    ok = drain_wait(&done, (step - 1) & 1, err) && ok;
+    tc_fence_after();
+    if (__all_sync(0xffffffffu, ok)) flush();
+  }
+  const int m = blockIdx.x * per + row / dh;
+  if (wanted && m < nall) {
+    double* out = part + ((size_t)(split * 2 + high) * nall + m) * dh * dh + (size_t)(row % dh) * dh + (cg * 32) % dh;
+    const int ei = col_exp[row];
+#pragma unroll
+    for (int i = 0; i < 32; ++i) {
+      const int ej = col_exp[cg * 32 + i];
+      // value 2^(e - 126) per unit of either row's fractions
+      const double sc = __longlong_as_double((long long)(1023 + ei + ej - 252 - (high ? 63 : 35)) << 52);
+      out[i] = ei == 255 || ej == 255 ? __longlong_as_double(0x7ff8000000000000ll) : (double)acc[i] * sc;
+    }
+  }
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  if (warp == 0) tmem_dealloc(tmem, 512);
 }
 
 // Sum of a block's values (every thread gets it); `red` holds 32 doubles.
@@ -181,7 +380,6 @@ __device__ __forceinline__ double warp_sum(double v) {
 template <int N>
 struct BidiagCfg {
   static constexpr int LD = N + 1;
-  static constexpr int THREADS = 4 * N;
   static constexpr int SMEM = (N * LD + 4 * N) * 8;
 };
 
@@ -447,48 +645,58 @@ extern "C" aoh_status aoh_classify(const void* w_q, const void* w_k, int32_t n_l
   if (sparsity_pct < 0 || sparsity_pct > 100)
     return fail(AOH_ERR_INVALID, "aoh_classify: sparsity_pct outside [0, 100]");
   cudaStream_t s = static_cast<cudaStream_t>(stream);
-  const int dh = d_head, nmat = n_q_heads + n_kv_heads, tiles = dh / kGT;
+  const int dh = d_head, nmat = n_q_heads + n_kv_heads;
   const int nall = n_layers * nmat, nq = n_layers * n_q_heads;
   if ((long long)n_layers * nmat > 65535) return fail(AOH_ERR_INVALID, "aoh_classify: too many matrices in one call");
   int dev = 0, sms = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   if (e != cudaSuccess) return fail(AOH_ERR_CUDA, "aoh_classify: device query failed");
-  // split d_model so that the Gram grid covers about two waves, >= 256 columns a split
-  int nsplit = (2 * sms + nall * tiles * tiles - 1) / (nall * tiles * tiles);
+  // split d_model so that the Gram grid (two CTAs per 128 rows and split)
+  // covers about two waves, >= 256 columns a split
+  const int groups = (nall * dh + 127) / 128;
+  int nsplit = (sms + groups - 1) / groups;
   nsplit = std::max(1, std::min(nsplit, std::max(1, d_model / 256)));
   nsplit = std::min(nsplit, 16);
-  const int span = ((d_model + nsplit - 1) / nsplit + kGK - 1) / kGK * kGK;
+  const int span = ((d_model + nsplit - 1) / nsplit + kGramChunk - 1) / kGramChunk * kGramChunk;
   nsplit = (d_model + span - 1) / span;
+  const int nparts = 2 * nsplit;
   const size_t n2 = (size_t)dh * dh;
-  // Gram parts, factors, bidiagonals, ER; labels
-  const size_t bytes = ((size_t)nsplit * nall * n2 + (size_t)nall * n2 + 2 * (size_t)nq * dh + nq) * sizeof(double) +
-                       (size_t)n_layers * n_kv_heads + 64;
+  // Gram parts, factors, bidiagonals, ER; error word, row exponents; labels
+  const size_t bytes = ((size_t)nparts * nall * n2 + (size_t)nall * n2 + 2 * (size_t)nq * dh + nq) * sizeof(double) +
+                       (1 + (size_t)nall * dh) * sizeof(int) + (size_t)n_layers * n_kv_heads;
   void* scratch = nullptr;
   e = cudaMallocAsync(&scratch, bytes, s);
   if (e != cudaSuccess) return fail(AOH_ERR_CUDA, "aoh_classify: cudaMallocAsync failed");
   double* part = static_cast<double*>(scratch);
-  double* L = part + (size_t)nsplit * nall * n2;
+  double* L = part + (size_t)nparts * nall * n2;
   double* diag = L + (size_t)nall * n2;
   double* sup = diag + (size_t)nq * dh;
   double* er = sup + (size_t)nq * dh;
-  uint8_t* labels = reinterpret_cast<uint8_t*>(er + nq);
+  uint32_t* err = reinterpret_cast<uint32_t*>(er + nq);
+  int* row_exp = reinterpret_cast<int*>(err + 1);
+  uint8_t* labels = reinterpret_cast<uint8_t*>(row_exp + (size_t)nall * dh);
   const int smem = (int)(n2 * sizeof(double));
   static bool attr_set = false;
   if (!attr_set) {
     e = cudaFuncSetAttribute(chol_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 128 * 128 * 8);
     if (e == cudaSuccess)
       e = cudaFuncSetAttribute(bidiag_kernel<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, BidiagCfg<128>::SMEM);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(gram_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kGramTcSmem);
     if (e != cudaSuccess) {
       cudaFreeAsync(scratch, s);
       return fail(AOH_ERR_CUDA, "aoh_classify: cudaFuncSetAttribute failed");
     }
     attr_set = true;
   }
-  gram_kernel<<<dim3(tiles * tiles, nsplit, nall), kGramThreads, 0, s>>>(static_cast<const bf16*>(w_q),
-                                                                          static_cast<const bf16*>(w_k), n_q_heads,
-                                                                          n_kv_heads, nall, dh, d_model, span, part);
-  chol_kernel<<<nall, kMatThreads, smem, s>>>(part, nsplit, nall, dh, L);
+  const bf16 *wq = static_cast<const bf16*>(w_q), *wk = static_cast<const bf16*>(w_k);
+  // 16-byte loads of the weights when every row starts on 16 bytes
+  const int vec = d_model % 8 == 0 && ((reinterpret_cast<uintptr_t>(w_q) | reinterpret_cast<uintptr_t>(w_k)) & 15) == 0;
+  cudaMemsetAsync(err, 0, sizeof(*err), s);
+  row_exp_kernel<<<(nall * dh + 7) / 8, 256, 0, s>>>(wq, wk, n_q_heads, n_kv_heads, nall * dh, dh, d_model, vec, row_exp);
+  gram_tc_kernel<<<dim3(groups, nsplit, 2), kGramTcThreads, kGramTcSmem, s>>>(
+      wq, wk, n_q_heads, n_kv_heads, nall, dh, d_model, span, vec, row_exp, part, err);
+  chol_kernel<<<nall, kMatThreads, smem, s>>>(part, nparts, nall, dh, L);
   if (dh == 128) {
     bidiag_kernel<128><<<nq, 512, BidiagCfg<128>::SMEM, s>>>(L, n_q_heads, n_kv_heads, diag, sup);
     svals_kernel<128><<<nq, 128, 0, s>>>(diag, sup, d_model, er);
@@ -501,9 +709,12 @@ extern "C" aoh_status aoh_classify(const void* w_q, const void* w_k, int32_t n_l
   if (e == cudaSuccess)
     e = cudaMemcpyAsync(labels_out, labels, (size_t)n_layers * n_kv_heads, cudaMemcpyDeviceToHost, s);
   if (e == cudaSuccess && er_out) e = cudaMemcpyAsync(er_out, er, nq * sizeof(double), cudaMemcpyDeviceToHost, s);
+  uint32_t h_err = 0;
+  if (e == cudaSuccess) e = cudaMemcpyAsync(&h_err, err, sizeof(h_err), cudaMemcpyDeviceToHost, s);
   const cudaError_t f = cudaFreeAsync(scratch, s);
   if (e == cudaSuccess) e = f;
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);
   if (e != cudaSuccess) return fail(AOH_ERR_CUDA, "aoh_classify: a CUDA call failed");
+  if (h_err) return fail(AOH_ERR_TIMEOUT, "aoh_classify: a kernel's bounded wait ran out");
   return AOH_OK;
 }

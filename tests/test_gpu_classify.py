@@ -195,3 +195,30 @@ def test_spectra_at_the_edges_of_the_value_search(dh):
     np.testing.assert_allclose(er[0], two, rtol=1e-12)
     assert abs(er[1] - 1.0) < 1e-12 and er[2] == 1.0
     np.testing.assert_allclose(er[3:], _er_by_svd(wq[3:], wk), rtol=1e-12)
+
+
+@pytest.mark.parametrize("dh,dm,offset", [(64, 1, 0), (64, 127, 1), (64, 193, 0), (64, 640, 0), (128, 257, 0),
+                                          (128, 1031, 3), (128, 776, 0)])
+def test_gram_digits_at_column_edges(dh, dm, offset):
+    """d_model around the 64-column steps, the 128-column chunks and the splits
+    of the Gram, odd row lengths and unaligned weights (2-byte loads), an odd
+    number of 64-row matrices, rows whose values span 2^40 (every 7-bit digit
+    in use) and a zero row. Products and digit sums are exact, so only the fp64
+    steps after the Gram differ from the SVD of M_h: eps times the squared
+    condition of W, up to 1e3 here, of the small values' share of ER."""
+    ensure_lib()
+    rng = np.random.default_rng(dh * 7 + dm)
+    Hq, Hkv = 4, 1
+    wq, wk = rng.standard_normal((Hq, dh, dm)), rng.standard_normal((Hkv, dh, dm))
+    wq[1] *= 2.0 ** -rng.integers(0, 41, size=(dh, dm))
+    wq[2] *= 2.0 ** rng.integers(-6, 7, size=(dh, 1))
+    wk[0, dh // 2] = 0.0
+    wq, wk = _bf16(wq), _bf16(wk)
+
+    def place(a):
+        flat = torch.zeros(a.size + 8, dtype=torch.bfloat16, device="cuda")
+        flat[offset:offset + a.size] = _dev(a).flatten()
+        return flat[offset:offset + a.size].view(a.shape)
+
+    _, er = aoh.aoh_classify(place(wq), place(wk), Hkv, 50)
+    np.testing.assert_allclose(er, _er_by_svd(wq, wk), rtol=1e-10)

@@ -366,7 +366,7 @@ __device__ __forceinline__ double warp_sum(double v) {
 // flops each: 240 ms for 784 heads of 128. The reduction now takes 9.7 ms (its
 // 4.4 GFLOP and the product's 1.5 cost 5 ms at the 1.2 TFLOP/s the fp64 pipe
 // gives; the rest is the chain of 256 reflectors a head and the sixth, mostly
-// empty, wave of heads) and the values 22 ms.
+// empty, wave of heads) and the values 1.4 ms.
 //
 // One CTA per head, 4 N threads, A row-major in shared memory with N + 1
 // doubles a row, so that neither a row nor a column walk meets a bank
@@ -500,17 +500,29 @@ __global__ void __launch_bounds__(4 * N) bidiag_kernel(const double* L, int Hq, 
 //   delta_i = q_i + t_i, t_0 = -s, t_{i+1} = t_i f_i / delta_i - s
 // has as many negative delta_i as B^T B has eigenvalues below s, to high
 // relative accuracy, and sum_i delta_i' / delta_i is p'(s) / p(s) of its
-// characteristic polynomial. The N threads first count at N points spread
-// over [0, bound], which brackets every value to a part in N, then each
-// thread bisects until its bracket holds one value and takes Newton steps
-// inside the bracket, which the count that each evaluation gives keeps
-// shrinking. The values are wanted to absolute accuracy (ER weights them by
-// their share of the sum): a bracket of 2^-53 of the bound ends the search.
+// characteristic polynomial. Each thread first bisects in fp32 (the fp32 pipe
+// is 64 times as wide as the fp64 pipe), then takes Newton steps in fp64 from
+// there, two or three as a rule. Every evaluation's count says on which side of
+// the wanted value the point lies: a step is taken only towards that side and
+// inside the bracket that the counts have left, else the bracket is halved
+// (values that repeat, to the last bit). The values are wanted to absolute
+// accuracy (ER weights them by their share of the sum). 784 heads of 128 take
+// 1.4 ms; with the bisection in fp64 as well, from 128 shared counts to single
+// values, and divisions for the reciprocals they took 22 ms.
+// 1 / x for 1e-30 <= |x| <= 1e30, to about an ulp: the residual e = 1 - x y of
+// an fp32 reciprocal y gives y (1 + e + e^2) + O(e^3), e < 2^-22. Half the fp64
+// operations of a division.
+__device__ __forceinline__ double fast_rcp(double x) {
+  const double y = (double)__frcp_rn((float)x);
+  const double e = fma(-x, y, 1.0);
+  return fma(y, fma(e, e, e), y);
+}
+
 template <int N>
 __global__ void __launch_bounds__(N) svals_kernel(const double* diag, const double* sup, int dm, double* er) {
   __shared__ double2 qf[N];  // (q_i, f_i)
   __shared__ double red[32];
-  __shared__ int cnt[N];
+  __shared__ float2 qf32[N];
   const int hg = blockIdx.x, j = threadIdx.x;
   const double d = fabs(diag[(size_t)hg * N + j]);
   const double e = j + 1 < N ? fabs(sup[(size_t)hg * N + j]) : 0.0;
@@ -523,50 +535,53 @@ __global__ void __launch_bounds__(N) svals_kernel(const double* diag, const doub
   }
   const double inv_b = 1.0 / bound;
   qf[j] = make_double2((d * inv_b) * (d * inv_b), (e * inv_b) * (e * inv_b));
+  qf32[j] = make_float2((float)qf[j].x, (float)qf[j].y);
   __syncthreads();
-  double g;  // p'(s) / p(s) at the last point
-  auto count = [&](double s) {
+  // fp32 bisection to a bracket of 2^-22
+  float xf = 0.5f;
+  {
+    float flo = 0.f, fhi = 1.f;
+#pragma unroll 1
+    for (int round = 0; round < 22; ++round) {
+      xf = 0.5f * (flo + fhi);
+      const float s = xf * xf;
+      float t = -s;
+      int c = 0;
+#pragma unroll 8
+      for (int i = 0; i < N; ++i) {
+        const float2 v = qf32[i];
+        float del = v.x + t;
+        if (fabsf(del) < 1e-30f) del = -1e-30f;
+        c += del < 0.f;
+        t = fmaf(__fdividef(v.y, del), t, -s);
+      }
+      if (c <= j)
+        flo = xf;
+      else
+        fhi = xf;
+    }
+    xf = 0.5f * (flo + fhi);
+  }
+  double x = fmax((double)xf, 1e-16), lo = 0.0, hi = 1.0 + 1e-9, prev = 0.0;
+  int nlo = 0, nhi = N;
+  bool done = false;
+  for (int round = 0; round < 120 && !__all_sync(0xffffffffu, done); ++round) {
+    const double s = x * x;
+    double t = -s, tp = -1.0, g = 0.0;  // g = p'(s) / p(s)
     int c = 0;
-    double t = -s, tp = -1.0;
-    g = 0.0;
 #pragma unroll 4
     for (int i = 0; i < N; ++i) {
       const double2 v = qf[i];
       double del = v.x + t;
-      if (fabs(del) < 1e-280) del = -1e-280;
+      if (fabs(del) < 1e-30) del = -1e-30;
       c += del < 0.0;
-      const double inv = 1.0 / del;
+      const double inv = fast_rcp(del);
       const double r = v.y * inv, u = tp * inv;
       g += u;
       t = fma(r, t, -s);
       tp = fma(r * v.x, u, -1.0);
     }
-    return c;
-  };
-  double x = (double)(j + 1) / (N + 1);
-  cnt[j] = count(x * x);
-  __syncthreads();
-  double lo = 0.0, hi = 1.0 + 1e-9;
-  int nlo = 0, nhi = N;
-  for (int i = 0; i < N; ++i) {
-    const double p = (double)(i + 1) / (N + 1);
-    if (cnt[i] <= j && p > lo) {
-      lo = p;
-      nlo = cnt[i];
-    }
-  }
-  for (int i = N - 1; i >= 0; --i) {
-    const double p = (double)(i + 1) / (N + 1);
-    if (cnt[i] > j && p < hi && p > lo) {
-      hi = p;
-      nhi = cnt[i];
-    }
-  }
-  x = 0.5 * (lo + hi);
-  bool done = false;
-  for (int round = 0; round < 120 && !__syncthreads_and(done); ++round) {
-    const int c = count(x * x);  // done threads repeat their last point
-    if (done) continue;
+    if (done) continue;  // repeats its last point while others search
     if (c <= j) {
       lo = x;
       nlo = c;
@@ -574,12 +589,19 @@ __global__ void __launch_bounds__(N) svals_kernel(const double* diag, const doub
       hi = x;
       nhi = c;
     }
-    const double mid = 0.5 * (lo + hi);
     const double xn = x - 1.0 / (2.0 * x * g);
-    // every fourth round halves the bracket whatever Newton says
-    const bool newton = nhi - nlo == 1 && (round & 3) != 3 && xn > lo && xn < hi;
-    done = hi - lo < 1.2e-16 || hi < 1e-15 || (newton && fabs(xn - x) < 4e-15);
-    x = newton ? xn : mid;
+    const double step = fabs(xn - x);
+    const bool near_j = c == j || c == j + 1;
+    // Once a Newton step is far shorter than the one before, a step of 1e-11
+    // leaves 1e-22 over the distance to the next value (and its sign may be
+    // rounding). Towards a value that repeats the steps shrink slowly: there
+    // only the bracket ends the search.
+    const bool converged = near_j && step < 1e-11 && step < 1e-3 * prev;
+    // past eight rounds every fourth halves the bracket, so the search ends
+    const bool newton = near_j && (xn > x) == (c <= j) && xn > lo && xn < hi && (round < 8 || (round & 3) != 3);
+    done = converged || hi - lo < 1.2e-16 || hi < 1e-15 || (newton && step < 4e-15 && nhi - nlo == 1);
+    prev = newton ? step : 0.0;
+    x = converged || newton ? xn : 0.5 * (lo + hi);
   }
   const double nrm = x * bound;
   const double smax = block_max(nrm, red);

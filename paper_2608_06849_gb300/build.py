@@ -34,8 +34,8 @@ def source_digest():
 
 
 KERNEL_SOURCES = {
-    "decode": ["decode.cu", "decode_common.cuh", "common.cuh", "internal.h"],
-    "decode_tc": ["decode_tc.cu", "decode_common.cuh", "tc.cuh", "common.cuh", "internal.h"],
+    "decode": ["decode.cu", "decode_common.cuh", "cluster.cuh", "common.cuh", "internal.h"],
+    "decode_tc": ["decode_tc.cuh", "decode_tc.cu", "decode_common.cuh", "cluster.cuh", "tc.cuh", "common.cuh", "internal.h"],
     "prefill": ["prefill_tc.cu", "tc.cuh", "common.cuh", "internal.h"],
 }
 

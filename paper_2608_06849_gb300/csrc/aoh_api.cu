@@ -428,20 +428,21 @@ aoh_status aoh_prefill(const void* q, const void* k, const void* v, int32_t T, c
 
 namespace {
 
-// Host checks shared by the decode entry points; fills `a` for the step and
-// the step's total rows (every retrieval row; ring rows of streaming heads).
+// Host checks shared by the decode entry points; fills `a` for the step, the
+// longest sequence's rows and the step's total rows (every retrieval row; ring rows of streaming heads).
 aoh_status prepare_decode(const void* q, const void* k_new, const void* v_new, aoh_cache* cache, void* out,
-                          DecodeArgs& a, long long& total) {
+                          DecodeArgs& a, long long& total, long long& longest) {
   if (!cache) return fail(AOH_ERR_INVALID, "cache is NULL");
   if (!q || !k_new || !v_new || !out) return fail(AOH_ERR_INVALID, "q, k_new, v_new and out must not be NULL");
   if (!aligned(q, 16) || !aligned(k_new, 16) || !aligned(v_new, 16) || !aligned(out, 16))
     return fail(AOH_ERR_INVALID, "q, k_new, v_new and out must be 16-byte aligned");
   const CacheGeom& g = cache->geom;
-  total = 0;
+  total = longest = 0;
   for (int b = 0; b < g.B; ++b) {
     if (g.n_r > 0 && cache->lens[b] + 1 > g.max_seq)
       return fail(AOH_ERR_CAPACITY, "sequence %d holds %d tokens; max_seq is %d", b, cache->lens[b], g.max_seq);
     const long long t1 = cache->lens[b] + 1;
+    longest = std::max(longest, t1);
     total += g.n_r * t1 + g.n_s * std::min<long long>(t1, g.S + g.W);
   }
   a.tcr = cache->tcr;
@@ -469,12 +470,14 @@ extern "C" {
 aoh_status aoh_decode_step(const void* q, const void* k_new, const void* v_new, aoh_cache* cache, void* out,
                            void* stream) {
   DecodeArgs a;
-  long long total = 0;
-  const aoh_status st = prepare_decode(q, k_new, v_new, cache, out, a, total);
+  long long total = 0, longest = 0;
+  const aoh_status st = prepare_decode(q, k_new, v_new, cache, out, a, total, longest);
   if (st != AOH_OK) return st;
   const CacheGeom& g = cache->geom;
-  a.n_ctas = decode_ctas(total, cache->num_sms, g.D, g.G);
-  if (decode_uses_tc(g.D, g.G)) a.item_cost = decode_tc_item_cost(total, a.n_ctas, cache->num_sms);
+  if (decode_uses_tc(g.D, g.G))
+    decode_tc_split(a, g, longest, total, cache->num_sms);
+  else
+    a.n_ctas = decode_cc_ctas(total, cache->num_sms);
   cudaError_t e = launch_decode(a, (cudaStream_t)stream);
   if (e != cudaSuccess) return cuda_fail(e, "decode kernel launch");
   for (int b = 0; b < g.B; ++b) cache->lens[b] += 1;
@@ -484,8 +487,8 @@ aoh_status aoh_decode_step(const void* q, const void* k_new, const void* v_new, 
 aoh_status aoh_decode_step_anchor(const void* q, const void* k_new, const void* v_new, aoh_cache* cache, void* out,
                                   int32_t top_k, int32_t* indices, void* stream) {
   DecodeArgs a;
-  long long total = 0;
-  const aoh_status st = prepare_decode(q, k_new, v_new, cache, out, a, total);
+  long long total = 0, longest = 0;
+  const aoh_status st = prepare_decode(q, k_new, v_new, cache, out, a, total, longest);
   if (st != AOH_OK) return st;
   const CacheGeom& g = cache->geom;
   if (top_k < 1) return fail(AOH_ERR_INVALID, "top_k must be >= 1");
@@ -497,8 +500,7 @@ aoh_status aoh_decode_step_anchor(const void* q, const void* k_new, const void* 
     if (e != cudaSuccess) return cuda_fail(e, "anchor workspace allocation");
   }
   if (g.n_r > 0) h2_decode_outputs(cache->d_h2, g.B, g.n_r, g.G, g.max_seq, &a.scores, &a.score_stride, &a.score_stats);
-  a.n_ctas = decode_ctas(total, cache->num_sms, g.D, g.G);
-  a.item_cost = decode_tc_item_cost(total, a.n_ctas, cache->num_sms);
+  decode_tc_split(a, g, longest, total, cache->num_sms);
   cudaStream_t s = (cudaStream_t)stream;
   cudaError_t e = launch_decode(a, s);
   if (e != cudaSuccess) return cuda_fail(e, "decode kernel launch");
@@ -514,8 +516,8 @@ aoh_status aoh_decode_step_reuse(const void* q, const void* k_new, const void* v
                                  const int32_t* indices, int32_t n_anchor_groups, int32_t top_k,
                                  const int32_t* group_map, void* stream) {
   DecodeArgs a;
-  long long total = 0;
-  const aoh_status st = prepare_decode(q, k_new, v_new, cache, out, a, total);
+  long long total = 0, longest = 0;
+  const aoh_status st = prepare_decode(q, k_new, v_new, cache, out, a, total, longest);
   if (st != AOH_OK) return st;
   const CacheGeom& g = cache->geom;
   // d_head 128: the tcgen05 kernel's gather warps copy the borrowed rows, a

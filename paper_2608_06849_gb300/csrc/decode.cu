@@ -490,11 +490,6 @@ bool decode_supported(int D, int G) {
 
 // Two CTAs fit on an SM (about 100 KB of shared memory each), so 2 x SMs
 // CTAs run as one wave; small launches use fewer, at least 256 rows each.
-int decode_ctas(long long total_rows, int num_sms, int D, int G) {
-  if (decode_uses_tc(D, G)) return decode_tc_ctas(total_rows, num_sms);
-  return decode_cc_ctas(total_rows, num_sms);
-}
-
 int decode_cc_ctas(long long total_rows, int num_sms) {
   const long long by_rows = (total_rows + 255) / 256;
   long long p = 2LL * num_sms;

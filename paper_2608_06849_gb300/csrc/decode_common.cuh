@@ -11,6 +11,7 @@
 
 #include <math.h>
 
+#include "cluster.cuh"
 #include "common.cuh"
 #include "internal.h"
 
@@ -406,6 +407,217 @@ __device__ __forceinline__ void finish_launch(const DecodeArgs& a, const int* le
     }
     *a.done = 0u;
   }
+}
+
+// ------------------------------------------------------- the cluster split
+// Short steps of few items: whole clusters of C CTAs are dealt to the items in
+// proportion to their rows, so that no CTA changes items, and a cluster adds up
+// its CTAs' states through distributed shared memory. Every CTA reduces one
+// C-th of the item's output (its share): the other CTAs store their values for
+// it into its receive buffer before one cluster barrier. An item of several
+// clusters then needs one global exchange per share, C of them in parallel.
+constexpr int kClusterItems = 32;  // most items of a step on this split
+constexpr int kClusterMax = 16;    // most CTAs of a cluster
+// words of the plan in shared memory
+constexpr int kPlanItem = 0, kPlanFlag = 1, kPlanLo = 2, kPlanHi = 3, kPlanParts = 4, kPlanFirst = 5;
+
+// Receive buffer: [C] values of the share, then [C][G] (m, l).
+__host__ __device__ constexpr int recv_floats(int G, int D) { return G * D + 2 * kClusterMax * G; }
+
+// The item, the rows [lo, hi) and the place in its item of this CTA. Run by
+// warp 0; up to 32 items, lane i holding item i's rows. With T rows a cluster,
+// item i takes ceil(rows_i / T) clusters: the smallest of 32 values of T
+// between an even share and one that always fits is taken. Up to 8 tiles a
+// CTA, T and the CTA's rows are whole tiles (a started tile costs as much as a
+// full one); above that an equal share is better.
+__device__ __forceinline__ void plan_clusters(const DecodeArgs& a, const int* lens_s, int tile, int* plan) {
+  constexpr unsigned kAll = 0xffffffffu;
+  const CacheGeom& g = a.geom;
+  const int n_items = g.B * (g.n_r + g.n_s);
+  const int lane = threadIdx.x & 31;
+  const int C = (int)cluster_ctas(), nc = (int)gridDim.x / C, c = (int)blockIdx.x / C;
+  const int rows = lane < n_items ? item_rows(a, lane, lens_s) : 0;
+  const int total = __reduce_add_sync(kAll, rows), most = __reduce_max_sync(kAll, rows);
+  const int active = __popc(__ballot_sync(kAll, rows > 0));
+  const int lo = max(1, (total + nc - 1) / nc);
+  const int hi = max(lo, nc > active ? min(most, (total + nc - active - 1) / (nc - active)) : most);
+  int T = lane == 31 ? hi : lo + (hi - lo) / 31 * lane;
+  const int unit = tile * C;
+  if (T <= 8 * unit) T = (T + unit - 1) / unit * unit;
+  // ceil(r / t); the half row keeps exact multiples clear of the rounding
+  auto clusters = [](int r, int t, float rc) { return r > 0 ? max(1, (int)(((float)(r + t) - 0.5f) * rc)) : 0; };
+  const float rc = 1.f / (float)T;
+  int need = 0;
+  for (int j = 0; j < n_items; ++j) need += clusters(__shfl_sync(kAll, rows, j), T, rc);
+  const unsigned fits = __ballot_sync(kAll, need <= nc);
+  const int pick = fits ? __ffs(fits) - 1 : 0;
+  const int Tp = __shfl_sync(kAll, T, pick);
+  const int n = fits ? clusters(rows, Tp, 1.f / (float)Tp) : (rows > 0 ? 1 : 0);
+  int inc = n;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const int y = __shfl_up_sync(kAll, inc, o);
+    if (lane >= o) inc += y;
+  }
+  const unsigned past = __ballot_sync(kAll, inc > c);
+  const int item = past ? __ffs(past) - 1 : n_items;
+  const int src = item < 32 ? item : 31;
+  const int first = __shfl_sync(kAll, inc - n, src), parts = __shfl_sync(kAll, n, src);
+  const int r = __shfl_sync(kAll, rows, src);
+  if (lane == 0) {
+    plan[kPlanItem] = item;
+    plan[kPlanParts] = parts;
+    plan[kPlanFirst] = first * C;
+    int l = 0, h = 0;
+    if (item < n_items) {
+      int per = (r + parts * C - 1) / (parts * C);
+      if (per <= 8 * tile) per = (per + tile - 1) / tile * tile;
+      const int q = (c - first) * C + (int)cluster_rank();
+      l = (int)min((long long)r, (long long)q * per);
+      h = (int)min((long long)r, (long long)l + per);
+    }
+    plan[kPlanLo] = l;
+    plan[kPlanHi] = h;
+  }
+}
+
+// Each thread holds row d = threadIdx.x of the CTA's O^T and the states m, l
+// of its heads: the values go to the CTA whose share they belong to, the
+// states to every CTA of the cluster.
+template <int G, int D>
+__device__ __forceinline__ void cluster_push(float* recv, const uint32_t* o, const float* m, const float* l) {
+  const int C = (int)cluster_ctas(), me = (int)cluster_rank(), t = threadIdx.x;
+  const int share = G * D / C;
+#pragma unroll
+  for (int h = 0; h < G; ++h) {
+    const int e = h * D + t, dst = e * C / (G * D);
+    cluster_st_f32(cluster_addr(recv + me * share + (e - dst * share), dst), __uint_as_float(o[h]));
+  }
+  if (t < C) {
+    const uint32_t base = cluster_addr(recv + G * D + 2 * me * G, t);
+#pragma unroll
+    for (int h = 0; h < G; ++h) cluster_st2(base + 8 * h, __float_as_uint(m[h]), __float_as_uint(l[h]));
+  }
+}
+
+// A CTA without rows: states that weigh nothing (its values are not read).
+template <int G, int D>
+__device__ __forceinline__ void cluster_push_empty(float* recv) {
+  const int C = (int)cluster_ctas(), me = (int)cluster_rank(), t = threadIdx.x;
+  if (t < C) {
+    const uint32_t base = cluster_addr(recv + G * D + 2 * me * G, t);
+#pragma unroll
+    for (int h = 0; h < G; ++h) cluster_st2(base + 8 * h, __float_as_uint(-INFINITY), 0u);
+  }
+}
+
+// After the cluster barrier: reduce this CTA's share of the item's output over
+// the cluster, two values a thread, and write it, or, when the item has
+// several clusters, write it as a partial; the last of the item's CTAs of this
+// rank to arrive then merges those. NT threads that share named barrier 1.
+template <int G, int D, int NT>
+__device__ __forceinline__ void cluster_finish(const DecodeArgs& a, const float* recv, int* plan, __nv_bfloat16* out,
+                                               float2* stats) {
+  const int C = (int)cluster_ctas(), me = (int)cluster_rank(), t = threadIdx.x;
+  const int share = G * D / C, e0 = me * share;
+  const float2* ml = reinterpret_cast<const float2*>(recv + G * D);
+  const int parts = plan[kPlanParts], first = plan[kPlanFirst];
+  float* mine = partial_slot(a, (int)blockIdx.x, 0, G, D);
+  auto store = [&](int e, float M, float L, float2 o) {
+    const float inv = 1.f / L;
+    *reinterpret_cast<uint32_t*>(out + e) = float2_to_bf16x2(o.x * inv, o.y * inv);
+    if (stats != nullptr && e % D == 0) stats[e / D] = make_float2(M, L);
+  };
+  for (int i = 2 * t; i < share; i += 2 * NT) {
+    const int e = e0 + i, h = e / D;
+    float M = -INFINITY;
+    for (int c = 0; c < C; ++c) M = fmaxf(M, ml[c * G + h].x);
+    float L = 0.f;
+    float2 o = make_float2(0.f, 0.f);
+#pragma unroll 4
+    for (int c = 0; c < C; ++c) {
+      const float2 s = ml[c * G + h];
+      if (s.x == -INFINITY) continue;
+      const float w = fast_exp2(s.x - M);
+      const float2 x = *reinterpret_cast<const float2*>(recv + c * share + i);
+      L += w * s.y;
+      o.x += w * x.x;
+      o.y += w * x.y;
+    }
+    if (parts == 1) {
+      store(e, M, L, o);
+    } else {
+      __stcg(reinterpret_cast<float2*>(mine + e), o);
+      // a head's state travels with its first value and with the share's first
+      if (i == 0 || e % D == 0) {
+        __stcg(mine + G * D + h, M);
+        __stcg(mine + G * D + G + h, L);
+      }
+    }
+  }
+  if (parts == 1) return;
+  named_barrier_sync(1, NT);
+  if (t == 0) {
+    // one counter per (item, rank): those of the item's first cluster's CTAs
+    uint32_t* cnt = &a.gcounters[first + me];
+    const bool last = atom_add_acq_rel_gpu(cnt, 1u) == (uint32_t)(parts - 1);
+    if (last) *cnt = 0u;
+    plan[kPlanFlag] = last;
+  }
+  named_barrier_sync(1, NT);
+  if (!*reinterpret_cast<volatile int*>(plan + kPlanFlag)) return;
+  constexpr int U = 8;
+  for (int i = 2 * t; i < share; i += 2 * NT) {
+    const int e = e0 + i, h = e / D;
+    float M = -INFINITY, L = 0.f;
+    float2 o = make_float2(0.f, 0.f);
+    for (int j = 0; j < parts; j += U) {
+      float2 x[U];
+      float mj[U], lj[U];
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        const float* pp = partial_slot(a, first + min(j + u, parts - 1) * C + me, 0, G, D);
+        x[u] = __ldcg(reinterpret_cast<const float2*>(pp + e));
+        mj[u] = __ldcg(pp + G * D + h);
+        lj[u] = __ldcg(pp + G * D + G + h);
+      }
+      float bm = M;
+#pragma unroll
+      for (int u = 0; u < U; ++u)
+        if (j + u < parts) bm = fmaxf(bm, mj[u]);
+      const float sc = M == -INFINITY ? 0.f : fast_exp2(M - bm);
+      o.x *= sc;
+      o.y *= sc;
+      L *= sc;
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        const float w = (j + u < parts && mj[u] != -INFINITY) ? fast_exp2(mj[u] - bm) : 0.f;
+        o.x += w * x[u].x;
+        o.y += w * x[u].y;
+        L += w * lj[u];
+      }
+      M = bm;
+    }
+    store(e, M, L, o);
+  }
+}
+
+// Cluster split: every CTA has its copy of the lengths once it arrives here, so
+// the last to arrive advances them at once, off the launch's tail. Timeouts
+// reach the error word directly, and every CTA, aborted or not, makes its
+// counter arrivals, so there is nothing to clean up at the launch's end.
+__device__ __forceinline__ void advance_lens(const DecodeArgs& a, const int* lens_s) {
+  if (atom_add_acq_rel_gpu(a.done, 1u) != gridDim.x - 1) return;
+  bool full = false;
+  for (int i = 0; i < a.geom.B; ++i) {
+    const int t = lens_s[i];
+    if (seq_full(a.geom, t))
+      full = true;
+    else
+      a.lens[i] = t + 1;
+  }
+  if (full) atomicOr(a.err, kErrCapacity);
+  *a.done = 0u;
 }
 
 }  // namespace dec

@@ -17,6 +17,7 @@
 #include <math.h>
 #include <stdio.h>
 
+#include <algorithm>
 #include <mutex>
 
 #include "../../include/aoh.h"
@@ -138,16 +139,18 @@ aoh_status noalloc_step(const aoh_config* cfg, const uint8_t* head_labels, void*
   const long long t1 = (long long)max_len + 1;
   const long long win = t1 < c.sink + c.window ? t1 : c.sink + c.window;
   const long long total = (long long)c.batch * ((long long)n_r * t1 + (long long)n_s * win);
-  int n_ctas = decode_ctas(total, num_sms, c.d_head, G);
+  DecodeArgs a;
+  if (decode_uses_tc(c.d_head, G))
+    decode_tc_split(a, g, t1, total, num_sms);
+  else
+    a.n_ctas = decode_cc_ctas(total, num_sms);
   const int cap_ctas = (int)(kNoAllocPartialBytes / (decode_partial_floats(1, G, c.d_head) * 4));
-  if (n_ctas > cap_ctas) n_ctas = cap_ctas;
-  if (n_ctas > kNoAllocMaxCtas) n_ctas = kNoAllocMaxCtas;
+  if (a.cluster == 0) a.n_ctas = std::min({a.n_ctas, cap_ctas, kNoAllocMaxCtas});
   // err, done and the arrival counters start at zero: the array is
   // zero-initialised, and every launch leaves them at zero (self-cleaning,
   // timeouts included), so consecutive calls need no clearing launch and
   // each decode launch overlaps the previous one's tail (programmatic
   // dependent launch).
-  DecodeArgs a;
   if (!make_cache_region_maps(&a.tcr, &a.tcs, g, kv_buffer))
     return set_err(AOH_ERR_CUDA, "aoh_decode_step_noalloc: cuTensorMapEncodeTiled failed");
   a.geom = g;
@@ -162,13 +165,13 @@ aoh_status noalloc_step(const aoh_config* cfg, const uint8_t* head_labels, void*
   a.counters = header + 64;
   a.gcounters = header + 64 + items;
   a.partials = reinterpret_cast<float*>(static_cast<unsigned char*>(scratch) + kNoAllocHeaderBytes);
-  a.n_ctas = n_ctas;
-  if (decode_uses_tc(c.d_head, G)) a.item_cost = decode_tc_item_cost(total, n_ctas, num_sms);
   a.self_clean = 1;
   a.status = header + kStatusWord;
+  if (a.cluster > 0) a.err = a.status;
   // the self-test stalls the launch's last CTA: the step's last row is
   // always its, whereas an item charge can leave the first CTAs without rows
-  a.stall_cta = stall_cta >= 0 ? n_ctas - 1 : -1;
+  // (on the cluster split the first CTA holds the first item's first row)
+  a.stall_cta = stall_cta < 0 ? -1 : a.cluster > 0 ? 0 : a.n_ctas - 1;
   a.scale_log2 = (float)(1.4426950408889634 / sqrt((double)c.d_head));
   e = launch_decode(a, s);
   if (e != cudaSuccess) return set_err(AOH_ERR_CUDA, "aoh_decode_step_noalloc: kernel launch failed");

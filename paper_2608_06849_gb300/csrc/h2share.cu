@@ -36,6 +36,7 @@
 //      overflowed walks its run again, 128 rows at a time.
 #include <stdint.h>
 
+#include "cluster.cuh"
 #include "common.cuh"
 #include "internal.h"
 
@@ -56,33 +57,6 @@ constexpr int kRegion = kClus * kCandC * 8 > kBins * 4 ? kClus * kCandC * 8 : kB
 constexpr int kTopSmem = kSliceCap * 4 + kBins * 4 + kRegion + kWarps * kKeepW * 8;
 static_assert(kClus * kWarps == 128, "CTA 0 plans four warps per lane");
 static_assert(kRegion % 16 == 0, "16-byte aligned list region");
-
-__device__ __forceinline__ uint32_t cluster_rank() {
-  uint32_t r;
-  asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
-  return r;
-}
-// Address of `p`'s counterpart in the shared memory of cluster CTA `rank`.
-__device__ __forceinline__ uint32_t cluster_addr(const void* p, uint32_t rank) {
-  uint32_t a;
-  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"(smem_u32(p)), "r"(rank));
-  return a;
-}
-__device__ __forceinline__ void cluster_red_add(uint32_t addr, uint32_t v) {
-  asm volatile("red.relaxed.cluster.shared::cluster.add.u32 [%0], %1;" ::"r"(addr), "r"(v) : "memory");
-}
-__device__ __forceinline__ void cluster_st(uint32_t addr, uint32_t x) {
-  asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(addr), "r"(x) : "memory");
-}
-__device__ __forceinline__ void cluster_st2(uint32_t addr, uint32_t x, uint32_t y) {
-  asm volatile("st.shared::cluster.v2.u32 [%0], {%1, %2};" ::"r"(addr), "r"(x), "r"(y) : "memory");
-}
-__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
-__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
-__device__ __forceinline__ void cluster_sync() {
-  cluster_arrive();
-  cluster_wait();
-}
 
 __device__ __forceinline__ int warp_inclusive_scan(int v) {
   const int lane = threadIdx.x & 31;

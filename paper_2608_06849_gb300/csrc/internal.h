@@ -98,6 +98,11 @@ struct DecodeArgs {
   // Work units charged ahead of each non-empty item's first row (the cost of
   // a CTA's switch to it), so the CTA that switches owns fewer rows.
   int item_cost = 0;
+  // CTAs per cluster when the step runs on the cluster split (tcgen05 kernel;
+  // n_ctas is a multiple of it), 0 on the stream-K split. On the cluster split
+  // `err` is the word that takes every flag of the launch (the sticky status
+  // word when there is one).
+  int cluster = 0;
   uint8_t idx_map[kMaxKvHeads] = {};
 };
 
@@ -164,9 +169,6 @@ void h2_decode_outputs(float* ws, int B, int n_r, int G, int max_seq, float** sc
 // lengths after the anchor step's append.
 cudaError_t launch_h2_topk(float* ws, int max_seq, const int32_t* lens, int B, int n_r, int G, int top_k,
                            int32_t* idx_out, cudaStream_t s);
-// CTAs for a decode launch over `total_rows` cached rows on `num_sms` SMs
-// (the kernel is chosen by D and G).
-int decode_ctas(long long total_rows, int num_sms, int D, int G);
 // The tcgen05 decode kernel serves (D, G) (else the CUDA-core kernel does).
 bool decode_uses_tc(int D, int G);
 // Work units of a gathered row and of a contiguous row in the reuse step's
@@ -182,6 +184,16 @@ void reuse_tc_weights(int G, int* gather_w, int* ring_w);
 int decode_tc_item_cost(long long total_rows, int n_ctas, int num_sms);
 int decode_tc_ctas(long long total_rows, int num_sms);
 cudaError_t launch_decode_tc(const DecodeArgs& a, cudaStream_t s);
+cudaError_t launch_decode_tc_reuse(const DecodeArgs& a, cudaStream_t s);
+// Clusters of `size` CTAs of the tcgen05 decode kernel that the current device
+// runs at once.
+int decode_tc_max_clusters(int size);
+cudaError_t launch_decode_tc_cluster(const DecodeArgs& a, int cluster, cudaStream_t s);
+// Split of a plain or anchor step on the tcgen05 kernel, whose longest
+// sequence attends `longest` rows on a retrieval head and whose items hold
+// total_rows rows in all (upper bounds will do): sets a.n_ctas, a.item_cost and
+// a.cluster.
+void decode_tc_split(DecodeArgs& a, const CacheGeom& g, long long longest, long long total_rows, int num_sms);
 // Floats of the partial buffer for `n_ctas` CTAs.
 size_t decode_partial_floats(int n_ctas, int G, int D);
 cudaError_t launch_append(const AppendArgs& a, cudaStream_t s);

@@ -104,7 +104,7 @@ size_t bytes_for(const aoh_config& c, int n_r, int n_s) {
 void aoh::record_error(const char* msg) { g_last_error = msg; }
 
 struct aoh_cache {
-  CUtensorMap tcr, tcs;  // cache regions for TMA (built once: the buffer does not move)
+  DecodeArgs maps;  // the decode step's tensor maps (built once: the buffer does not move)
   aoh_config cfg;
   CacheGeom geom;
   std::vector<uint8_t> labels;
@@ -248,7 +248,7 @@ aoh_status aoh_cache_init(const aoh_config* cfg, const uint8_t* head_labels, voi
   h->d_done = h->d_gcounters + n_gcnt;
   h->d_err = h->d_done + 32;
   h->d_partials = reinterpret_cast<float*>(base + 2 * n_lens + n_cnt + n_gcnt + 64);
-  if (!make_cache_region_maps(&h->tcr, &h->tcs, h->geom, h->kv)) {
+  if (!make_decode_maps(&h->maps, h->geom, h->kv)) {
     cudaFree(h->meta);
     delete h;
     return fail(AOH_ERR_CUDA, "cuTensorMapEncodeTiled failed for the cache regions");
@@ -445,8 +445,10 @@ aoh_status prepare_decode(const void* q, const void* k_new, const void* v_new, a
     longest = std::max(longest, t1);
     total += g.n_r * t1 + g.n_s * std::min<long long>(t1, g.S + g.W);
   }
-  a.tcr = cache->tcr;
-  a.tcs = cache->tcs;
+  a.tcr = cache->maps.tcr;
+  a.tcs = cache->maps.tcs;
+  a.tcr_odd = cache->maps.tcr_odd;
+  a.tcs_odd = cache->maps.tcs_odd;
   a.geom = g;
   a.q = q;
   a.k_new = k_new;
@@ -474,11 +476,8 @@ aoh_status aoh_decode_step(const void* q, const void* k_new, const void* v_new, 
   const aoh_status st = prepare_decode(q, k_new, v_new, cache, out, a, total, longest);
   if (st != AOH_OK) return st;
   const CacheGeom& g = cache->geom;
-  if (decode_uses_tc(g.D, g.G))
-    decode_tc_split(a, g, longest, total, cache->num_sms);
-  else
-    a.n_ctas = decode_cc_ctas(total, cache->num_sms);
-  cudaError_t e = launch_decode(a, (cudaStream_t)stream);
+  decode_tc_split(a, g, longest, total, cache->num_sms);
+  cudaError_t e = launch_decode_tc(a, (cudaStream_t)stream);
   if (e != cudaSuccess) return cuda_fail(e, "decode kernel launch");
   for (int b = 0; b < g.B; ++b) cache->lens[b] += 1;
   return AOH_OK;
@@ -502,7 +501,7 @@ aoh_status aoh_decode_step_anchor(const void* q, const void* k_new, const void* 
   if (g.n_r > 0) h2_decode_outputs(cache->d_h2, g.B, g.n_r, g.G, g.max_seq, &a.scores, &a.score_stride, &a.score_stats);
   decode_tc_split(a, g, longest, total, cache->num_sms);
   cudaStream_t s = (cudaStream_t)stream;
-  cudaError_t e = launch_decode(a, s);
+  cudaError_t e = launch_decode_tc(a, s);
   if (e != cudaSuccess) return cuda_fail(e, "decode kernel launch");
   for (int b = 0; b < g.B; ++b) cache->lens[b] += 1;
   if (g.n_r > 0) {

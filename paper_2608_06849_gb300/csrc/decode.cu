@@ -1,9 +1,8 @@
 // Split-KV flash-decode for head-heterogeneous attention on CUDA cores (Sec.
-// 5, "Decode Stage", Eq. 8): one new token per sequence; retrieval KV heads
-// attend over their whole history, streaming KV heads over their S sink + W
-// window slots. This kernel serves d_head 64 (d_head 128 runs on the tensor
-// cores, decode_tc.cu), including the d_head 64 H2Share reuse step, whose
-// retrieval rows are borrowed positions gathered one row at a time.
+// 5, "Decode Stage", Eq. 8): the H2Share reuse step of d_head 64, whose
+// retrieval heads attend to borrowed positions, gathered one row at a time, and
+// whose streaming heads attend over their S sink + W window slots. Every other
+// step runs on the tensor cores (decode_tc.cuh).
 //
 // One CTA = one (sequence b, KV head, split) work unit; a split is a
 // contiguous range of cache rows. All G query heads of the GQA group are
@@ -479,14 +478,9 @@ cudaError_t launch_cfg(const DecodeArgs& a, cudaStream_t s) {
 
 }  // namespace
 
-bool decode_cc_supported(int D, int G) {
-  return (D == 64 || D == 128) && (G == 1 || G == 2 || G == 4 || G == 7 || G == 8);
-}
+bool decode_cc_supported(int D, int G) { return D == 64 && (G == 1 || G == 2 || G == 4 || G == 7 || G == 8); }
 
-bool decode_supported(int D, int G) {
-  if (D == 128) return decode_uses_tc(D, G);
-  return decode_cc_supported(D, G);
-}
+bool decode_supported(int D, int G) { return decode_on_tc(D, G); }
 
 // Two CTAs fit on an SM (about 100 KB of shared memory each), so 2 x SMs
 // CTAs run as one wave; small launches use fewer, at least 256 rows each.
@@ -505,16 +499,9 @@ cudaError_t launch_decode_cc(const DecodeArgs& args, cudaStream_t s) {
   DecodeArgs a = args;
   a.gather_w = a.ring_w = 1;
   a.item_cost = 0;
+  a.row_keys = 1;
   const int D = a.geom.D, G = a.geom.G;
-  if (D == 128) {
-    switch (G) {
-      case 1: return launch_cfg<128, 1>(a, s);
-      case 2: return launch_cfg<128, 2>(a, s);
-      case 4: return launch_cfg<128, 4>(a, s);
-      case 7: return launch_cfg<128, 7>(a, s);
-      case 8: return launch_cfg<128, 8>(a, s);
-    }
-  } else if (D == 64) {
+  if (D == 64) {
     switch (G) {
       case 1: return launch_cfg<64, 1>(a, s);
       case 2: return launch_cfg<64, 2>(a, s);
@@ -524,11 +511,6 @@ cudaError_t launch_decode_cc(const DecodeArgs& args, cudaStream_t s) {
     }
   }
   return cudaErrorInvalidValue;
-}
-
-cudaError_t launch_decode(const DecodeArgs& a, cudaStream_t s) {
-  if (decode_uses_tc(a.geom.D, a.geom.G)) return launch_decode_tc(a, s);
-  return launch_decode_cc(a, s);
 }
 
 }  // namespace aoh

@@ -49,6 +49,10 @@ __device__ __forceinline__ int item_rows(const DecodeArgs& a, int id, const int*
   return min(t + 1, g.S + g.W);
 }
 
+// Rows as the split counts them: a.row_keys cache rows each (2 where the
+// kernel takes neighbouring keys in pairs).
+__device__ __forceinline__ int split_rows(const DecodeArgs& a, int rows) { return a.row_keys == 2 ? (rows + 1) / 2 : rows; }
+
 // Work units of item `id`: its rows, weighted in the reuse step by gather_w
 // (gathered rows) and ring_w (contiguous rows). The CTAs split the units
 // equally.
@@ -60,7 +64,7 @@ __device__ __forceinline__ int item_weight(const DecodeArgs& a, int id) {
 // the cost of switching to it, charged to the CTA whose range holds its
 // start.
 __device__ __forceinline__ long long item_units(const DecodeArgs& a, int id, const int* lens_s = nullptr) {
-  const int rows = item_rows(a, id, lens_s);
+  const int rows = split_rows(a, item_rows(a, id, lens_s));
   return rows > 0 ? (long long)rows * item_weight(a, id) + a.item_cost : 0;
 }
 
@@ -68,13 +72,15 @@ __device__ __forceinline__ long long item_units(const DecodeArgs& a, int id, con
 // [start, end) owns: row r sits at unit off + cost + r * w, so every row
 // belongs to exactly one CTA. lo >= hi when the CTA owns none.
 struct Span {
+  int keys;  // cache rows of the item; the other fields count split rows
   int rows, w, cost, lo, hi;
   long long units;
 };
 __device__ __forceinline__ Span item_span(const DecodeArgs& a, int id, const int* lens_s, long long off,
                                           long long start, long long end) {
   Span s;
-  s.rows = item_rows(a, id, lens_s);
+  s.keys = item_rows(a, id, lens_s);
+  s.rows = split_rows(a, s.keys);
   s.w = item_weight(a, id);
   s.cost = s.rows > 0 ? a.item_cost : 0;
   s.units = (long long)s.rows * s.w + s.cost;
@@ -419,7 +425,7 @@ __device__ __forceinline__ void finish_launch(const DecodeArgs& a, const int* le
 constexpr int kClusterItems = 32;  // most items of a step on this split
 constexpr int kClusterMax = 16;    // most CTAs of a cluster
 // words of the plan in shared memory
-constexpr int kPlanItem = 0, kPlanFlag = 1, kPlanLo = 2, kPlanHi = 3, kPlanParts = 4, kPlanFirst = 5;
+constexpr int kPlanItem = 0, kPlanFlag = 1, kPlanLo = 2, kPlanHi = 3, kPlanParts = 4, kPlanFirst = 5, kPlanKeys = 6;
 
 // Receive buffer: [C] values of the share, then [C][G] (m, l).
 __host__ __device__ constexpr int recv_floats(int G, int D) { return G * D + 2 * kClusterMax * G; }
@@ -436,7 +442,8 @@ __device__ __forceinline__ void plan_clusters(const DecodeArgs& a, const int* le
   const int n_items = g.B * (g.n_r + g.n_s);
   const int lane = threadIdx.x & 31;
   const int C = (int)cluster_ctas(), nc = (int)gridDim.x / C, c = (int)blockIdx.x / C;
-  const int rows = lane < n_items ? item_rows(a, lane, lens_s) : 0;
+  const int keys = lane < n_items ? item_rows(a, lane, lens_s) : 0;
+  const int rows = split_rows(a, keys);
   const int total = __reduce_add_sync(kAll, rows), most = __reduce_max_sync(kAll, rows);
   const int active = __popc(__ballot_sync(kAll, rows > 0));
   const int lo = max(1, (total + nc - 1) / nc);
@@ -463,11 +470,12 @@ __device__ __forceinline__ void plan_clusters(const DecodeArgs& a, const int* le
   const int item = past ? __ffs(past) - 1 : n_items;
   const int src = item < 32 ? item : 31;
   const int first = __shfl_sync(kAll, inc - n, src), parts = __shfl_sync(kAll, n, src);
-  const int r = __shfl_sync(kAll, rows, src);
+  const int r = __shfl_sync(kAll, rows, src), rk = __shfl_sync(kAll, keys, src);
   if (lane == 0) {
     plan[kPlanItem] = item;
     plan[kPlanParts] = parts;
     plan[kPlanFirst] = first * C;
+    plan[kPlanKeys] = rk;
     int l = 0, h = 0;
     if (item < n_items) {
       int per = (r + parts * C - 1) / (parts * C);
@@ -481,8 +489,8 @@ __device__ __forceinline__ void plan_clusters(const DecodeArgs& a, const int* le
   }
 }
 
-// Each thread holds row d = threadIdx.x of the CTA's O^T and the states m, l
-// of its heads: the values go to the CTA whose share they belong to, the
+// Thread t < D holds row d = t of the CTA's O^T and every thread the
+// states m, l of its heads: the values go to the CTA whose share they belong to, the
 // states to every CTA of the cluster.
 template <int G, int D>
 __device__ __forceinline__ void cluster_push(float* recv, const uint32_t* o, const float* m, const float* l) {
@@ -490,6 +498,7 @@ __device__ __forceinline__ void cluster_push(float* recv, const uint32_t* o, con
   const int share = G * D / C;
 #pragma unroll
   for (int h = 0; h < G; ++h) {
+    if (t >= D) break;
     const int e = h * D + t, dst = e * C / (G * D);
     cluster_st_f32(cluster_addr(recv + me * share + (e - dst * share), dst), __uint_as_float(o[h]));
   }

@@ -140,10 +140,7 @@ aoh_status noalloc_step(const aoh_config* cfg, const uint8_t* head_labels, void*
   const long long win = t1 < c.sink + c.window ? t1 : c.sink + c.window;
   const long long total = (long long)c.batch * ((long long)n_r * t1 + (long long)n_s * win);
   DecodeArgs a;
-  if (decode_uses_tc(c.d_head, G))
-    decode_tc_split(a, g, t1, total, num_sms);
-  else
-    a.n_ctas = decode_cc_ctas(total, num_sms);
+  decode_tc_split(a, g, t1, total, num_sms);
   const int cap_ctas = (int)(kNoAllocPartialBytes / (decode_partial_floats(1, G, c.d_head) * 4));
   if (a.cluster == 0) a.n_ctas = std::min({a.n_ctas, cap_ctas, kNoAllocMaxCtas});
   // err, done and the arrival counters start at zero: the array is
@@ -151,7 +148,7 @@ aoh_status noalloc_step(const aoh_config* cfg, const uint8_t* head_labels, void*
   // timeouts included), so consecutive calls need no clearing launch and
   // each decode launch overlaps the previous one's tail (programmatic
   // dependent launch).
-  if (!make_cache_region_maps(&a.tcr, &a.tcs, g, kv_buffer))
+  if (!make_decode_maps(&a, g, kv_buffer))
     return set_err(AOH_ERR_CUDA, "aoh_decode_step_noalloc: cuTensorMapEncodeTiled failed");
   a.geom = g;
   a.q = q;
@@ -173,7 +170,7 @@ aoh_status noalloc_step(const aoh_config* cfg, const uint8_t* head_labels, void*
   // (on the cluster split the first CTA holds the first item's first row)
   a.stall_cta = stall_cta < 0 ? -1 : a.cluster > 0 ? 0 : a.n_ctas - 1;
   a.scale_log2 = (float)(1.4426950408889634 / sqrt((double)c.d_head));
-  e = launch_decode(a, s);
+  e = launch_decode_tc(a, s);
   if (e != cudaSuccess) return set_err(AOH_ERR_CUDA, "aoh_decode_step_noalloc: kernel launch failed");
   return AOH_OK;
 }

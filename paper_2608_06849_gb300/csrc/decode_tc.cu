@@ -8,7 +8,11 @@ namespace aoh {
 
 using namespace dtc;
 
-bool decode_uses_tc(int D, int G) { return D == kD && ((G >= 1 && G <= 8) || G == 16); }
+bool decode_uses_tc(int D, int G) { return D == 128 && ((G >= 1 && G <= 8) || G == 16); }
+
+bool decode_on_tc(int D, int G) {
+  return decode_uses_tc(D, G) || (D == 64 && (G == 1 || G == 2 || G == 4 || G == 7 || G == 8));
+}
 
 int decode_tc_item_cost(long long total_rows, int n_ctas, int num_sms) {
   if (total_rows >= kItemCostMaxShare * n_ctas) return 0;
@@ -61,11 +65,15 @@ long long clusters_for(long long n, long long rows, int C, int k) {
 // larger sizes run out of clusters.
 void decode_tc_split(DecodeArgs& a, const CacheGeom& g, long long longest, long long total_rows, int num_sms) {
   constexpr int kSpared = 6;
+  a.row_keys = g.D == 64 ? 2 : 1;
+  long long ring = std::min<long long>(longest, (long long)g.S + g.W);
+  longest = (longest + a.row_keys - 1) / a.row_keys;
+  ring = (ring + a.row_keys - 1) / a.row_keys;
+  total_rows = (total_rows + a.row_keys - 1) / a.row_keys;
   a.cluster = 0;
   a.n_ctas = decode_tc_ctas(total_rows, num_sms);
   a.item_cost = decode_tc_item_cost(total_rows, a.n_ctas, num_sms);
   const long long n_r = (long long)g.B * g.n_r, n_s = (long long)g.B * g.n_s;
-  const long long ring = std::min<long long>(longest, (long long)g.S + g.W);
   const long long widest = g.n_r > 0 ? longest : ring;
   if (n_r + n_s > dec::kClusterItems || widest * (n_r + n_s) > (1ll << 30)) return;
   const long long even = (n_r * longest + n_s * ring + (long long)kBN * num_sms - 1) / ((long long)kBN * num_sms);
@@ -91,8 +99,9 @@ void decode_tc_split(DecodeArgs& a, const CacheGeom& g, long long longest, long 
 // The reuse step (a.idx set) launches the variant with gather warps.
 cudaError_t launch_decode_tc(const DecodeArgs& a, cudaStream_t s) {
   if (a.idx != nullptr) return launch_decode_tc_reuse(a, s);
+  if (a.geom.D == 64) return launch_decode_tc64(a, s);
   if (a.cluster > 0) return launch_decode_tc_cluster(a, a.cluster, s);
-  return launch_mode<kStream>(a, 1, s);
+  return launch_mode<128, kStream>(a, 1, s);
 }
 
 }  // namespace aoh

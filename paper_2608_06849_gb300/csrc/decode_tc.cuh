@@ -1,5 +1,5 @@
 // Split-KV decode on tcgen05 tensor cores (Sec. 5, "Decode Stage", Eq. 8;
-// d_head = 128, GQA groups of 1-8 and 16). With G query heads per KV head,
+// d_head 128 with GQA groups of 1-8 and 16, d_head 64 with 1, 2, 4, 7 and 8). With G query heads per KV head,
 // every cached K/V row meets G queries: 4*G*d flops per 4*d bytes. On CUDA
 // cores that arithmetic (plus the shuffles that reduce the dot products)
 // stops hiding under the HBM stream above g = 4, and even at g = 4 it costs a
@@ -9,6 +9,7 @@
 //   S^T[128 keys][16]  = K_tile[128][d] . Q^T           (A = K, K-major; B = Q, K-major)
 //   O^T[d][16]        += V_tile^T[d][128] . P^T[128][16] (A = V, MN-major; B = P, K-major)
 //
+// (d_head 128; d_head 64 puts two keys into an MMA row, see Lay.)
 // Both accumulators live in TMEM: S^T in one of two 16-column buffers (row =
 // key), O^T in 16 more columns (row = d). The split of the step's rows over
 // CTAs, the partial format and the merge are those of the CUDA-core kernel
@@ -56,14 +57,11 @@ namespace aoh {
 namespace dtc {
 
 using bf16 = __nv_bfloat16;
-constexpr int kD = 128;
 constexpr int kBN = 128;                   // keys per tile
 constexpr int kN = 16;                     // N of both MMAs (query heads, padded)
 constexpr int kNS = 3;                     // ring stages
 constexpr int kThreads = 192;              // warps 0-5 (see the file comment)
 constexpr int kSoftmaxThreads = 128;
-constexpr uint32_t kTmemCols = 64;         // S[0] [0,16), S[1] [16,32), O [32,48)
-constexpr uint32_t kOcol = 32;
 constexpr float kRescaleThreshold = 8.0f;  // log2 units
 // Rows charged for a switch from one item to the next (DecodeArgs::
 // item_cost), in steps whose CTAs hold fewer than kItemCostMaxShare rows
@@ -87,24 +85,54 @@ constexpr long long kItemCostMaxShare = 16384;
 constexpr int kBox = kBN * 64 * 2;         // one [128 rows][64] TMA box, 16 KB
 constexpr int kTile = 2 * kBox;            // a K or V tile (d = 128)
 constexpr int kStage = 2 * kTile;          // K then V
-constexpr int kOpBuf = 2 * kN * 128;       // [16 rows][128] bf16 operand, two 64-wide blocks
-constexpr int OFF_KV = 0;
-constexpr int OFF_Q = OFF_KV + kNS * kStage;
-constexpr int OFF_P = OFF_Q + 2 * kOpBuf;
-constexpr int OFF_RED = OFF_P + 2 * kOpBuf;   // [2][4][16] warp maxima, [4][16] warp sums
-constexpr int OFF_MS = OFF_RED + (2 * 64 + 64) * 4;
-constexpr int MS_FLOATS = 1024;               // merge scratch
-constexpr int OFF_BAR = OFF_MS + MS_FLOATS * 4;
-constexpr int NBAR = 3 * kNS + 2 + 2 + 2 + 2 + 1 + 1;
-constexpr int OFF_MISC = OFF_BAR + NBAR * 8;
-constexpr int kLensCap = 2048;                // sequence lengths mirrored in shared memory
-constexpr int OFF_LENS = OFF_MISC + 64;
-constexpr int SMEM = OFF_LENS + kLensCap * 4 + 4096 + 1024;
-static_assert(dec::kClusterItems * 4 + dec::recv_floats(kN, kD) * 4 <= kLensCap * 4 + 4096, "receive buffer");
-constexpr uint32_t IDESC_S = idesc_bf16(kBN, kN, false, false);
-constexpr uint32_t IDESC_PV = idesc_bf16(kD, kN, false, true);
-static_assert(SMEM <= 232448, "shared memory");
-static_assert(OFF_Q % 1024 == 0 && OFF_P % 1024 == 0, "operand alignment");
+
+// Shapes and shared memory of one head size and group. At d_head 128 an MMA row
+// is one key. At d_head 64 it is a pair of neighbouring keys, whose two 128-byte
+// rows fill the two 64-wide column blocks of the same tile: the scores of the
+// even and of the odd keys are two MMA sets over one block each, and P has a
+// column per head and parity. O^T then holds the even keys' sum in rows 0-63 of
+// the even columns and the odd keys' in rows 64-127 of the odd ones (the other
+// halves are not used). P keeps its 24 bits at d_head 64: each weight is the
+// sum of three bf16 parts, each a column of its own (outputs as close to 64 bits
+// as with fp32 weights: both are the rounded exact value in 99.9% of 2,048
+// outputs at 100K keys). On CUDA cores this head size was bound by the shuffles
+// and FMAs of the dot products, 3.6 TB/s where this kernel reaches 5.0: a step
+// of 8 sequences of 12K-32K keys, 32/8 heads, half of them streaming (213 MB),
+// went from 59.5 to 45.7 us, a length copy included.
+template <int D, int G>
+struct Lay {
+  static constexpr bool PAIR = D == 64;
+  static constexpr int NK = PAIR ? 2 : 1;                      // keys per MMA row
+  static constexpr int PARTS = PAIR ? 3 : 1;                   // bf16 parts of a weight
+  static constexpr int HP = PAIR ? (G <= 4 ? 4 : 8) : kN;      // P columns of one parity
+  static constexpr int NP = NK * HP;                           // P columns of one part
+  static constexpr int NPV = (PARTS * NP + 15) / 16 * 16;      // N of the P V MMA
+  static constexpr int SCOLS = NK * kN;                        // TMEM columns of an S buffer
+  static constexpr uint32_t OCOL = 2 * SCOLS;                  // O after S[0], S[1]
+  static constexpr uint32_t TMEM_COLS = PAIR ? 128 : 64;
+  static constexpr int QBUF = (PAIR ? 1 : 2) * kN * 128;       // [16 rows][D], 64-wide blocks
+  static constexpr int PBUF = 2 * NPV * 128;                   // [NPV rows][128 MMA rows]
+  static constexpr int NPB = PAIR && G > 4 ? 1 : 2;            // P buffers that fit
+  static constexpr int LENS_CAP = PAIR ? 512 : 2048;           // sequence lengths mirrored in shared memory
+  static constexpr int OFF_KV = 0;
+  static constexpr int OFF_Q = OFF_KV + kNS * kStage;
+  static constexpr int OFF_P = OFF_Q + 2 * QBUF;
+  static constexpr int OFF_RED = OFF_P + NPB * PBUF;           // [2][4][16] warp maxima, [4][16] warp sums
+  static constexpr int OFF_MS = OFF_RED + (2 * 64 + 64) * 4;
+  static constexpr int MS_FLOATS = 1024;                       // merge scratch; the odd keys' O at d_head 64
+  static constexpr int OFF_BAR = OFF_MS + MS_FLOATS * 4;
+  static constexpr int NBAR = 3 * kNS + 2 + 2 + 2 + 2 + 1 + 1;
+  static constexpr int OFF_MISC = OFF_BAR + NBAR * 8;
+  static constexpr int OFF_LENS = OFF_MISC + 64;
+  static constexpr int RECV = dec::kClusterItems * 4 + dec::recv_floats(G, D) * 4;
+  static constexpr int SMEM = OFF_LENS + cmax(LENS_CAP * 4, RECV) + 1024;
+  static constexpr uint32_t IDESC_S = idesc_bf16(kBN, kN, false, false);
+  static constexpr uint32_t IDESC_PV = idesc_bf16(128, NPV, false, true);
+  static_assert(SMEM <= 232448, "shared memory");
+  static_assert(OFF_Q % 1024 == 0 && OFF_P % 1024 == 0 && PBUF % 1024 == 0, "operand alignment");
+  static_assert(OCOL + NPV <= TMEM_COLS, "TMEM columns");
+  static_assert(!PAIR || G * 64 <= MS_FLOATS, "exchange of the odd keys' O");
+};
 
 // Variants of the kernel: the stream-K split; the reuse step's, with gather
 // warps; and the split by whole clusters (short steps of few items).
@@ -145,6 +173,7 @@ struct Walk {
     }
     return false;
   }
+  __device__ __forceinline__ int keys() const { return sp.keys; }
   // another item of the range may follow: it starts at its row 0
   __device__ __forceinline__ bool more() const { return off < end && id + 1 < n_items; }
 };
@@ -158,6 +187,7 @@ struct Walk<true> {
   __device__ __forceinline__ Walk(const DecodeArgs&, const int*, int, long long, long long, int first, long long,
                                   const int* plan)
       : id(first) {
+    sp.keys = plan[dec::kPlanKeys];
     sp.lo = plan[dec::kPlanLo];
     sp.hi = plan[dec::kPlanHi];
     left = sp.lo < sp.hi;
@@ -167,6 +197,7 @@ struct Walk<true> {
     left = false;
     return r;
   }
+  __device__ __forceinline__ int keys() const { return sp.keys; }
   __device__ __forceinline__ bool more() const { return false; }
 };
 
@@ -176,24 +207,28 @@ struct Walk<true> {
 // MODE kCluster: the CTAs of a cluster share one item (dec::plan_clusters) and
 // add up their states through distributed shared memory
 // (dec::cluster_finish); see decode_tc_cluster.cu.
-template <int G, int MODE>
+template <int D, int G, int MODE>
 __global__ void __launch_bounds__(kThreads + 32 * gather_warps(G, MODE), 1)
     decode_tc_kernel(const __grid_constant__ DecodeArgs a) {
   constexpr bool GATHER = MODE == kGather, CLUSTER = MODE == kCluster;
+  using C = Lay<D, G>;
+  constexpr bool PAIR = C::PAIR;
+  constexpr int NK = C::NK;
+  static_assert(!(GATHER && PAIR), "borrowed rows of d_head 64 run on the CUDA cores");
   static_assert(G >= 1 && G <= kN, "group size");
   constexpr int GW = gather_warps(G, MODE);
   constexpr int RPW = GATHER ? kBN / GW : kBN;  // rows of each tile a gather warp copies
   constexpr int NT = kThreads + 32 * GW;
-  static_assert(2 * (dec::kGroup + 8) * G + 2 * G <= MS_FLOATS, "merge scratch");
+  static_assert(2 * (dec::kGroup + 8) * G + 2 * G <= C::MS_FLOATS, "merge scratch");
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = smem_raw + ((1024 - (smem_u32(smem_raw) & 1023)) & 1023);
-  uint8_t* sKV = smem + OFF_KV;
-  uint8_t* sQ = smem + OFF_Q;
-  uint8_t* sP = smem + OFF_P;
-  float* red = reinterpret_cast<float*>(smem + OFF_RED);  // [2][4][16]
+  uint8_t* sKV = smem + C::OFF_KV;
+  uint8_t* sQ = smem + C::OFF_Q;
+  uint8_t* sP = smem + C::OFF_P;
+  float* red = reinterpret_cast<float*>(smem + C::OFF_RED);  // [2][4][16]
   float* lsum = red + 2 * 64;                             // [4][16]
-  float* ms = reinterpret_cast<float*>(smem + OFF_MS);
-  uint64_t* full = reinterpret_cast<uint64_t*>(smem + OFF_BAR);  // [kNS] a TMA-loaded tile landed
+  float* ms = reinterpret_cast<float*>(smem + C::OFF_MS);
+  uint64_t* full = reinterpret_cast<uint64_t*>(smem + C::OFF_BAR);  // [kNS] a TMA-loaded tile landed
   uint64_t* empty = full + kNS;
   uint64_t* gfull = empty + kNS;    // [kNS] a gathered tile landed (reuse variant)
   uint64_t* s_full = gfull + kNS;   // [2] S(j) in TMEM
@@ -202,13 +237,13 @@ __global__ void __launch_bounds__(kThreads + 32 * gather_warps(G, MODE), 1)
   uint64_t* p_free = p_full + 2;    // [2] O += P(j) V(j) done
   uint64_t* o_free = p_free + 2;    // the item's final O read
   uint64_t* drain = o_free + 1;
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smem + OFF_MISC);
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smem + C::OFF_MISC);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
-  long long* sh64 = reinterpret_cast<long long*>(smem + OFF_MISC + 8);  // [0] total, [1] first offset
+  long long* sh64 = reinterpret_cast<long long*>(smem + C::OFF_MISC + 8);  // [0] total, [1] first offset
   int* sh32 = reinterpret_cast<int*>(sh64 + 2);                         // [0] first item, [1] merge flag
-  int* lens_s = reinterpret_cast<int*>(smem + OFF_LENS);
+  int* lens_s = reinterpret_cast<int*>(smem + C::OFF_LENS);
   // cluster split: the states of the cluster's CTAs for this CTA's share of the output
-  float* recv = reinterpret_cast<float*>(smem + OFF_LENS + dec::kClusterItems * 4);
+  float* recv = reinterpret_cast<float*>(smem + C::OFF_LENS + dec::kClusterItems * 4);
 
   const CacheGeom& g = a.geom;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -219,7 +254,7 @@ __global__ void __launch_bounds__(kThreads + 32 * gather_warps(G, MODE), 1)
   // Prologue that touches no global memory; it may overlap the tail of the
   // previous kernel on the stream (programmatic dependent launch).
   // Q and P rows >= G stay zero for the whole launch
-  for (int i = threadIdx.x; i < 4 * kOpBuf / 16; i += NT)
+  for (int i = threadIdx.x; i < (2 * C::QBUF + C::NPB * C::PBUF) / 16; i += NT)
     reinterpret_cast<uint4*>(sQ)[i] = make_uint4(0, 0, 0, 0);
   fence_proxy_async_smem();
   if (threadIdx.x == 0) {
@@ -240,7 +275,7 @@ __global__ void __launch_bounds__(kThreads + 32 * gather_warps(G, MODE), 1)
     fence_mbar_init();
   }
   if (warp == 5) {
-    tmem_alloc(tmem_slot, kTmemCols);
+    tmem_alloc(tmem_slot, C::TMEM_COLS);
     tmem_relinquish();
   }
   tc_fence_before();
@@ -255,7 +290,7 @@ __global__ void __launch_bounds__(kThreads + 32 * gather_warps(G, MODE), 1)
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   // the lengths cannot change during the launch (the last CTA to finish
   // advances them), so every role reads this copy
-  const int* ls = g.B <= kLensCap ? lens_s : nullptr;
+  const int* ls = g.B <= C::LENS_CAP ? lens_s : nullptr;
   if (ls != nullptr) {
     for (int i = threadIdx.x; i < g.B; i += NT) lens_s[i] = __ldcg(&a.lens[i]);
     __syncthreads();
@@ -284,6 +319,8 @@ __global__ void __launch_bounds__(kThreads + 32 * gather_warps(G, MODE), 1)
     if (!GATHER && lane == 0) {
       if (g.n_r > 0) prefetch_tmap(&a.tcr);
       if (g.n_s > 0) prefetch_tmap(&a.tcs);
+      if (PAIR && g.n_r > 0) prefetch_tmap(&a.tcr_odd);
+      if (PAIR && g.n_s > 0) prefetch_tmap(&a.tcs_odd);
       int it = 0;
       bool ok = true;
       while (ok && walk.next()) {
@@ -292,6 +329,7 @@ __global__ void __launch_bounds__(kThreads + 32 * gather_warps(G, MODE), 1)
         const bool strm = k >= g.n_r;
         const int region = strm ? b * g.n_s + (k - g.n_r) : b * g.n_r + k;
         const CUtensorMap* map = strm ? &a.tcs : &a.tcr;
+        const CUtensorMap* map_odd = strm ? &a.tcs_odd : &a.tcr_odd;
         for (int row0 = lo; row0 < hi; row0 += kBN, ++it) {
           const int st = it % kNS;
           if (it >= kNS && !wait_bar(&empty[st], ((it / kNS) & 1) ^ 1, a.err, abort_flag)) {
@@ -304,7 +342,8 @@ __global__ void __launch_bounds__(kThreads + 32 * gather_warps(G, MODE), 1)
           for (int sel = 0; sel < 2; ++sel)
 #pragma unroll
             for (int db = 0; db < 2; ++db)
-              tma_load_4d(dst + sel * kTile + db * kBox, map, db * 64, row0, sel, region, &full[st]);
+              tma_load_4d(dst + sel * kTile + db * kBox, PAIR && db == 1 ? map_odd : map, PAIR ? 0 : db * 64, row0,
+                          sel, region, &full[st]);
         }
       }
       if constexpr (CLUSTER) dec::advance_lens(a, lens_s);
@@ -373,9 +412,9 @@ __global__ void __launch_bounds__(kThreads + 32 * gather_warps(G, MODE), 1)
       const int32_t* rowlist = a.idx + ((size_t)b * a.n_idx_groups + a.idx_map[k]) * a.top_k;
       const int t = dec::seq_len(a, b, ls);
       const bf16* src_base =
-          static_cast<const bf16*>(a.kv) + g.r_region(b, k) + (half ? (size_t)g.max_seq * kD : 0) + ch * 8;
+          static_cast<const bf16*>(a.kv) + g.r_region(b, k) + (half ? (size_t)g.max_seq * D : 0) + ch * 8;
       const bf16* src_new =
-          static_cast<const bf16*>(half ? a.v_new : a.k_new) + ((size_t)b * g.Hkv + g.r_head[k]) * kD + ch * 8;
+          static_cast<const bf16*>(half ? a.v_new : a.k_new) + ((size_t)b * g.Hkv + g.r_head[k]) * D + ch * 8;
       const bool idx_lane = lane < RPW;
       const int j0 = lo + RPW * gw + lane;
       int ia = idx_lane && j0 < hi ? __ldg(rowlist + j0) : 0;
@@ -393,7 +432,7 @@ __global__ void __launch_bounds__(kThreads + 32 * gather_warps(G, MODE), 1)
           const int r = RPW * gw + j;
           if (c >= 0)
             cp_async16(tile + r * 128 + ((swz ^ (uint32_t)(r & 7)) << 4),
-                       c == t ? src_new : src_base + (size_t)c * kD);
+                       c == t ? src_new : src_base + (size_t)c * D);
         }
         cp_async_mbar_arrive(&gfull[st]);
         __syncwarp();
@@ -449,12 +488,12 @@ __global__ void __launch_bounds__(kThreads + 32 * gather_warps(G, MODE), 1)
       if (lane == 0) {
         tc_fence_after();
         const uint32_t v_addr = kv_addr + t.st * kStage + kTile;
-        const uint32_t pb = p_addr + (t.it & 1) * kOpBuf;
+        const uint32_t pb = p_addr + (t.it % C::NPB) * C::PBUF;
 #pragma unroll
         for (int kk = 0; kk < kBN / 16; ++kk) {
           const uint64_t ad = sdesc_sw128(v_addr + kk * 2048, kBox, 1024);
-          const uint64_t bd = sdesc_sw128(pb + (kk >> 2) * (kN * 128) + (kk & 3) * 32, 16, 1024);
-          tc_mma(tmem + kOcol, ad, bd, IDESC_PV, (t.first && kk == 0) ? 0u : 1u);
+          const uint64_t bd = sdesc_sw128(pb + (kk >> 2) * (C::NPV * 128) + (kk & 3) * 32, 16, 1024);
+          tc_mma(tmem + C::OCOL, ad, bd, C::IDESC_PV, (t.first && kk == 0) ? 0u : 1u);
         }
         tc_commit(&p_free[t.it & 1]);
         tc_commit(&empty[t.st]);
@@ -466,27 +505,29 @@ __global__ void __launch_bounds__(kThreads + 32 * gather_warps(G, MODE), 1)
     // row) are fetched into registers one item ahead: under the saturated
     // HBM stream a plain load takes microseconds, which at an item switch
     // would sit between this item's last P V and the next item's first S.
-    // Lane l holds 16-byte chunks l, l + 32, ... of the G x 128 query block
-    // (head c / 16, chunk c % 16); lanes 0-15 the new K row's chunks, lanes
-    // 16-31 the new V row's.
-    constexpr int QV = (G * 16 + 31) / 32;
+    // Lane l holds 16-byte chunks l, l + 32, ... of the G x D query block (CPR
+    // chunks a head); lanes 0 .. CPR - 1 the new K row's chunks, the next CPR
+    // lanes the new V row's.
+    constexpr int CPR = D / 8;
+    constexpr int QV = (G * CPR + 31) / 32;
     uint4 qr[QV];
     uint4 nvr;
-    const int ch = lane & 15;
+    const int ch = lane % CPR;
+    const bool new_v = lane >= CPR, new_lane = lane < 2 * CPR;
     auto kv_head_of = [&](int id) {
       const int k = id % HK;
       return k >= g.n_r ? (int)g.s_head[k - g.n_r] : (int)g.r_head[k];
     };
     auto fetch_inputs = [&](int id) {
       const int b = id / HK, kvh = kv_head_of(id);
-      const bf16* qg = static_cast<const bf16*>(a.q) + ((size_t)b * g.Hq + (size_t)kvh * G) * kD;
+      const bf16* qg = static_cast<const bf16*>(a.q) + ((size_t)b * g.Hq + (size_t)kvh * G) * D;
 #pragma unroll
       for (int i = 0; i < QV; ++i) {
         const int c = lane + 32 * i;
-        if (c < G * 16) qr[i] = *reinterpret_cast<const uint4*>(qg + (size_t)(c >> 4) * kD + (c & 15) * 8);
+        if (c < G * CPR) qr[i] = *reinterpret_cast<const uint4*>(qg + (size_t)(c / CPR) * D + (c % CPR) * 8);
       }
-      const size_t new_off = ((size_t)b * g.Hkv + kvh) * kD + ch * 8;
-      nvr = *reinterpret_cast<const uint4*>(static_cast<const bf16*>(lane < 16 ? a.k_new : a.v_new) + new_off);
+      const size_t new_off = ((size_t)b * g.Hkv + kvh) * D + ch * 8;
+      nvr = *reinterpret_cast<const uint4*>(static_cast<const bf16*>(new_v ? a.v_new : a.k_new) + new_off);
     };
     int fetched = -1;  // the item whose inputs the registers hold
     if (first_id < n_items) {
@@ -503,7 +544,7 @@ __global__ void __launch_bounds__(kThreads + 32 * gather_warps(G, MODE), 1)
       const int cap = strm ? g.S + g.W : g.max_seq;
       const int xr = strm ? (t < g.S ? t : g.S + (t - g.S) % g.W) : t;  // the new token's row
       bf16* Kc = static_cast<bf16*>(a.kv) + (strm ? g.s_region(b, hi_idx) : g.r_region(b, hi_idx));
-      bf16* Vc = Kc + (size_t)cap * kD;
+      bf16* Vc = Kc + (size_t)cap * D;
 
       // this item's Q into buffer item_k & 1, last read by the MMAs of item item_k - 2
       wait_ofree(item_k - 1);
@@ -513,12 +554,12 @@ __global__ void __launch_bounds__(kThreads + 32 * gather_warps(G, MODE), 1)
         fetched = id;
       }
       {
-        uint8_t* qs = sQ + (item_k & 1) * kOpBuf;
+        uint8_t* qs = sQ + (item_k & 1) * C::QBUF;
 #pragma unroll
         for (int i = 0; i < QV; ++i) {
           const int c = lane + 32 * i;
-          if (c < G * 16) {
-            const int h = c >> 4, cc = c & 15;
+          if (c < G * CPR) {
+            const int h = c / CPR, cc = c % CPR;
             *reinterpret_cast<uint4*>(qs + (cc >> 3) * (kN * 128) + h * 128 + (((cc & 7) ^ (h & 7)) << 4)) = qr[i];
           }
         }
@@ -544,21 +585,24 @@ __global__ void __launch_bounds__(kThreads + 32 * gather_warps(G, MODE), 1)
         else
           fpar ^= 1u << st;
         if (!ok) break;
-        auto put_new_row = [&](int r) {  // the new token's K / V chunk into tile slot r
-          uint8_t* dst = sKV + st * kStage + (lane < 16 ? 0 : kTile) + (ch >> 3) * kBox + r * 128 +
-                         (((ch & 7) ^ (r & 7)) << 4);
+        auto put_new_row = [&](int r) {  // the new token's K / V chunk into tile row r
+          const int box = PAIR ? xr & 1 : ch >> 3;
+          uint8_t* dst =
+              sKV + st * kStage + (new_v ? kTile : 0) + box * kBox + r * 128 + (((ch & 7) ^ (r & 7)) << 4);
           *reinterpret_cast<uint4*>(dst) = nv;
         };
         if (gathered) {
           // the gather warps wrote this tile with cp.async (generic proxy):
           // order it before the tensor core's reads; the item's owner of row
           // 0 appends the new token
-          if (row0 == 0) *reinterpret_cast<uint4*>((lane < 16 ? Kc : Vc) + (size_t)xr * kD + ch * 8) = nv;
+          if (row0 == 0) *reinterpret_cast<uint4*>((new_v ? Vc : Kc) + (size_t)xr * D + ch * 8) = nv;
           fence_proxy_async_smem();
           __syncwarp();
-        } else if (xr >= row0 && xr < row0 + cnt) {
-          put_new_row(xr - row0);
-          *reinterpret_cast<uint4*>((lane < 16 ? Kc : Vc) + (size_t)xr * kD + ch * 8) = nv;  // append
+        } else if (xr / NK >= row0 && xr / NK < row0 + cnt) {
+          if (new_lane) {
+            put_new_row(xr / NK - row0);
+            *reinterpret_cast<uint4*>((new_v ? Vc : Kc) + (size_t)xr * D + ch * 8) = nv;  // append
+          }
           fence_proxy_async_smem();
           __syncwarp();
         }
@@ -567,12 +611,14 @@ __global__ void __launch_bounds__(kThreads + 32 * gather_warps(G, MODE), 1)
         if (lane == 0) {
           tc_fence_after();
           const uint32_t k_addr = kv_addr + st * kStage;
-          const uint32_t qb = q_addr + (item_k & 1) * kOpBuf;
+          const uint32_t qb = q_addr + (item_k & 1) * C::QBUF;
 #pragma unroll
-          for (int kk = 0; kk < kD / 16; ++kk) {
+          for (int kk = 0; kk < 8; ++kk) {
+            // d_head 128: 8 K-steps over both blocks; 64: 4 over each parity's block
+            const int y = PAIR ? kk >> 2 : 0;
             const uint64_t ad = sdesc_sw128(k_addr + (kk >> 2) * kBox + (kk & 3) * 32, 16, 1024);
-            const uint64_t bd = sdesc_sw128(qb + (kk >> 2) * (kN * 128) + (kk & 3) * 32, 16, 1024);
-            tc_mma(tmem + (it & 1) * kN, ad, bd, IDESC_S, kk > 0 ? 1u : 0u);
+            const uint64_t bd = sdesc_sw128(qb + (PAIR ? 0 : kk >> 2) * (kN * 128) + (kk & 3) * 32, 16, 1024);
+            tc_mma(tmem + (it & 1) * C::SCOLS + y * kN, ad, bd, C::IDESC_S, (PAIR ? kk & 3 : kk) > 0 ? 1u : 0u);
           }
           tc_commit(&s_full[it & 1]);
         }
@@ -615,7 +661,7 @@ __global__ void __launch_bounds__(kThreads + 32 * gather_warps(G, MODE), 1)
     bool ok = true, local_ok = true;
     uint32_t fpar = 0, gpar = 0;  // bit st: parity of stage st's next full[] / gfull[] phase
     if constexpr (CLUSTER) {
-      if (!walk.left) dec::cluster_push_empty<G, kD>(recv);
+      if (!walk.left) dec::cluster_push_empty<G, D>(recv);
     }
     while (ok && walk.next()) {
       const int id = walk.id, lo = walk.sp.lo, hi = walk.sp.hi;
@@ -640,21 +686,33 @@ __global__ void __launch_bounds__(kThreads + 32 * gather_warps(G, MODE), 1)
           fpar ^= 1u << st;
         local_ok = wait_bar(&s_full[x], (it >> 1) & 1, a.err, abort_flag) && local_ok;
         tc_fence_after();
-        uint32_t v[16];
-        tmem_ld16(tl + x * kN, v);
+        uint32_t v[NK][PAIR ? 8 : 16];
+        if constexpr (PAIR) {
+          tmem_ld8(tl + x * C::SCOLS, v[0]);
+          tmem_ld8(tl + x * C::SCOLS + kN, v[1]);
+        } else {
+          tmem_ld16(tl + x * C::SCOLS, v[0]);
+        }
         tmem_ld_wait();
         tc_fence_before();
         __syncwarp();
         if (lane == 0) mbar_arrive(&s_free[x]);
-        const bool valid = t < cnt;
-        float s[G];
+        // keys of this thread's row that the item holds (at d_head 64 the item's
+        // last pair may hold one)
+        const int kv = PAIR ? min(2 * cnt, walk.keys() - 2 * row0) : cnt;
+        bool valid[NK];
+        float s[NK][G];
 #pragma unroll
-        for (int h = 0; h < G; ++h) s[h] = valid ? __uint_as_float(v[h]) * a.scale_log2 : -INFINITY;
-        if (a.scores != nullptr && !strm && valid) {
+        for (int y = 0; y < NK; ++y) {
+          valid[y] = NK * t + y < kv;
+#pragma unroll
+          for (int h = 0; h < G; ++h) s[y][h] = valid[y] ? __uint_as_float(v[y][h]) * a.scale_log2 : -INFINITY;
+        }
+        if (!PAIR && a.scores != nullptr && !strm && valid[0]) {
           // H2Share anchor step: this row's scores for the top-k selection
           float* sc = a.scores + ((size_t)(b * g.n_r + k) * G) * a.score_stride + row0 + t;
 #pragma unroll
-          for (int h = 0; h < G; ++h) sc[(size_t)h * a.score_stride] = s[h];
+          for (int h = 0; h < G; ++h) sc[(size_t)h * a.score_stride] = s[0][h];
         }
 
         // per-head maximum over the tile: each warp, then the four warps
@@ -662,7 +720,7 @@ __global__ void __launch_bounds__(kThreads + 32 * gather_warps(G, MODE), 1)
         float wm = -INFINITY;
 #pragma unroll
         for (int h = 0; h < G; ++h) {
-          const float r = warp_max(s[h]);
+          const float r = warp_max(PAIR ? fmaxf(s[0][h], s[NK - 1][h]) : s[0][h]);
           wm = (lane == h) ? r : wm;
         }
         if (lane < G) rx[warp * 16 + lane] = wm;
@@ -682,42 +740,60 @@ __global__ void __launch_bounds__(kThreads + 32 * gather_warps(G, MODE), 1)
             resc = true;
           }
         }
-        // P buffer x is free once O += P(it - 2) V is done
-        if (it >= 2) local_ok = wait_bar(&p_free[x], ((it >> 1) - 1) & 1, a.err, abort_flag) && local_ok;
+        // the P buffer is free once O += P(it - NPB) V is done
+        if (it >= C::NPB)
+          local_ok = wait_bar(&p_free[(it - C::NPB) & 1], ((it - C::NPB) >> 1) & 1, a.err, abort_flag) && local_ok;
         if (resc && row0 != lo) {
           // rescale row t of O^T; O += P(it - 1) V must have landed first
           local_ok = wait_bar(&p_free[x ^ 1], ((it - 1) >> 1) & 1, a.err, abort_flag) && local_ok;
           tc_fence_after();
-          uint32_t o[16];
-          tmem_ld16(tl + kOcol, o);
-          tmem_ld_wait();
+          uint32_t o[C::NP];
 #pragma unroll
-          for (int h = 0; h < G; ++h) o[h] = __float_as_uint(__uint_as_float(o[h]) * alpha[h]);
-          tmem_st16(tl + kOcol, o);
+          for (int q = 0; q < C::PARTS; ++q) {
+            tmem_ld(tl + C::OCOL + q * C::NP, o);
+            tmem_ld_wait();
+#pragma unroll
+            for (int c = 0; c < C::NP; ++c)
+              if (c % C::HP < G) o[c] = __float_as_uint(__uint_as_float(o[c]) * alpha[c % C::HP]);
+            tmem_st(tl + C::OCOL + q * C::NP, o);
+          }
           tmem_st_wait();
         }
-        float pr[G];
+        float pr[NK][G];
 #pragma unroll
-        for (int h = 0; h < G; ++h) {
-          pr[h] = valid ? fast_exp2(s[h] - m[h]) : 0.f;
-          l[h] += pr[h];
-        }
-        if (!valid) {
-          // the tile has landed (its S is complete); zero V row t
+        for (int y = 0; y < NK; ++y)
+#pragma unroll
+          for (int h = 0; h < G; ++h) {
+            pr[y][h] = valid[y] ? fast_exp2(s[y][h] - m[h]) : 0.f;
+            l[h] += pr[y][h];
+          }
+        if (!valid[NK - 1]) {
+          // the tile has landed (its S is complete); zero the V rows of this
+          // thread's keys that the item does not hold (d_head 128: both halves)
           wait_bar(gathered ? &gfull[st] : &full[st], land_par, a.err, abort_flag);
           uint8_t* vr = sKV + st * kStage + kTile + t * 128;
 #pragma unroll
           for (int c = 0; c < 8; ++c) {
-            reinterpret_cast<uint4*>(vr)[c] = make_uint4(0, 0, 0, 0);
+            if (!valid[0]) reinterpret_cast<uint4*>(vr)[c] = make_uint4(0, 0, 0, 0);
             reinterpret_cast<uint4*>(vr + kBox)[c] = make_uint4(0, 0, 0, 0);
           }
         }
-        // P^T row t -> column t of the K-major [16 heads][128 keys] buffer
-        uint8_t* pb = sP + x * kOpBuf + (t >> 6) * (kN * 128) + (t & 7) * 2;
+        // P^T row t -> column t of the K-major [NPV][128 rows] buffer
+        uint8_t* pb = sP + (it % C::NPB) * C::PBUF + (t >> 6) * (C::NPV * 128) + (t & 7) * 2;
         const int j = (t & 63) >> 3;
 #pragma unroll
-        for (int h = 0; h < G; ++h)
-          *reinterpret_cast<bf16*>(pb + h * 128 + ((j ^ (h & 7)) << 4)) = __float2bfloat16_rn(pr[h]);
+        for (int y = 0; y < NK; ++y)
+#pragma unroll
+          for (int h = 0; h < G; ++h) {
+            float rest = pr[y][h];
+#pragma unroll
+            for (int q = 0; q < C::PARTS; ++q) {
+              const int n = q * C::NP + y * C::HP + h;
+              const bf16 part = __float2bfloat16_rn(rest);
+              *reinterpret_cast<bf16*>(pb + n * 128 + ((j ^ (n & 7)) << 4)) = part;
+              rest -= __bfloat162float(part);
+            }
+          }
         fence_proxy_async_smem();
         tc_fence_before();
         __syncwarp();
@@ -729,12 +805,26 @@ __global__ void __launch_bounds__(kThreads + 32 * gather_warps(G, MODE), 1)
       const int last = it - 1;
       local_ok = wait_bar(&p_free[last & 1], (last >> 1) & 1, a.err, abort_flag) && local_ok;
       tc_fence_after();
-      uint32_t o[16];
-      tmem_ld16(tl + kOcol, o);
-      tmem_ld_wait();
+      uint32_t o[C::NP];
+      tmem_ld(tl + C::OCOL, o);
+      if constexpr (PAIR) {
+        uint32_t o1[C::NP], o2[C::NP];
+        tmem_ld(tl + C::OCOL + C::NP, o1);
+        tmem_ld(tl + C::OCOL + 2 * C::NP, o2);
+        tmem_ld_wait();
+#pragma unroll
+        for (int c = 0; c < C::NP; ++c)
+          o[c] = __float_as_uint(__uint_as_float(o[c]) + (__uint_as_float(o1[c]) + __uint_as_float(o2[c])));
+      } else {
+        tmem_ld_wait();
+      }
       tc_fence_before();
       __syncwarp();
       if (lane == 0) mbar_arrive(o_free);
+      if (PAIR && t >= 64) {
+#pragma unroll
+        for (int h = 0; h < G; ++h) ms[h * 64 + t - 64] = __uint_as_float(o[NK * C::HP - C::HP + h]);
+      }
 #pragma unroll
       for (int h = 0; h < G; ++h) {
         float v = l[h];
@@ -744,21 +834,27 @@ __global__ void __launch_bounds__(kThreads + 32 * gather_warps(G, MODE), 1)
       }
       ok = named_barrier_and(1, kSoftmaxThreads, local_ok);
       if (!ok) break;
+      if (PAIR && t < 64) {
+#pragma unroll
+        for (int h = 0; h < G; ++h) o[h] = __float_as_uint(__uint_as_float(o[h]) + ms[h * 64 + t]);
+      }
+      const bool row_d = t < D;  // this thread holds row d = t of the result
       float L[G];
 #pragma unroll
       for (int h = 0; h < G; ++h) L[h] = (lsum[h] + lsum[16 + h]) + (lsum[32 + h] + lsum[48 + h]);
 
       if constexpr (CLUSTER) {
-        dec::cluster_push<G, kD>(recv, o, m, L);
+        dec::cluster_push<G, D>(recv, o, m, L);
       } else {
         const long long row_off = walk.item_off + walk.sp.cost;  // unit of the item's row 0
         const int f = dec::cta_of(row_off, total, P);
         const int lst = dec::cta_of(row_off + (long long)(walk.sp.rows - 1) * walk.sp.w, total, P);
-        bf16* outp = static_cast<bf16*>(a.out) + ((size_t)b * g.Hq + (size_t)kvh * G) * kD;
+        bf16* outp = static_cast<bf16*>(a.out) + ((size_t)b * g.Hq + (size_t)kvh * G) * D;
         float2* st = (a.scores != nullptr && !strm) ? a.score_stats + (size_t)(b * g.n_r + k) * G : nullptr;
         if (f == lst) {
 #pragma unroll
-          for (int h = 0; h < G; ++h) outp[h * kD + t] = __float2bfloat16_rn(__uint_as_float(o[h]) / L[h]);
+          for (int h = 0; h < G; ++h)
+            if (row_d) outp[h * D + t] = __float2bfloat16_rn(__uint_as_float(o[h]) / L[h]);
           if (st != nullptr && t < G) {
             float mt = m[0], lt = L[0];
 #pragma unroll
@@ -769,9 +865,10 @@ __global__ void __launch_bounds__(kThreads + 32 * gather_warps(G, MODE), 1)
             st[t] = make_float2(mt, lt);
           }
         } else {
-          float* pbase = dec::partial_slot(a, p, p == f ? 1 : 0, G, kD);
+          float* pbase = dec::partial_slot(a, p, p == f ? 1 : 0, G, D);
 #pragma unroll
-          for (int h = 0; h < G; ++h) __stcg(pbase + h * kD + t, __uint_as_float(o[h]));
+          for (int h = 0; h < G; ++h)
+            if (row_d) __stcg(pbase + h * D + t, __uint_as_float(o[h]));
           float mt = m[0], lt = L[0];
 #pragma unroll
           for (int h = 1; h < G; ++h) {
@@ -779,10 +876,10 @@ __global__ void __launch_bounds__(kThreads + 32 * gather_warps(G, MODE), 1)
             lt = (t == h) ? L[h] : lt;
           }
           if (t < G) {
-            __stcg(pbase + G * kD + t, mt);
-            __stcg(pbase + G * kD + G + t, lt);
+            __stcg(pbase + G * D + t, mt);
+            __stcg(pbase + G * D + G + t, lt);
           }
-          dec::merge_item<G, kD, kSoftmaxThreads, true>(a, p, f, lst, id, outp, ms, sh32 + 1, st);
+          dec::merge_item<G, D, kSoftmaxThreads, true>(a, p, f, lst, id, outp, ms, sh32 + 1, st);
         }
         named_barrier_sync(1, kSoftmaxThreads);
       }
@@ -799,27 +896,27 @@ __global__ void __launch_bounds__(kThreads + 32 * gather_warps(G, MODE), 1)
       const int b = first_id / HK, k = first_id - b * HK;
       const bool strm = k >= g.n_r;
       const int kvh = strm ? g.s_head[k - g.n_r] : g.r_head[k];
-      bf16* outp = static_cast<bf16*>(a.out) + ((size_t)b * g.Hq + (size_t)kvh * G) * kD;
+      bf16* outp = static_cast<bf16*>(a.out) + ((size_t)b * g.Hq + (size_t)kvh * G) * D;
       float2* st = (a.scores != nullptr && !strm) ? a.score_stats + (size_t)(b * g.n_r + k) * G : nullptr;
-      dec::cluster_finish<G, kD, kSoftmaxThreads>(a, recv, sh32, outp, st);
+      dec::cluster_finish<G, D, kSoftmaxThreads>(a, recv, sh32, outp, st);
     }
   }
   __syncthreads();
   tc_fence_after();
-  if (warp == 5) tmem_dealloc(tmem, kTmemCols);
+  if (warp == 5) tmem_dealloc(tmem, C::TMEM_COLS);
   if constexpr (!CLUSTER)
     if (threadIdx.x == 0) dec::finish_launch(a, ls);
 }
 
 // `cluster`: CTAs per cluster (kCluster; it divides a.n_ctas).
-template <int G, int MODE>
+template <int D, int G, int MODE>
 cudaError_t launch_g(const DecodeArgs& a, int cluster, cudaStream_t s) {
   static bool attr_set = false;
   if (!attr_set) {
     cudaError_t e =
-        cudaFuncSetAttribute(decode_tc_kernel<G, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM);
+        cudaFuncSetAttribute(decode_tc_kernel<D, G, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, Lay<D, G>::SMEM);
     if (e == cudaSuccess && MODE == kCluster)
-      e = cudaFuncSetAttribute(decode_tc_kernel<G, MODE>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+      e = cudaFuncSetAttribute(decode_tc_kernel<D, G, MODE>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
     if (e != cudaSuccess) return e;
     attr_set = true;
   }
@@ -828,7 +925,7 @@ cudaError_t launch_g(const DecodeArgs& a, int cluster, cudaStream_t s) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(a.n_ctas);
   cfg.blockDim = dim3(kThreads + 32 * gather_warps(G, MODE));
-  cfg.dynamicSmemBytes = SMEM;
+  cfg.dynamicSmemBytes = Lay<D, G>::SMEM;
   cfg.stream = s;
   cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -841,21 +938,25 @@ cudaError_t launch_g(const DecodeArgs& a, int cluster, cudaStream_t s) {
     attr[1].val.clusterDim.y = attr[1].val.clusterDim.z = 1;
     cfg.numAttrs = 2;
   }
-  return cudaLaunchKernelEx(&cfg, decode_tc_kernel<G, MODE>, a);
+  return cudaLaunchKernelEx(&cfg, decode_tc_kernel<D, G, MODE>, a);
 }
 
-template <int MODE>
+template <int D, int MODE>
 cudaError_t launch_mode(const DecodeArgs& a, int cluster, cudaStream_t s) {
   switch (a.geom.G) {
-    case 1: return launch_g<1, MODE>(a, cluster, s);
-    case 2: return launch_g<2, MODE>(a, cluster, s);
-    case 3: return launch_g<3, MODE>(a, cluster, s);
-    case 4: return launch_g<4, MODE>(a, cluster, s);
-    case 5: return launch_g<5, MODE>(a, cluster, s);
-    case 6: return launch_g<6, MODE>(a, cluster, s);
-    case 7: return launch_g<7, MODE>(a, cluster, s);
-    case 8: return launch_g<8, MODE>(a, cluster, s);
-    case 16: return launch_g<16, MODE>(a, cluster, s);
+    case 1: return launch_g<D, 1, MODE>(a, cluster, s);
+    case 2: return launch_g<D, 2, MODE>(a, cluster, s);
+    case 4: return launch_g<D, 4, MODE>(a, cluster, s);
+    case 7: return launch_g<D, 7, MODE>(a, cluster, s);
+    case 8: return launch_g<D, 8, MODE>(a, cluster, s);
+  }
+  if constexpr (D == 128) {
+    switch (a.geom.G) {
+      case 3: return launch_g<D, 3, MODE>(a, cluster, s);
+      case 5: return launch_g<D, 5, MODE>(a, cluster, s);
+      case 6: return launch_g<D, 6, MODE>(a, cluster, s);
+      case 16: return launch_g<D, 16, MODE>(a, cluster, s);
+    }
   }
   return cudaErrorInvalidValue;
 }

@@ -6,7 +6,7 @@
 namespace aoh {
 
 cudaError_t launch_decode_tc_cluster(const DecodeArgs& a, int cluster, cudaStream_t s) {
-  return dtc::launch_mode<dtc::kCluster>(a, cluster, s);
+  return dtc::launch_mode<128, dtc::kCluster>(a, cluster, s);
 }
 
 // Clusters of `size` CTAs (one an SM) that the current device runs at once.
@@ -19,18 +19,19 @@ int decode_tc_max_clusters(int size) {
   std::lock_guard<std::mutex> lock(mu);
   int& n = known[dev][size];
   if (n == 0) {
-    auto kernel = dtc::decode_tc_kernel<1, dtc::kCluster>;
+    constexpr int smem = dtc::Lay<128, 1>::SMEM;
+    auto kernel = dtc::decode_tc_kernel<128, 1, dtc::kCluster>;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(size * 64);
     cfg.blockDim = dim3(dtc::kThreads);
-    cfg.dynamicSmemBytes = dtc::SMEM;
+    cfg.dynamicSmemBytes = smem;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeClusterDimension;
     attr[0].val.clusterDim.x = size;
     attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, dtc::SMEM) != cudaSuccess ||
+    if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess ||
         cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess ||
         cudaOccupancyMaxActiveClusters(&n, kernel, &cfg) != cudaSuccess) {
       cudaGetLastError();

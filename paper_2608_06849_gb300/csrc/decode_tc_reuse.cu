@@ -4,6 +4,6 @@
 
 namespace aoh {
 
-cudaError_t launch_decode_tc_reuse(const DecodeArgs& a, cudaStream_t s) { return dtc::launch_mode<dtc::kGather>(a, 1, s); }
+cudaError_t launch_decode_tc_reuse(const DecodeArgs& a, cudaStream_t s) { return dtc::launch_mode<128, dtc::kGather>(a, 1, s); }
 
 }  // namespace aoh

@@ -49,7 +49,9 @@ struct CacheGeom {
 };
 
 struct DecodeArgs {
-  CUtensorMap tcr, tcs;  // cache regions (see PrefillTcArgs); read by the tcgen05 kernel
+  // cache regions, read by the tcgen05 kernel: as in PrefillTcArgs at d_head
+  // 128; at d_head 64 the even rows, and the odd rows in maps of their own
+  CUtensorMap tcr, tcs, tcr_odd, tcs_odd;
   CacheGeom geom;
   const void* q;      // [B][Hq][D]
   const void* k_new;  // [B][Hkv][D]
@@ -63,6 +65,7 @@ struct DecodeArgs {
   uint32_t* gcounters;  // [n_ctas][2] part arrivals per group (indexed by the group's first CTA)
   uint32_t* done;     // CTAs finished in this launch
   uint32_t* err;      // error word
+  int row_keys = 1;   // cache rows per row of the split (2: the tcgen05 kernel at d_head 64)
   int n_ctas;         // CTAs sharing the rows of all items equally
   // nonzero: the launch's last CTA also leaves the error word and every
   // counter at zero after a timed-out launch, so the next launch needs no
@@ -150,10 +153,12 @@ bool prefill_tc_make_cache_maps(PrefillTcArgs* a, const void* kv);
 // [regions][K, V][capacity rows][D] with box [1][1][128][64] and 128-byte
 // swizzle; a kind with no heads leaves its map untouched.
 bool make_cache_region_maps(CUtensorMap* tcr, CUtensorMap* tcs, const CacheGeom& g, const void* kv);
+// The maps of a decode step on the tcgen05 kernel (DecodeArgs); at d_head 64
+// box [1][1][128][64] over every second row.
+bool make_decode_maps(DecodeArgs* a, const CacheGeom& g, const void* kv);
 cudaError_t launch_prefill_tc(const PrefillTcArgs& a, int n_items, cudaStream_t s);
-cudaError_t launch_decode(const DecodeArgs& a, cudaStream_t s);
-// The CUDA-core decode kernel for any supported (D, G) (the H2Share reuse
-// step takes this path at d_head 128 too), with its CTA count.
+// The CUDA-core decode kernel: the H2Share reuse step of d_head 64, with its
+// CTA count.
 cudaError_t launch_decode_cc(const DecodeArgs& a, cudaStream_t s);
 int decode_cc_ctas(long long total_rows, int num_sms);
 bool decode_cc_supported(int D, int G);
@@ -169,7 +174,9 @@ void h2_decode_outputs(float* ws, int B, int n_r, int G, int max_seq, float** sc
 // lengths after the anchor step's append.
 cudaError_t launch_h2_topk(float* ws, int max_seq, const int32_t* lens, int B, int n_r, int G, int top_k,
                            int32_t* idx_out, cudaStream_t s);
-// The tcgen05 decode kernel serves (D, G) (else the CUDA-core kernel does).
+// The tcgen05 decode kernel serves plain steps of (D, G).
+bool decode_on_tc(int D, int G);
+// It serves every kind of step, the H2Share ones included (d_head 128).
 bool decode_uses_tc(int D, int G);
 // Work units of a gathered row and of a contiguous row in the reuse step's
 // split on the tcgen05 kernel (a borrowed K and V row copied by the gather
@@ -184,6 +191,7 @@ void reuse_tc_weights(int G, int* gather_w, int* ring_w);
 int decode_tc_item_cost(long long total_rows, int n_ctas, int num_sms);
 int decode_tc_ctas(long long total_rows, int num_sms);
 cudaError_t launch_decode_tc(const DecodeArgs& a, cudaStream_t s);
+cudaError_t launch_decode_tc64(const DecodeArgs& a, cudaStream_t s);
 cudaError_t launch_decode_tc_reuse(const DecodeArgs& a, cudaStream_t s);
 // Clusters of `size` CTAs of the tcgen05 decode kernel that the current device
 // runs at once.

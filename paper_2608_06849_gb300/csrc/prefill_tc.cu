@@ -551,11 +551,15 @@ bool prefill_tc_make_maps(PrefillTcArgs* a, const void* q, const void* k, const 
 
 // 4D map over one kind of cache region: [regions][K, V][cap rows][D], box
 // [1][1][128][64], 128-byte swizzle. Rows past `cap` read as zeros.
-static bool make_region_map(CUtensorMap* map, const void* base, int regions, int cap, int D) {
+// With `step` 2 the map holds every second of the cap rows, `base` being the
+// first of them and `rows` their number.
+static bool make_region_map(CUtensorMap* map, const void* base, int regions, int cap, int D, int step = 1,
+                            int rows = 0) {
   auto fn = encode_fn();
   if (!fn) return false;
-  cuuint64_t dims[4] = {(cuuint64_t)D, (cuuint64_t)cap, 2, (cuuint64_t)regions};
-  cuuint64_t strides[3] = {(cuuint64_t)D * 2, (cuuint64_t)cap * D * 2, (cuuint64_t)cap * D * 2 * 2};
+  if (step == 1) rows = cap;
+  cuuint64_t dims[4] = {(cuuint64_t)D, (cuuint64_t)rows, 2, (cuuint64_t)regions};
+  cuuint64_t strides[3] = {(cuuint64_t)D * 2 * step, (cuuint64_t)cap * D * 2, (cuuint64_t)cap * D * 2 * 2};
   cuuint32_t box[4] = {64, 128, 1, 1};
   cuuint32_t estr[4] = {1, 1, 1, 1};
   CUresult r = fn(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void*>(base), dims, strides, box, estr,
@@ -569,6 +573,24 @@ bool make_cache_region_maps(CUtensorMap* tcr, CUtensorMap* tcs, const CacheGeom&
   bool ok = true;
   if (g.n_r > 0) ok = ok && make_region_map(tcr, base + g.r_region(0, 0), g.B * g.n_r, g.max_seq, g.D);
   if (g.n_s > 0) ok = ok && make_region_map(tcs, base + g.s_region(0, 0), g.B * g.n_s, g.S + g.W, g.D);
+  return ok;
+}
+
+bool make_decode_maps(DecodeArgs* a, const CacheGeom& g, const void* kv) {
+  if (g.D != 64) return make_cache_region_maps(&a->tcr, &a->tcs, g, kv);
+  const bf16* base = static_cast<const bf16*>(kv);
+  bool ok = true;
+  for (int odd = 0; odd < 2; ++odd) {
+    auto pair_map = [&](CUtensorMap* map, const bf16* first, int regions, int cap) {
+      // a region of one row has no odd row: its map repeats the even one
+      const int shift = odd && cap > 1 ? g.D : 0;
+      return make_region_map(map, first + shift, regions, cap, g.D, 2, odd && cap > 1 ? cap / 2 : (cap + 1) / 2);
+    };
+    if (g.n_r > 0)
+      ok = ok && pair_map(odd ? &a->tcr_odd : &a->tcr, base + g.r_region(0, 0), g.B * g.n_r, g.max_seq);
+    if (g.n_s > 0)
+      ok = ok && pair_map(odd ? &a->tcs_odd : &a->tcs, base + g.s_region(0, 0), g.B * g.n_s, g.S + g.W);
+  }
   return ok;
 }
 

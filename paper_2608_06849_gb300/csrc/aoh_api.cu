@@ -94,6 +94,18 @@ std::vector<int4> prefill_schedule(const CacheGeom& g, const std::vector<int32_t
   return items;
 }
 
+// Whether clusters of two CTAs halve each item's KV tiles: when every item's
+// cluster runs at once, the call lasts as long as its longest item.
+// Measured (8 heads of 128, one sequence, us of the kernel without / with):
+// 256 rows (2 tiles) 11.2 / 11.5, 384 11.8 / 13.4, 512 15.4 / 13.5, 1024 21.1 /
+// 17.5, 2048 34.8 / 24.4; heads of 64: 384 11.4 / 11.6, 512 13.9 / 11.7, 2048
+// 30.8 / 21.1. In more waves it does not pay: 4K rows after a long prefix (448
+// items) took 2% longer, the exchange of the states and the second start of a
+// pipeline costing more than the fuller last wave gives.
+bool prefill_split(const std::vector<int4>& items, int num_sms) {
+  return (int)items.size() <= num_sms / 2 && items[0].w >= 4;
+}
+
 size_t bytes_for(const aoh_config& c, int n_r, int n_s) {
   const size_t tokens = (size_t)n_r * c.max_seq + (size_t)n_s * (size_t)(c.sink + c.window);
   return (size_t)c.batch * tokens * c.d_head * 2 * 2;
@@ -404,7 +416,7 @@ aoh_status aoh_prefill(const void* q, const void* k, const void* v, int32_t T, c
       return fail(AOH_ERR_CUDA, "cuTensorMapEncodeTiled failed for q/k/v");
     if (chunked && !prefill_tc_make_cache_maps(&pa, cache->kv))
       return fail(AOH_ERR_CUDA, "cuTensorMapEncodeTiled failed for the cache");
-    e = launch_prefill_tc(pa, (int)items.size(), s);
+    e = launch_prefill_tc(pa, (int)items.size(), prefill_split(items, cache->num_sms), s);
     if (e != cudaSuccess) return cuda_fail(e, "prefill kernel launch");
   }
 

@@ -156,7 +156,8 @@ bool make_cache_region_maps(CUtensorMap* tcr, CUtensorMap* tcs, const CacheGeom&
 // The maps of a decode step on the tcgen05 kernel (DecodeArgs); at d_head 64
 // box [1][1][128][64] over every second row.
 bool make_decode_maps(DecodeArgs* a, const CacheGeom& g, const void* kv);
-cudaError_t launch_prefill_tc(const PrefillTcArgs& a, int n_items, cudaStream_t s);
+// One CTA a work item, or a cluster of two that halve its KV tiles (`split`).
+cudaError_t launch_prefill_tc(const PrefillTcArgs& a, int n_items, bool split, cudaStream_t s);
 // The CUDA-core decode kernel: the H2Share reuse step of d_head 64, with its
 // CTA count.
 cudaError_t launch_decode_cc(const DecodeArgs& a, cudaStream_t s);

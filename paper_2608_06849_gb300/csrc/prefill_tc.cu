@@ -39,6 +39,7 @@
 // O_B [256+D, 256+2D).
 #include <math.h>
 
+#include "cluster.cuh"
 #include "common.cuh"
 #include "internal.h"
 #include "tc.cuh"
@@ -69,6 +70,7 @@ struct PfCfg {
   static constexpr uint32_t IDESC_PV = idesc_bf16(kBM, D, true);
   static_assert(SMEM <= 232448, "shared memory");
   static_assert(256 + 2 * D <= (int)kTmemCols, "TMEM columns");
+  static_assert(128 * (D * 4 + 8) <= OFF_BAR, "receive buffer of the split");
 };
 
 // Bits lo..hi-1 of a 32-bit word (lo, hi clamped to [0, 32]).
@@ -80,7 +82,11 @@ __device__ __forceinline__ uint32_t range_bits(int lo, int hi) {
   return top & ~((1u << lo) - 1u);
 }
 
-template <int D>
+// SPLIT: a cluster of two CTAs shares one work item. Each visits half of its KV
+// tiles; then each finishes one of the two query tiles: it receives the other
+// CTA's state of that tile (O, running max and sum) in shared memory that the
+// main loop no longer needs, adds its own and writes the rows.
+template <int D, bool SPLIT>
 __global__ void __launch_bounds__(kThreads, 1) prefill_tc_kernel(const __grid_constant__ PrefillTcArgs a) {
   using C = PfCfg<D>;
   extern __shared__ uint8_t smem_raw[];
@@ -104,7 +110,7 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_tc_kernel(const __grid_co
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int4 item = a.work[blockIdx.x];
+  const int4 item = a.work[SPLIT ? blockIdx.x >> 1 : blockIdx.x];
   const int b = item.x, h = item.y, q0 = item.z;
   const CacheGeom& g = a.geom;
   const int kvh = h / g.G;
@@ -124,10 +130,15 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_tc_kernel(const __grid_co
     c_begin = max(a_end, max(0, g.wstart(q0)) / kBN);
     c_end = max(c_begin, (q_end + kBN - 1) / kBN);
   }
-  const int n_tiles = n_c + a_end + (c_end - c_begin);
+  const int n_all = n_c + a_end + (c_end - c_begin);
+  // this CTA visits tiles t0 .. t0 + n_tiles - 1 of the item's n_all
+  const int rank = SPLIT ? (int)cluster_rank() : 0;
+  const int t0 = rank * ((n_all + 1) / 2);
+  const int n_tiles = !SPLIT ? n_all : rank == 0 ? (n_all + 1) / 2 : n_all / 2;
   // keys of KV tile jj that hold data (the rest: cache rows not yet written,
   // or chunk padding); fewer than kBN makes the tile partial
-  auto tile_valid = [&](int jj) {
+  auto tile_valid = [&](int i) {
+    const int jj = t0 + i;
     if (jj < n_c) return (streaming ? min(Lb, g.S + g.W) : Lb) - jj * kBN;
     const int jc = jj - n_c;
     return len - (jc < a_end ? jc : c_begin + (jc - a_end)) * kBN;
@@ -160,6 +171,9 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_tc_kernel(const __grid_co
   tc_fence_after();
   const uint32_t tmem = *tmem_slot;
 
+  // SPLIT: a row's final softmax state (softmax warps)
+  float end_m = -INFINITY, end_l = 0.f;
+  bool end_ok = true;
   if (warp == 0) {
     // ------------------------------------------------------------ producer
     // Lane 0 issues the copies. Rows of a V tile past its valid keys may hold
@@ -179,7 +193,7 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_tc_kernel(const __grid_co
     int issued = 0, n_partial = 0;
     bool ok = true;
     for (int jj = 0; jj < n_tiles && ok; ++jj) {
-      const int jc = jj - n_c;
+      const int ja = t0 + jj, jc = ja - n_c;
       const int j = jc < a_end ? jc : c_begin + (jc - a_end);
       for (int sel = 0; sel < 2; ++sel) {
         const int it = 2 * jj + sel;
@@ -189,12 +203,12 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_tc_kernel(const __grid_co
             ok = false;
           } else {
             mbar_arrive_expect_tx(&kv_full[st], C::KVBYTES);
-            if (jj < n_c) {
+            if (ja < n_c) {
               // cache region viewed as [regions][K, V][rows][D]
               const CUtensorMap* map = streaming ? &a.tcs : &a.tcr;
               const int region = streaming ? b * g.n_s + g.idx[kvh] : b * g.n_r + g.idx[kvh];
               for (int db = 0; db < C::DBLK; ++db)
-                tma_load_4d(sKV + st * C::KVBYTES + db * C::BOX, map, db * 64, jj * kBN, sel, region,
+                tma_load_4d(sKV + st * C::KVBYTES + db * C::BOX, map, db * 64, ja * kBN, sel, region,
                             &kv_full[st]);
             } else {
               const CUtensorMap* map = sel ? &a.tv : &a.tk;
@@ -267,7 +281,7 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_tc_kernel(const __grid_co
         }
         return true;
       };
-      bool ok = wait_bar(q_full, 0, a.err, abort_flag) && wait_k(0);
+      bool ok = n_tiles > 0 && wait_bar(q_full, 0, a.err, abort_flag) && wait_k(0);
       if (ok) {
         tc_fence_after();
         issue_s(0, 0);
@@ -313,8 +327,8 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_tc_kernel(const __grid_co
     float m = -INFINITY, l = 0.f;
     bool ok = true;
     for (int jj = 0; jj < n_tiles; ++jj) {
-      const int jc = jj - n_c;
-      const int j = jj < n_c ? jj : (jc < a_end ? jc : c_begin + (jc - a_end));
+      const int ja = t0 + jj, jc = ja - n_c;
+      const int j = ja < n_c ? ja : (jc < a_end ? jc : c_begin + (jc - a_end));
       const int j0 = j * kBN;
       if (!__all_sync(0xffffffffu, wait_bar(&s_full[x], jj & 1, a.err, abort_flag))) {
         ok = false;
@@ -350,7 +364,7 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_tc_kernel(const __grid_co
       // an immediate and one select.
       bool need_mask;
       int e_hi = kBN, a0 = 0, a1 = 0, b0 = 0, b1 = 0;
-      if (jj < n_c) {
+      if (ja < n_c) {
         if (!streaming) {
           need_mask = j0 + kBN > Lb;
           e_hi = Lb - j0;
@@ -467,7 +481,12 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_tc_kernel(const __grid_co
       __syncwarp();
       if (lane == 0) mbar_arrive(&p_full[x]);
     }
-    if (ok && __all_sync(0xffffffffu, wait_bar(&pv_done[x], (n_tiles - 1) & 1, a.err, abort_flag))) {
+    if constexpr (SPLIT) {
+      end_m = m;
+      end_l = l;
+      end_ok = ok && (n_tiles == 0 ||
+                      __all_sync(0xffffffffu, wait_bar(&pv_done[x], (n_tiles - 1) & 1, a.err, abort_flag)));
+    } else if (ok && __all_sync(0xffffffffu, wait_bar(&pv_done[x], (n_tiles - 1) & 1, a.err, abort_flag))) {
       tc_fence_after();
       const float inv = 1.f / l;
       bf16* op = static_cast<bf16*>(a.out) + (((size_t)b * a.T + min(i, len - 1)) * g.Hq + h) * D;
@@ -494,6 +513,72 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_tc_kernel(const __grid_co
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
+  if constexpr (SPLIT) {
+    // both CTAs' copies and MMAs are done with their shared memory
+    cluster_arrive();
+    cluster_wait();
+    const int x = (warp - 2) >> 2, q4 = warp & 3, r = q4 * 32 + lane;
+    const uint32_t tl = tmem + ((uint32_t)(q4 * 32) << 16) + 256 + x * D;
+    float4* recv = reinterpret_cast<float4*>(smem);  // [D / 4][128 rows], then (m, l) per row
+    float2* recv_ml = reinterpret_cast<float2*>(recv + D / 4 * 128);
+    if (warp >= 2 && x != rank) {
+      const uint32_t dst = cluster_addr(recv + r, (uint32_t)(rank ^ 1));
+      cluster_st2(cluster_addr(recv_ml + r, (uint32_t)(rank ^ 1)), __float_as_uint(end_m), __float_as_uint(end_l));
+      if (n_tiles > 0) {
+#pragma unroll
+        for (int c = 0; c < D / 32; ++c) {
+          uint32_t v[32];
+          tmem_ld32(tl + c * 32, v);
+          tmem_ld_wait();
+#pragma unroll
+          for (int e = 0; e < 32; e += 4)
+            cluster_st4(dst + (uint32_t)((c * 8 + e / 4) * 128 * 16), v[e], v[e + 1], v[e + 2], v[e + 3]);
+        }
+      }
+      tc_fence_before();
+    }
+    cluster_arrive();
+    cluster_wait();
+    if (warp >= 2 && x == rank && end_ok) {
+      const int i = q0 + x * kBM + r;
+      const float2 o_ml = recv_ml[r];
+      const float M = fmaxf(end_m, o_ml.x);
+      // the other CTA may have had no tile (-inf and unwritten values)
+      const float w0 = end_m == -INFINITY ? 0.f : fast_exp2(end_m - M),
+                  w1 = o_ml.x == -INFINITY ? 0.f : fast_exp2(o_ml.x - M);
+      const float inv = 1.f / (end_l * w0 + o_ml.y * w1);
+      const float f0 = w0 * inv, f1 = w1 * inv;
+      bf16* op = static_cast<bf16*>(a.out) + (((size_t)b * a.T + min(i, len - 1)) * g.Hq + h) * D;
+#pragma unroll
+      for (int c = 0; c < D / 32; ++c) {
+        uint32_t v[32];
+        tmem_ld32(tl + c * 32, v);
+        tmem_ld_wait();
+#pragma unroll
+        for (int e = 0; e < 32; e += 8) {
+          float y[8];
+#pragma unroll
+          for (int k = 0; k < 8; k += 4) {
+            const float4 z = recv[(c * 8 + (e + k) / 4) * 128 + r];
+            // a weight of 0 must not meet values that were never written
+            y[k + 0] = (w0 == 0.f ? 0.f : __uint_as_float(v[e + k + 0]) * f0) + (w1 == 0.f ? 0.f : z.x * f1);
+            y[k + 1] = (w0 == 0.f ? 0.f : __uint_as_float(v[e + k + 1]) * f0) + (w1 == 0.f ? 0.f : z.y * f1);
+            y[k + 2] = (w0 == 0.f ? 0.f : __uint_as_float(v[e + k + 2]) * f0) + (w1 == 0.f ? 0.f : z.z * f1);
+            y[k + 3] = (w0 == 0.f ? 0.f : __uint_as_float(v[e + k + 3]) * f0) + (w1 == 0.f ? 0.f : z.w * f1);
+          }
+          uint4 w;
+          w.x = float2_to_bf16x2(y[0], y[1]);
+          w.y = float2_to_bf16x2(y[2], y[3]);
+          w.z = float2_to_bf16x2(y[4], y[5]);
+          w.w = float2_to_bf16x2(y[6], y[7]);
+          if (i < len) *reinterpret_cast<uint4*>(op + c * 32 + e) = w;
+        }
+      }
+      tc_fence_before();
+    }
+    __syncthreads();
+    tc_fence_after();
+  }
   if (warp == 1) tmem_dealloc(tmem, kTmemCols);
 }
 
@@ -528,17 +613,28 @@ bool make_map(CUtensorMap* map, const void* base, int B, int T, int H, int D) {
   return r == CUDA_SUCCESS;
 }
 
-template <int D>
+template <int D, bool SPLIT>
 cudaError_t launch_cfg(const PrefillTcArgs& a, int n_items, cudaStream_t s) {
   using C = PfCfg<D>;
   static bool attr_set = false;
   if (!attr_set) {
-    cudaError_t e = cudaFuncSetAttribute(prefill_tc_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM);
+    cudaError_t e =
+        cudaFuncSetAttribute(prefill_tc_kernel<D, SPLIT>, cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM);
     if (e != cudaSuccess) return e;
     attr_set = true;
   }
-  prefill_tc_kernel<D><<<n_items, kThreads, C::SMEM, s>>>(a);
-  return cudaGetLastError();
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(SPLIT ? 2 * n_items : n_items);
+  cfg.blockDim = dim3(kThreads);
+  cfg.dynamicSmemBytes = C::SMEM;
+  cfg.stream = s;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = 2;
+  attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = SPLIT ? 1 : 0;
+  return cudaLaunchKernelEx(&cfg, prefill_tc_kernel<D, SPLIT>, a);
 }
 
 }  // namespace
@@ -598,10 +694,10 @@ bool prefill_tc_make_cache_maps(PrefillTcArgs* a, const void* kv) {
   return make_cache_region_maps(&a->tcr, &a->tcs, a->geom, kv);
 }
 
-cudaError_t launch_prefill_tc(const PrefillTcArgs& a, int n_items, cudaStream_t s) {
+cudaError_t launch_prefill_tc(const PrefillTcArgs& a, int n_items, bool split, cudaStream_t s) {
   if (n_items <= 0) return cudaSuccess;
-  if (a.geom.D == 128) return launch_cfg<128>(a, n_items, s);
-  if (a.geom.D == 64) return launch_cfg<64>(a, n_items, s);
+  if (a.geom.D == 128) return split ? launch_cfg<128, true>(a, n_items, s) : launch_cfg<128, false>(a, n_items, s);
+  if (a.geom.D == 64) return split ? launch_cfg<64, true>(a, n_items, s) : launch_cfg<64, false>(a, n_items, s);
   return cudaErrorInvalidValue;
 }
 

@@ -1,0 +1,50 @@
+"""Prefill calls small enough that clusters of two CTAs share each work item,
+around the rule's edges (four visited tiles, 76 items), against the oracle: odd
+lengths, a cached prefix, streaming heads whose halves see no key of some rows,
+the chunk-eviction rule."""
+
+import numpy as np
+import pytest
+import torch
+
+from gpu_cases import assert_matches, ensure_lib, f64, run_case
+from oracle import attention as oatt
+from paper_2608_06849_gb300 import aoh
+from paper_2608_06849_gb300.workloads import randn_bf16
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("B,Hq,Hkv,d,T,S,W,labels,lens", [
+    (1, 8, 2, 128, 384, 4, 60, [0, 1], None),             # three tiles: not split
+    (1, 8, 2, 128, 385, 4, 60, [0, 1], None),             # four
+    (1, 8, 2, 64, 1025, 16, 100, [0, 1], None),           # a last item of one row
+    (2, 14, 2, 128, 700, 200, 130, [1, 0], [700, 513]),   # ragged, sinks past a tile
+    (1, 4, 4, 128, 2300, 0, 1, [1, 0, 1, 0], None),       # a window of one
+    (1, 32, 4, 64, 512, 4, 60, [0, 1, 0, 0], None),       # 64 items
+])
+def test_small_calls(B, Hq, Hkv, d, T, S, W, labels, lens):
+    run_case(B, Hq, Hkv, d, T, S, W, labels, seq_lens=lens)
+
+
+@pytest.mark.parametrize("d,rule", [(128, 0), (64, 0), (128, 300)])
+def test_after_a_cached_prefix(d, rule):
+    """A second chunk reads the first one's rows through the cache tiles."""
+    ensure_lib()
+    Hq, Hkv, S, W, labels, cut, T = 8, 2, 5, 130, [0, 1], 600, 1111
+    q, k, v = (randn_bf16((1, T, h, d), 40 + h, "cuda") for h in (Hq, Hkv, Hkv + 1))
+    v = v[:, :, :Hkv].contiguous()
+    cache = aoh.Cache(1, Hq, Hkv, d, T, S, W, labels, chunk=rule)
+    got = []
+    for a, b in ((0, cut), (cut, T)):
+        out = torch.full_like(q[:, a:b], float("nan")).contiguous()
+        cache.prefill(*(x[:, a:b].contiguous() for x in (q, k, v)), out)
+        got.append(f64(out[0]))
+    cache.check()
+    assert cache.lens() == [T]
+    qn, kn, vn = f64(q[0]), f64(k[0]), f64(v[0])
+    kw = {"chunk": rule} if rule else {}
+    want = oatt.prefill(qn, kn, vn, labels, S, W, **kw)
+    mag = oatt.prefill(qn, kn, np.abs(vn), labels, S, W, **kw)
+    assert_matches(np.concatenate(got), want, "two chunks", mag)
+    cache.close()

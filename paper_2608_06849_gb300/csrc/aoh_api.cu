@@ -390,8 +390,17 @@ aoh_status aoh_prefill(const void* q, const void* k, const void* v, int32_t T, c
       return fail(AOH_ERR_CAPACITY, "sequence %d would hold %d tokens; max_seq is %d", b, lens[b], g.max_seq);
   }
   cudaStream_t s = (cudaStream_t)stream;
-  cudaError_t e = cudaMemcpyAsync(cache->d_chunk, clen.data(), sizeof(int32_t) * g.B, cudaMemcpyHostToDevice, s);
-  if (e != cudaSuccess) return cuda_fail(e, "cudaMemcpyAsync(chunk lengths)");
+  cudaError_t e = cudaSuccess;
+  ChunkLens cl;
+  const bool by_value = g.B <= ChunkLens::kMost;
+  cl.lens = by_value ? nullptr : cache->d_chunk;
+  cl.base = by_value ? nullptr : cache->d_lens;
+  if (by_value) {
+    for (int b = 0; b < g.B; ++b) cl.by_value[b] = make_int2(clen[b], base[b]);
+  } else {
+    e = cudaMemcpyAsync(cache->d_chunk, clen.data(), sizeof(int32_t) * g.B, cudaMemcpyHostToDevice, s);
+    if (e != cudaSuccess) return cuda_fail(e, "cudaMemcpyAsync(chunk lengths)");
+  }
 
   // attention first: a chunk's own writes to a streaming ring would overwrite
   // positions its rows still read
@@ -406,8 +415,7 @@ aoh_status aoh_prefill(const void* q, const void* k, const void* v, int32_t T, c
     memset(&pa, 0, sizeof(pa));
     pa.geom = g;
     pa.out = out;
-    pa.lens = cache->d_chunk;
-    pa.base = cache->d_lens;
+    pa.chunk = cl;
     pa.work = cache->d_work;
     pa.err = cache->d_err;
     pa.T = T;
@@ -425,13 +433,16 @@ aoh_status aoh_prefill(const void* q, const void* k, const void* v, int32_t T, c
   ap.k = k;
   ap.v = v;
   ap.kv = cache->kv;
-  ap.lens = cache->d_chunk;
-  ap.base = cache->d_lens;
+  ap.chunk = cl;
+  ap.new_lens = by_value ? cache->d_lens : nullptr;
+  ap.after_prefill = by_value && out != nullptr;
   ap.T = T;
   e = launch_append(ap, s);
   if (e != cudaSuccess) return cuda_fail(e, "append kernel launch");
-  e = launch_lens_add(cache->d_lens, cache->d_chunk, g.B, s);
-  if (e != cudaSuccess) return cuda_fail(e, "length update launch");
+  if (!by_value) {
+    e = launch_lens_add(cache->d_lens, cache->d_chunk, g.B, s);
+    if (e != cudaSuccess) return cuda_fail(e, "length update launch");
+  }
   cache->lens = lens;
   return AOH_OK;
 }

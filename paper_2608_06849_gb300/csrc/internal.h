@@ -109,13 +109,28 @@ struct DecodeArgs {
   uint8_t idx_map[kMaxKvHeads] = {};
 };
 
+// Rows of the chunk and tokens cached before it, per sequence: by value up to
+// kMost sequences (no copy to the device precedes the launch), in device
+// arrays above.
+struct ChunkLens {
+  static constexpr int kMost = 64;
+  int2 by_value[kMost];  // {rows, tokens before}
+  const int32_t* lens;   // device [B], or null: by value
+  const int32_t* base;
+  __host__ __device__ int2 of(int b) const { return lens ? make_int2(lens[b], base[b]) : by_value[b]; }
+};
+
 struct AppendArgs {
   CacheGeom geom;
   const void* k;  // [B][T][Hkv][D]
   const void* v;
   void* kv;
-  const int32_t* lens;  // device [B]: rows of the chunk
-  const int32_t* base;  // device [B]: tokens cached before the chunk
+  ChunkLens chunk;
+  // device [B] lengths that the kernel sets to the new ones (chunk by value),
+  // or null
+  int32_t* new_lens;
+  // the prefill kernel precedes the launch, which may start under its tail
+  int after_prefill;
   int T;
 };
 
@@ -127,8 +142,7 @@ struct PrefillTcArgs {
   CUtensorMap tcr, tcs;    // cache: retrieval / streaming regions as [regions][K, V][rows][D]
   CacheGeom geom;
   void* out;            // [B][T][Hq][D]
-  const int32_t* lens;  // device [B]: rows of the chunk
-  const int32_t* base;  // device [B]: tokens cached before the chunk
+  ChunkLens chunk;
   const int4* work;     // {b, h, q0, cost}
   uint32_t* err;
   int T;

@@ -110,13 +110,15 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_tc_kernel(const __grid_co
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  // the append may start once the last CTAs of this grid run (append.cu)
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   const int4 item = a.work[SPLIT ? blockIdx.x >> 1 : blockIdx.x];
   const int b = item.x, h = item.y, q0 = item.z;
   const CacheGeom& g = a.geom;
   const int kvh = h / g.G;
   const bool streaming = g.kind[kvh] != 0;
-  const int len = a.lens[b];
-  const int Lb = a.base[b];
+  const int2 chunk = a.chunk.of(b);
+  const int len = chunk.x, Lb = chunk.y;
   const int q_end = min(q0 + 2 * kBM, len);
   const int S_rel = g.S - Lb;
   const int n_c = Lb == 0 ? 0 : ((streaming ? min(Lb, g.S + g.W) : Lb) + kBN - 1) / kBN;

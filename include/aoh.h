@@ -110,7 +110,7 @@ size_t aoh_cache_bytes(const aoh_config* cfg, const uint8_t* head_labels);
  * returns the offsets.
  * Allocates the handle's metadata block and a prefill work list sized for
  * chunks of up to max_seq tokens (B * n_q_heads * ceil(max_seq / 256)
- * entries of 16 bytes), and synchronises the device once (metadata upload).
+ * entries of 8 bytes), and synchronises the device once (metadata upload).
  * Errors: INVALID, CAPACITY, UNSUPPORTED, CUDA.
  */
 aoh_status aoh_cache_init(const aoh_config* cfg, const uint8_t* head_labels, void* kv_buffer,
@@ -135,8 +135,10 @@ aoh_status aoh_cache_init(const aoh_config* cfg, const uint8_t* head_labels, voi
  *             or past seq_lens[b] are ignored: their contents (even NaN) do
  *             not affect any output, and their outputs are not written.
  *   out  [B][T][n_q_heads][d_head], or NULL to only fill the cache.
- * With out, the host lists the call's query tiles (longest first) and uploads
- * the list to the handle's work list. A chunk of at most max_seq tokens (or
+ * With out, the host lists the call's query tiles (pairs of 128 rows of a query
+ * head, longest first). Up to 3840 of them travel as kernel arguments; a longer
+ * list is uploaded to the handle's work list, a copy from pageable memory, which
+ * waits for the stream's earlier work. A chunk of at most max_seq tokens (or
  * of at most the max_tokens given to aoh_cache_reserve) fits the list as
  * allocated; only a longer chunk, which a cache without retrieval heads can
  * take, grows it with cudaMalloc (which synchronises the device).

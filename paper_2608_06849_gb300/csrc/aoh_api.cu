@@ -62,19 +62,24 @@ aoh_status check_config(const aoh_config* cfg, const uint8_t* labels, int* n_r, 
   return AOH_OK;
 }
 
-// Prefill work: one item per (b, query head, 128-row query tile), with the
-// number of 128-key tiles it visits as its cost; heaviest first so the
-// hardware block scheduler fills the machine longest-processing-time first.
-std::vector<int4> prefill_schedule(const CacheGeom& g, const std::vector<int32_t>& base,
-                                   const std::vector<int32_t>& lens) {
+// Prefill work: one item per (b, query head, pair of 128-row query tiles),
+// heaviest first so the hardware block scheduler fills the machine
+// longest-processing-time first. The cost, the number of 128-key tiles visited,
+// is the same for all heads of a kind, so (b, pair, kind) entries are sorted and
+// then expanded into heads. *longest receives the first item's cost.
+std::vector<uint64_t> prefill_schedule(const CacheGeom& g, const std::vector<int32_t>& base,
+                                       const std::vector<int32_t>& lens, int* longest) {
   constexpr int BM = 256, BN = 128;
-  std::vector<int4> items;
+  struct Entry {
+    int cost, b, pair, streaming;
+  };
+  std::vector<Entry> entries;
   for (int b = 0; b < g.B; ++b) {
-    for (int h = 0; h < g.Hq; ++h) {
-      const bool streaming = g.kind[h / g.G] != 0;
-      const int Lb = base[b];
+    const int Lb = base[b];
+    const int S_rel = g.S - Lb;
+    for (int streaming = 0; streaming < 2; ++streaming) {
+      if ((streaming ? g.n_s : g.n_r) == 0) continue;
       const int n_c = Lb == 0 ? 0 : ((streaming ? std::min(Lb, g.S + g.W) : Lb) + BN - 1) / BN;
-      const int S_rel = g.S - Lb;
       for (int q0 = 0; q0 < lens[b]; q0 += BM) {
         const int q_end = std::min(q0 + BM, (int)lens[b]);
         int n;
@@ -86,11 +91,19 @@ std::vector<int4> prefill_schedule(const CacheGeom& g, const std::vector<int32_t
           const int c_end = std::max(c_begin, (q_end + BN - 1) / BN);
           n = a_end + (c_end - c_begin);
         }
-        items.push_back(make_int4(b, h, q0, n_c + n));
+        entries.push_back({n_c + n, b, q0 / BM, streaming});
       }
     }
   }
-  std::stable_sort(items.begin(), items.end(), [](const int4& x, const int4& y) { return x.w > y.w; });
+  std::stable_sort(entries.begin(), entries.end(), [](const Entry& x, const Entry& y) { return x.cost > y.cost; });
+  std::vector<uint64_t> items;
+  items.reserve(entries.size() * (size_t)g.Hq);
+  for (const Entry& e : entries)
+    for (int i = 0; i < (e.streaming ? g.n_s : g.n_r); ++i) {
+      const int kvh = e.streaming ? g.s_head[i] : g.r_head[i];
+      for (int h = kvh * g.G; h < (kvh + 1) * g.G; ++h) items.push_back(prefill_item(e.b, h, e.pair));
+    }
+  *longest = entries.empty() ? 0 : entries[0].cost;
   return items;
 }
 
@@ -102,9 +115,7 @@ std::vector<int4> prefill_schedule(const CacheGeom& g, const std::vector<int32_t
 // 30.8 / 21.1. In more waves it does not pay: 4K rows after a long prefix (448
 // items) took 2% longer, the exchange of the states and the second start of a
 // pipeline costing more than the fuller last wave gives.
-bool prefill_split(const std::vector<int4>& items, int num_sms) {
-  return (int)items.size() <= num_sms / 2 && items[0].w >= 4;
-}
+bool prefill_split(size_t items, int longest, int num_sms) { return (int)items <= num_sms / 2 && longest >= 4; }
 
 size_t bytes_for(const aoh_config& c, int n_r, int n_s) {
   const size_t tokens = (size_t)n_r * c.max_seq + (size_t)n_s * (size_t)(c.sink + c.window);
@@ -135,7 +146,7 @@ struct aoh_cache {
   uint32_t* d_err = nullptr;
   float* d_partials = nullptr;
   // prefill work list (device), grown on demand
-  int4* d_work = nullptr;
+  uint64_t* d_work = nullptr;
   size_t work_cap = 0;
   // H2Share anchor workspace (scores, head states, importance overflow),
   // allocated on first use
@@ -151,7 +162,7 @@ cudaError_t reserve_work(aoh_cache* h, size_t n) {
   if (h->d_work) cudaFree(h->d_work);
   h->d_work = nullptr;
   h->work_cap = 0;
-  cudaError_t e = cudaMalloc(&h->d_work, n * sizeof(int4));
+  cudaError_t e = cudaMalloc(&h->d_work, n * sizeof(uint64_t));
   if (e == cudaSuccess) h->work_cap = n;
   return e;
 }
@@ -406,11 +417,17 @@ aoh_status aoh_prefill(const void* q, const void* k, const void* v, int32_t T, c
   // positions its rows still read
   if (out) {
     const float scale_log2 = (float)(1.4426950408889634 / sqrt((double)g.D));
-    std::vector<int4> items = prefill_schedule(g, base, clen);
-    e = reserve_work(cache, items.size());
-    if (e != cudaSuccess) return cuda_fail(e, "work list allocation");
-    e = cudaMemcpyAsync(cache->d_work, items.data(), items.size() * sizeof(int4), cudaMemcpyHostToDevice, s);
-    if (e != cudaSuccess) return cuda_fail(e, "cudaMemcpyAsync(work)");
+    int longest = 0;
+    const std::vector<uint64_t> items = prefill_schedule(g, base, clen, &longest);
+    // up to kPrefillByValue items travel as kernel arguments: a copy from
+    // pageable memory waits for the stream's earlier work, so the GPU would
+    // stand idle from one call to the next
+    if (items.size() > (size_t)kPrefillByValue) {
+      e = reserve_work(cache, items.size());
+      if (e != cudaSuccess) return cuda_fail(e, "work list allocation");
+      e = cudaMemcpyAsync(cache->d_work, items.data(), items.size() * sizeof(uint64_t), cudaMemcpyHostToDevice, s);
+      if (e != cudaSuccess) return cuda_fail(e, "cudaMemcpyAsync(work)");
+    }
     PrefillTcArgs pa;
     memset(&pa, 0, sizeof(pa));
     pa.geom = g;
@@ -424,7 +441,8 @@ aoh_status aoh_prefill(const void* q, const void* k, const void* v, int32_t T, c
       return fail(AOH_ERR_CUDA, "cuTensorMapEncodeTiled failed for q/k/v");
     if (chunked && !prefill_tc_make_cache_maps(&pa, cache->kv))
       return fail(AOH_ERR_CUDA, "cuTensorMapEncodeTiled failed for the cache");
-    e = launch_prefill_tc(pa, (int)items.size(), prefill_split(items, cache->num_sms), s);
+    e = launch_prefill_tc(pa, items.data(), (int)items.size(),
+                          prefill_split(items.size(), longest, cache->num_sms), s);
     if (e != cudaSuccess) return cuda_fail(e, "prefill kernel launch");
   }
 

@@ -143,7 +143,7 @@ struct PrefillTcArgs {
   CacheGeom geom;
   void* out;            // [B][T][Hq][D]
   ChunkLens chunk;
-  const int4* work;     // {b, h, q0, cost}
+  const uint64_t* work; // items in device memory (more than kPrefillByValue)
   uint32_t* err;
   int T;
   float scale_log2;
@@ -153,6 +153,11 @@ struct PrefillTcArgs {
 // lands in *err; *elapsed_ns receives how long the wait lasted (0 if it did
 // not give up).
 cudaError_t launch_wait_selftest(uint32_t* err, uint64_t limit_ns, unsigned long long* elapsed_ns, cudaStream_t s);
+
+// A prefill work item: sequence b, query head h, rows 256 pair .. 256 pair + 255.
+inline uint64_t prefill_item(int b, int h, int pair) { return (uint64_t)b << 34 | (uint64_t)h << 24 | (uint32_t)pair; }
+// Work items that travel as kernel arguments (32 KB of them at most).
+constexpr int kPrefillByValue = 3840;
 
 // cuTensorMapEncodeTiled from the driver (nullptr if unavailable).
 PFN_cuTensorMapEncodeTiled_v12000 encode_fn();
@@ -170,8 +175,10 @@ bool make_cache_region_maps(CUtensorMap* tcr, CUtensorMap* tcs, const CacheGeom&
 // The maps of a decode step on the tcgen05 kernel (DecodeArgs); at d_head 64
 // box [1][1][128][64] over every second row.
 bool make_decode_maps(DecodeArgs* a, const CacheGeom& g, const void* kv);
-// One CTA a work item, or a cluster of two that halve its KV tiles (`split`).
-cudaError_t launch_prefill_tc(const PrefillTcArgs& a, int n_items, bool split, cudaStream_t s);
+// One CTA a work item, or a cluster of two that halve its KV tiles (`split`;
+// up to 256 items). `items` is host memory, a copy of a.work when there are more
+// than kPrefillByValue.
+cudaError_t launch_prefill_tc(const PrefillTcArgs& a, const uint64_t* items, int n_items, bool split, cudaStream_t s);
 // The CUDA-core decode kernel: the H2Share reuse step of d_head 64, with its
 // CTA count.
 cudaError_t launch_decode_cc(const DecodeArgs& a, cudaStream_t s);

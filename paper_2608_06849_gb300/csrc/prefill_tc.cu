@@ -38,6 +38,7 @@
 // TMEM columns: S_A / P_A [0,128), S_B / P_B [128,256), O_A [256, 256+D),
 // O_B [256+D, 256+2D).
 #include <math.h>
+#include <string.h>
 
 #include "cluster.cuh"
 #include "common.cuh"
@@ -86,8 +87,15 @@ __device__ __forceinline__ uint32_t range_bits(int lo, int hi) {
 // tiles; then each finishes one of the two query tiles: it receives the other
 // CTA's state of that tile (O, running max and sum) in shared memory that the
 // main loop no longer needs, adds its own and writes the rows.
-template <int D, bool SPLIT>
-__global__ void __launch_bounds__(kThreads, 1) prefill_tc_kernel(const __grid_constant__ PrefillTcArgs a) {
+// CAP: the work items that travel as arguments at most (0: they are in a.work).
+template <int CAP>
+struct WorkList {
+  uint64_t item[CAP > 0 ? CAP : 1];
+};
+
+template <int D, bool SPLIT, int CAP>
+__global__ void __launch_bounds__(kThreads, 1)
+    prefill_tc_kernel(const __grid_constant__ PrefillTcArgs a, const __grid_constant__ WorkList<CAP> wl) {
   using C = PfCfg<D>;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = smem_raw + ((1024 - (smem_u32(smem_raw) & 1023)) & 1023);
@@ -112,8 +120,9 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_tc_kernel(const __grid_co
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   // the append may start once the last CTAs of this grid run (append.cu)
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-  const int4 item = a.work[SPLIT ? blockIdx.x >> 1 : blockIdx.x];
-  const int b = item.x, h = item.y, q0 = item.z;
+  const int item_i = SPLIT ? blockIdx.x >> 1 : blockIdx.x;
+  const uint64_t item = CAP > 0 ? wl.item[item_i] : a.work[item_i];
+  const int b = (int)(item >> 34), h = (int)(item >> 24) & 1023, q0 = (int)(item & 0xffffffu) * 2 * kBM;
   const CacheGeom& g = a.geom;
   const int kvh = h / g.G;
   const bool streaming = g.kind[kvh] != 0;
@@ -615,13 +624,13 @@ bool make_map(CUtensorMap* map, const void* base, int B, int T, int H, int D) {
   return r == CUDA_SUCCESS;
 }
 
-template <int D, bool SPLIT>
-cudaError_t launch_cfg(const PrefillTcArgs& a, int n_items, cudaStream_t s) {
+template <int D, bool SPLIT, int CAP>
+cudaError_t launch_cfg(const PrefillTcArgs& a, const uint64_t* items, int n_items, cudaStream_t s) {
   using C = PfCfg<D>;
   static bool attr_set = false;
   if (!attr_set) {
     cudaError_t e =
-        cudaFuncSetAttribute(prefill_tc_kernel<D, SPLIT>, cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM);
+        cudaFuncSetAttribute(prefill_tc_kernel<D, SPLIT, CAP>, cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM);
     if (e != cudaSuccess) return e;
     attr_set = true;
   }
@@ -636,7 +645,18 @@ cudaError_t launch_cfg(const PrefillTcArgs& a, int n_items, cudaStream_t s) {
   attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
   cfg.attrs = attr;
   cfg.numAttrs = SPLIT ? 1 : 0;
-  return cudaLaunchKernelEx(&cfg, prefill_tc_kernel<D, SPLIT>, a);
+  WorkList<CAP> wl;
+  if (CAP > 0) memcpy(wl.item, items, n_items * sizeof(uint64_t));
+  return cudaLaunchKernelEx(&cfg, prefill_tc_kernel<D, SPLIT, CAP>, a, wl);
+}
+
+template <int D>
+cudaError_t launch_d(const PrefillTcArgs& a, const uint64_t* items, int n_items, bool split, cudaStream_t s) {
+  constexpr int kSmall = 256;
+  if (n_items <= kSmall)
+    return split ? launch_cfg<D, true, kSmall>(a, items, n_items, s) : launch_cfg<D, false, kSmall>(a, items, n_items, s);
+  if (n_items <= kPrefillByValue) return launch_cfg<D, false, kPrefillByValue>(a, items, n_items, s);
+  return launch_cfg<D, false, 0>(a, items, n_items, s);
 }
 
 }  // namespace
@@ -696,10 +716,10 @@ bool prefill_tc_make_cache_maps(PrefillTcArgs* a, const void* kv) {
   return make_cache_region_maps(&a->tcr, &a->tcs, a->geom, kv);
 }
 
-cudaError_t launch_prefill_tc(const PrefillTcArgs& a, int n_items, bool split, cudaStream_t s) {
+cudaError_t launch_prefill_tc(const PrefillTcArgs& a, const uint64_t* items, int n_items, bool split, cudaStream_t s) {
   if (n_items <= 0) return cudaSuccess;
-  if (a.geom.D == 128) return split ? launch_cfg<128, true>(a, n_items, s) : launch_cfg<128, false>(a, n_items, s);
-  if (a.geom.D == 64) return split ? launch_cfg<64, true>(a, n_items, s) : launch_cfg<64, false>(a, n_items, s);
+  if (a.geom.D == 128) return launch_d<128>(a, items, n_items, split, s);
+  if (a.geom.D == 64) return launch_d<64>(a, items, n_items, split, s);
   return cudaErrorInvalidValue;
 }
 

@@ -279,31 +279,46 @@ struct Labels {
   uint8_t a[kMaxKvHeads], r[kMaxKvHeads];
 };
 
-// sim(h, h') = tr(A B) / sqrt(n_a(h) n_r(h')) from the traces, then the
-// group means and the argmax. fp64 divides and square roots are slow on this
-// part: 2 Hq of them (the inverse norms), spread over the block's threads.
-__global__ void map_kernel(const double* num, const double* na, const double* nr, int Hq, int Hkv, Labels lab,
-                           double* inv, double* sim, double* gsim, int32_t* map) {
-  const int g = Hq / Hkv;
+// Group means of sim(h, h') = tr(A B) / sqrt(n_a(h) n_r(h')) and the argmax,
+// one block. fp64 divides and square roots are slow on this part: 2 Hq of them
+// (the inverse norms), spread over the block's threads. A warp sums a group
+// pair's head pairs (every lane its loads at once; one thread a pair waited for
+// an L2 round trip per head pair: 17 us at 28 / 4 heads). The launch is a
+// programmatic dependent of the query-side one.
+__global__ void __launch_bounds__(1024) map_kernel(const double* num, const double* na, const double* nr, int Hq, int Hkv,
+                                                   Labels lab, double* inv, double* gsim, int32_t* map,
+                                                   const uint32_t* err) {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  const int g = Hq / Hkv, lane = threadIdx.x & 31;
   for (int id = threadIdx.x; id < 2 * Hq; id += blockDim.x) inv[id] = 1.0 / sqrt(id < Hq ? na[id] : nr[id - Hq]);
   __syncthreads();
-  for (int id = threadIdx.x; id < Hq * Hq; id += blockDim.x) sim[id] = num[id] * inv[id / Hq] * inv[Hq + id % Hq];
-  __syncthreads();
-  for (int id = threadIdx.x; id < Hkv * Hkv; id += blockDim.x) {
+  for (int id = threadIdx.x >> 5; id < Hkv * Hkv; id += blockDim.x >> 5) {
     const int ga = id / Hkv, gr = id % Hkv;
     double s = 0.0;
-    for (int i = 0; i < g; ++i)
-      for (int j = 0; j < g; ++j) s += sim[(ga * g + i) * Hq + gr * g + j];
-    gsim[id] = s / (g * g);
+    for (int e = lane; e < g * g; e += 32) {
+      const int h = ga * g + e / g, hp = gr * g + e % g;
+      s += num[(size_t)h * Hq + hp] * inv[h] * inv[Hq + hp];
+    }
+#pragma unroll
+    for (int o = 16; o >= 1; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    if (lane == 0) gsim[id] = s / (g * g);
   }
   __syncthreads();
   for (int gr = threadIdx.x; gr < Hkv; gr += blockDim.x) {
     int best = -1;
+    double top = 0.0;
     if (lab.r[gr] == AOH_RETRIEVAL)
-      for (int ga = 0; ga < Hkv; ++ga)
-        if (lab.a[ga] == AOH_RETRIEVAL && (best < 0 || gsim[ga * Hkv + gr] > gsim[best * Hkv + gr])) best = ga;
+      for (int ga = 0; ga < Hkv; ++ga) {
+        const double v = gsim[ga * Hkv + gr];
+        if (lab.a[ga] == AOH_RETRIEVAL && (best < 0 || v > top)) {
+          best = ga;
+          top = v;
+        }
+      }
     map[gr] = best;
   }
+  // the timeouts of the launches before, beside the results: one copy back
+  if (threadIdx.x == 0) map[Hkv] = (int32_t)__ldcg(err);
 }
 
 // One workspace per device, grown on demand and kept for the process (a
@@ -347,10 +362,10 @@ extern "C" aoh_status aoh_h2share_map(const void* w_q_anchor, const void* w_k_an
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   const int Hq = n_q_heads, Hkv = n_kv_heads, dh = d_head, dm = d_model;
   const int nq = Hq * dh, nk = Hkv * dh;
-  // key-side Y, G_ka, G_kr; traces (pairs, two norm sets); inverse norms;
-  // head and group similarities; map; error word
-  const size_t bytes = 3 * (size_t)nk * nk * 4 + ((size_t)Hq * Hq + 2 * Hq) * 8 + 2 * (size_t)Hq * 8 +
-                       (size_t)Hq * Hq * 8 + (size_t)Hkv * Hkv * 8 + Hkv * 4 + 256;
+  // error word; key-side Y, G_ka, G_kr; traces (pairs, two norm sets); inverse
+  // norms; group similarities; map and a copy of the error word
+  const size_t bytes = 256 + 3 * (size_t)nk * nk * 4 + ((size_t)Hq * Hq + 2 * Hq) * 8 + 2 * (size_t)Hq * 8 +
+                       (size_t)Hkv * Hkv * 8 + Hkv * 4 + 256;
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess || dev < 0 || dev >= kWsDevices) return fail(AOH_ERR_CUDA, "aoh_h2share_map: no usable device");
@@ -360,21 +375,27 @@ extern "C" aoh_status aoh_h2share_map(const void* w_q_anchor, const void* w_k_an
     g_ws[dev] = nullptr;
     g_ws_cap[dev] = 0;
     e = cudaMalloc(&g_ws[dev], bytes);
-    if (e != cudaSuccess) return fail(AOH_ERR_CUDA, "aoh_h2share_map: workspace allocation failed");
+    // the error word stays zero from call to call (a call that finds it set
+    // clears it)
+    if (e == cudaSuccess) e = cudaMemsetAsync(g_ws[dev], 0, 256, s);
+    if (e != cudaSuccess) {
+      if (g_ws[dev]) cudaFree(g_ws[dev]);
+      g_ws[dev] = nullptr;
+      return fail(AOH_ERR_CUDA, "aoh_h2share_map: workspace allocation failed");
+    }
     g_ws_cap[dev] = bytes;
   }
   void* ws = g_ws[dev];
-  float* Y = static_cast<float*>(ws);
+  uint32_t* err = static_cast<uint32_t*>(ws);
+  float* Y = reinterpret_cast<float*>(static_cast<unsigned char*>(ws) + 256);
   float* gka = Y + (size_t)nk * nk;
   float* gkr = gka + (size_t)nk * nk;
   double* num = reinterpret_cast<double*>(gkr + (size_t)nk * nk);
   double* na = num + (size_t)Hq * Hq;
   double* nr = na + Hq;
   double* inv = nr + Hq;
-  double* sim = inv + 2 * (size_t)Hq;
-  double* gsim = sim + (size_t)Hq * Hq;
+  double* gsim = inv + 2 * (size_t)Hq;
   int32_t* map = reinterpret_cast<int32_t*>(gsim + (size_t)Hkv * Hkv);
-  uint32_t* err = reinterpret_cast<uint32_t*>(map + Hkv);
   GemmArgs kg{}, qg{};
   kg.K = qg.K = dm;
   kg.dh = qg.dh = dh;
@@ -382,19 +403,29 @@ extern "C" aoh_status aoh_h2share_map(const void* w_q_anchor, const void* w_k_an
   kg.err = qg.err = err;
   kg.trace = 0;
   qg.trace = 1;
-  bool maps_ok = add_problem(kg, w_k_reuse, nk, w_k_anchor, nk, dm, false, Y, nullptr, 0, nullptr) &&
-                 add_problem(kg, w_k_anchor, nk, w_k_anchor, nk, dm, false, gka, nullptr, 0, nullptr) &&
-                 add_problem(kg, w_k_reuse, nk, w_k_reuse, nk, dm, false, gkr, nullptr, 0, nullptr) &&
-                 add_problem(qg, w_q_anchor, nq, w_q_reuse, nq, dm, false, nullptr, Y, nk, num) &&
-                 add_problem(qg, w_q_anchor, nq, w_q_anchor, nq, dm, true, nullptr, gka, nk, na) &&
-                 add_problem(qg, w_q_reuse, nq, w_q_reuse, nq, dm, true, nullptr, gkr, nk, nr);
-  if (!maps_ok) e = cudaErrorInvalidValue;
-  if (e == cudaSuccess) e = cudaMemsetAsync(err, 0, 4, s);
+  // the key side runs while the host encodes the query side's maps
+  if (!(add_problem(kg, w_k_reuse, nk, w_k_anchor, nk, dm, false, Y, nullptr, 0, nullptr) &&
+        add_problem(kg, w_k_anchor, nk, w_k_anchor, nk, dm, false, gka, nullptr, 0, nullptr) &&
+        add_problem(kg, w_k_reuse, nk, w_k_reuse, nk, dm, false, gkr, nullptr, 0, nullptr)))
+    e = cudaErrorInvalidValue;
   if (e == cudaSuccess) e = launch_gemm(kg, s);
+  if (e == cudaSuccess && !(add_problem(qg, w_q_anchor, nq, w_q_reuse, nq, dm, false, nullptr, Y, nk, num) &&
+                            add_problem(qg, w_q_anchor, nq, w_q_anchor, nq, dm, true, nullptr, gka, nk, na) &&
+                            add_problem(qg, w_q_reuse, nq, w_q_reuse, nq, dm, true, nullptr, gkr, nk, nr)))
+    e = cudaErrorInvalidValue;
   if (e == cudaSuccess) e = launch_gemm(qg, s);
   if (e == cudaSuccess) {
-    map_kernel<<<1, 1024, 0, s>>>(num, na, nr, Hq, Hkv, lab, inv, sim, gsim, map);
-    e = cudaGetLastError();
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(1);
+    cfg.blockDim = dim3(1024);
+    cfg.stream = s;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    e = cudaLaunchKernelEx(&cfg, map_kernel, (const double*)num, (const double*)na, (const double*)nr, Hq, Hkv, lab, inv,
+                           gsim, map, (const uint32_t*)err);
   }
   // group similarities, map and error word are contiguous: one copy back
   const size_t res_bytes = (size_t)Hkv * Hkv * 8 + (size_t)Hkv * 4 + 4;
@@ -406,6 +437,10 @@ extern "C" aoh_status aoh_h2share_map(const void* w_q_anchor, const void* w_k_an
   memcpy(map_out, res.data() + (size_t)Hkv * Hkv * 8, (size_t)Hkv * 4);
   if (group_sim_out) memcpy(group_sim_out, res.data(), (size_t)Hkv * Hkv * 8);
   memcpy(&h_err, res.data() + (size_t)Hkv * Hkv * 8 + (size_t)Hkv * 4, 4);
-  if (h_err) return fail(AOH_ERR_TIMEOUT, "aoh_h2share_map: a kernel's bounded wait ran out");
+  if (h_err) {
+    cudaMemsetAsync(err, 0, sizeof(*err), s);
+    cudaStreamSynchronize(s);
+    return fail(AOH_ERR_TIMEOUT, "aoh_h2share_map: a kernel's bounded wait ran out");
+  }
   return AOH_OK;
 }

@@ -201,16 +201,17 @@ __global__ void __launch_bounds__(kGramTcThreads, 1)
       }
     }
   };
-  auto issue = [&](bool fresh) {  // one thread: the step's digit pairs
-    const uint32_t base = smem_u32(smem);
+  auto issue = [&](bool fresh) {  // one elected lane: the step's digit pairs
+    const uint64_t base = sdesc_sw128(smem_u32(smem), 16, 1024);
     for (int a = 0; a < 4; ++a) {
       const int c = a + (high ? 6 : 2);
       const int i0 = max(1, c - kDigits), i1 = min(c - 1, kDigits);
       for (int i = i0; i <= i1; ++i) {
-        const uint32_t da = base + (i - 1) * kDigitTile, db = base + (c - i - 1) * kDigitTile;
+        const uint64_t da = base + (uint32_t)((i - 1) * sdesc_step(kDigitTile));
+        const uint64_t db = base + (uint32_t)((c - i - 1) * sdesc_step(kDigitTile));
 #pragma unroll
         for (int kk = 0; kk < 4; ++kk)
-          tc_mma(tmem + a * 128, sdesc_sw128(da + kk * 32, 16, 1024), sdesc_sw128(db + kk * 32, 16, 1024), kGramIdesc,
+          tc_mma(tmem + a * 128, da + sdesc_step(kk * 32), db + sdesc_step(kk * 32), kGramIdesc,
                  (fresh && i == i0 && kk == 0) ? 0u : 1u);
       }
     }
@@ -260,9 +261,9 @@ __global__ void __launch_bounds__(kGramTcThreads, 1)
     tc_fence_before();
     ok = __syncthreads_and(ok);
     if (!ok) break;
-    if (t == 0) {
+    if (warp == 0) {
       tc_fence_after();
-      issue(fresh);
+      if (elect_one()) issue(fresh);
     }
     __syncwarp();
   }

@@ -462,7 +462,9 @@ __global__ void __launch_bounds__(kThreads + 32 * gather_warps(G, MODE), 1)
     __syncwarp();
   } else if (warp == 5) {
     // ------------------------------------------------------------ MMA issuer
-    const uint32_t kv_addr = smem_u32(sKV), q_addr = smem_u32(sQ), p_addr = smem_u32(sP);
+    const uint64_t k_desc0 = sdesc_sw128(smem_u32(sKV), 16, 1024);
+    const uint64_t v_desc0 = sdesc_sw128(smem_u32(sKV) + kTile, kBox, 1024);
+    const uint64_t q_desc0 = sdesc_sw128(smem_u32(sQ), 16, 1024), p_desc0 = sdesc_sw128(smem_u32(sP), 16, 1024);
     int it = 0, item_k = 0, ofw = 0;
     uint32_t fpar = 0, gpar = 0;  // bit st: parity of stage st's next full[] / gfull[] phase
     bool ok = true;
@@ -485,14 +487,14 @@ __global__ void __launch_bounds__(kThreads + 32 * gather_warps(G, MODE), 1)
       wait_warp(&p_full[t.it & 1], (t.it >> 1) & 1);
       if (t.first && t.item >= 1) wait_ofree(t.item);  // accumulate = 0 overwrites the last item's O
       if (!ok) return;
-      if (lane == 0) {
+      if (elect_one()) {
         tc_fence_after();
-        const uint32_t v_addr = kv_addr + t.st * kStage + kTile;
-        const uint32_t pb = p_addr + (t.it % C::NPB) * C::PBUF;
+        const uint64_t v_desc = v_desc0 + (uint32_t)(t.st * sdesc_step(kStage));
+        const uint64_t p_desc = p_desc0 + (uint32_t)((t.it % C::NPB) * sdesc_step(C::PBUF));
 #pragma unroll
         for (int kk = 0; kk < kBN / 16; ++kk) {
-          const uint64_t ad = sdesc_sw128(v_addr + kk * 2048, kBox, 1024);
-          const uint64_t bd = sdesc_sw128(pb + (kk >> 2) * (C::NPV * 128) + (kk & 3) * 32, 16, 1024);
+          const uint64_t ad = v_desc + sdesc_step(kk * 2048);
+          const uint64_t bd = p_desc + sdesc_step((kk >> 2) * (C::NPV * 128) + (kk & 3) * 32);
           tc_mma(tmem + C::OCOL, ad, bd, C::IDESC_PV, (t.first && kk == 0) ? 0u : 1u);
         }
         tc_commit(&p_free[t.it & 1]);
@@ -608,16 +610,16 @@ __global__ void __launch_bounds__(kThreads + 32 * gather_warps(G, MODE), 1)
         }
         if (it >= 2) wait_warp(&s_free[it & 1], ((it >> 1) - 1) & 1);
         if (!ok) break;
-        if (lane == 0) {
+        if (elect_one()) {
           tc_fence_after();
-          const uint32_t k_addr = kv_addr + st * kStage;
-          const uint32_t qb = q_addr + (item_k & 1) * C::QBUF;
+          const uint64_t k_desc = k_desc0 + (uint32_t)(st * sdesc_step(kStage));
+          const uint64_t q_desc = q_desc0 + (uint32_t)((item_k & 1) * sdesc_step(C::QBUF));
 #pragma unroll
           for (int kk = 0; kk < 8; ++kk) {
             // d_head 128: 8 K-steps over both blocks; 64: 4 over each parity's block
             const int y = PAIR ? kk >> 2 : 0;
-            const uint64_t ad = sdesc_sw128(k_addr + (kk >> 2) * kBox + (kk & 3) * 32, 16, 1024);
-            const uint64_t bd = sdesc_sw128(qb + (PAIR ? 0 : kk >> 2) * (kN * 128) + (kk & 3) * 32, 16, 1024);
+            const uint64_t ad = k_desc + sdesc_step((kk >> 2) * kBox + (kk & 3) * 32);
+            const uint64_t bd = q_desc + sdesc_step((PAIR ? 0 : kk >> 2) * (kN * 128) + (kk & 3) * 32);
             tc_mma(tmem + (it & 1) * C::SCOLS + y * kN, ad, bd, C::IDESC_S, (PAIR ? kk & 3 : kk) > 0 ? 1u : 0u);
           }
           tc_commit(&s_full[it & 1]);
@@ -646,10 +648,9 @@ __global__ void __launch_bounds__(kThreads + 32 * gather_warps(G, MODE), 1)
       ++item_k;
     }
     if (has_pend) issue_pv(pend);
-    if (lane == 0) {
-      tc_commit(drain);
-      drain_wait(drain, 0, a.err);
-    }
+    if (elect_one()) tc_commit(drain);
+    __syncwarp();
+    drain_wait(drain, 0, a.err);
     __syncwarp();
   } else {
     // ------------------------------------------------------------ softmax

@@ -134,21 +134,23 @@ __global__ void __launch_bounds__(kGemmThreads, 2) gemm_kernel(const __grid_cons
         drain_wait(&full[j % kStages], (j / kStages) & 1, a.err);
     }
   } else if (warp == 1) {
-    if (lane == 0) {
-      for (int kc = 0; kc < nk; ++kc) {
-        const int st = kc % kStages;
-        if (!wait_bar(&full[st], (kc / kStages) & 1, a.err, abort_flag)) break;
-        tc_fence_after();
-        const uint32_t aa = smem_u32(sA + st * kTileBytes), bb = smem_u32(sB + st * kTileBytes);
+    const uint64_t a_desc = sdesc_sw128(smem_u32(sA), 16, 1024), b_desc = sdesc_sw128(smem_u32(sB), 16, 1024);
+    for (int kc = 0; kc < nk; ++kc) {
+      const int st = kc % kStages;
+      if (!__all_sync(0xffffffffu, wait_bar(&full[st], (kc / kStages) & 1, a.err, abort_flag))) break;
+      tc_fence_after();
+      const uint32_t off = st * sdesc_step(kTileBytes);
+      if (elect_one()) {
 #pragma unroll
         for (int kk = 0; kk < kTK / 16; ++kk)
-          tc_mma(tmem, sdesc_sw128(aa + kk * 32, 16, 1024), sdesc_sw128(bb + kk * 32, 16, 1024), IDESC,
+          tc_mma(tmem, a_desc + (off + sdesc_step(kk * 32)), b_desc + (off + sdesc_step(kk * 32)), IDESC,
                  (kc > 0 || kk > 0) ? 1u : 0u);
         tc_commit(&empty[st]);
       }
-      tc_commit(done);
-      drain_wait(done, 0, a.err);  // this warp frees TMEM: its MMAs must be done
     }
+    if (elect_one()) tc_commit(done);
+    __syncwarp();
+    drain_wait(done, 0, a.err);  // this warp frees TMEM: its MMAs must be done
   } else {
     // epilogue: warp w reads TMEM lanes 32 * (w % 4) .. + 31, rows of the
     // tile. M and N are multiples of 32, so a warp's rows and a 32-column

@@ -260,70 +260,82 @@ __global__ void __launch_bounds__(kThreads, 1)
     __syncwarp();
   } else if (warp == 1) {
     // ------------------------------------------------------------ MMA issuer
-    if (lane == 0) {
-      const uint32_t q_addr = smem_u32(sQ), kv_addr = smem_u32(sKV);
-      auto issue_s = [&](int x, int jj) {
-        const uint32_t k_addr = kv_addr + ((2 * jj) % kNS) * C::KVBYTES;
-        const uint32_t qa = q_addr + x * C::QBYTES;
+    // The whole warp runs the loop (its values stay warp-uniform); one elected
+    // lane, the same each time, issues.
+    const uint64_t q_desc = sdesc_sw128(smem_u32(sQ), 16, 1024);
+    const uint64_t k_desc0 = sdesc_sw128(smem_u32(sKV), 16, 1024);
+    const uint64_t v_desc0 = sdesc_sw128(smem_u32(sKV), C::BOX, 1024);
+    auto issue_s = [&](int x, int jj) {
+      const uint64_t k_desc = k_desc0 + (uint32_t)(((2 * jj) % kNS) * sdesc_step(C::KVBYTES));
+      if (elect_one()) {
 #pragma unroll
         for (int kk = 0; kk < D / 16; ++kk) {
-          const uint64_t ad = sdesc_sw128(qa + (kk >> 2) * C::BOX + (kk & 3) * 32, 16, 1024);
-          const uint64_t bd = sdesc_sw128(k_addr + (kk >> 2) * C::BOX + (kk & 3) * 32, 16, 1024);
-          tc_mma(tmem + x * 128, ad, bd, C::IDESC_S, kk > 0 ? 1u : 0u);
+          const uint32_t off = sdesc_step((kk >> 2) * C::BOX + (kk & 3) * 32);
+          tc_mma(tmem + x * 128, q_desc + (sdesc_step(x * C::QBYTES) + off), k_desc + off, C::IDESC_S, kk > 0 ? 1u : 0u);
         }
         tc_commit(&s_full[x]);
-      };
-      auto issue_pv = [&](int x, int jj) {
-        const uint32_t v_addr = kv_addr + ((2 * jj + 1) % kNS) * C::KVBYTES;
+      }
+    };
+    auto issue_pv = [&](int x, int jj) {
+      const uint64_t v_desc = v_desc0 + (uint32_t)(((2 * jj + 1) % kNS) * sdesc_step(C::KVBYTES));
+      if (elect_one()) {
 #pragma unroll
-        for (int kk = 0; kk < kBN / 16; ++kk) {
-          const uint64_t bd = sdesc_sw128(v_addr + kk * 16 * 128, C::BOX, 1024);
-          tc_mma_ts(tmem + 256 + x * D, tmem + x * 128 + kk * 8, bd, C::IDESC_PV, (jj > 0 || kk > 0) ? 1u : 0u);
-        }
+        for (int kk = 0; kk < kBN / 16; ++kk)
+          tc_mma_ts(tmem + 256 + x * D, tmem + x * 128 + kk * 8, v_desc + sdesc_step(kk * 16 * 128), C::IDESC_PV,
+                    (jj > 0 || kk > 0) ? 1u : 0u);
         tc_commit(&pv_done[x]);
-      };
-      auto wait_k = [&](int jj) { return wait_bar(&kv_full[(2 * jj) % kNS], ((2 * jj) / kNS) & 1, a.err, abort_flag); };
-      int n_partial = 0;  // partial V tiles seen so far (index into v_zeroed)
-      auto wait_v = [&](int jj) {
-        if (!wait_bar(&kv_full[(2 * jj + 1) % kNS], ((2 * jj + 1) / kNS) & 1, a.err, abort_flag)) return false;
-        if (tile_valid(jj) < kBN && n_partial < 2) {
-          if (!wait_bar(&v_zeroed[n_partial], 0, a.err, abort_flag)) return false;
-          ++n_partial;
-        }
-        return true;
-      };
-      bool ok = n_tiles > 0 && wait_bar(q_full, 0, a.err, abort_flag) && wait_k(0);
-      if (ok) {
-        tc_fence_after();
-        issue_s(0, 0);
-        issue_s(1, 0);
-        tc_commit(&kv_empty[0]);
       }
-      for (int jj = 0; jj < n_tiles && ok; ++jj) {
-        const bool more = jj + 1 < n_tiles;
-        const uint32_t ph = jj & 1;
-        // tile A: P_A(jj) sits in S_A's columns; S_A(jj+1) may overwrite them
-        // only after O_A += P_A(jj) V_jj is issued (same-thread MMAs run in order)
-        if (!wait_v(jj) || !wait_bar(&p_full[0], ph, a.err, abort_flag)) { ok = false; break; }
-        tc_fence_after();
-        issue_pv(0, jj);
-        if (more) {
-          if (!wait_k(jj + 1)) { ok = false; break; }
-          tc_fence_after();
-          issue_s(0, jj + 1);
-        }
-        if (!wait_bar(&p_full[1], ph, a.err, abort_flag)) { ok = false; break; }
-        tc_fence_after();
-        issue_pv(1, jj);
-        tc_commit(&kv_empty[(2 * jj + 1) % kNS]);
-        if (more) {
-          issue_s(1, jj + 1);
-          tc_commit(&kv_empty[(2 * (jj + 1)) % kNS]);
-        }
+    };
+    auto commit = [&](uint64_t* bar) {
+      if (elect_one()) tc_commit(bar);
+    };
+    bool ok = n_tiles > 0;
+    auto wait = [&](uint64_t* bar, uint32_t parity) {
+      if (ok) ok = __all_sync(0xffffffffu, wait_bar(bar, parity, a.err, abort_flag));
+      return ok;
+    };
+    auto wait_k = [&](int jj) { return wait(&kv_full[(2 * jj) % kNS], ((2 * jj) / kNS) & 1); };
+    int n_partial = 0;  // partial V tiles seen so far (index into v_zeroed)
+    auto wait_v = [&](int jj) {
+      if (!wait(&kv_full[(2 * jj + 1) % kNS], ((2 * jj + 1) / kNS) & 1)) return false;
+      if (tile_valid(jj) < kBN && n_partial < 2) {
+        if (!wait(&v_zeroed[n_partial], 0)) return false;
+        ++n_partial;
       }
-      tc_commit(drain);
-      drain_wait(drain, 0, a.err);
+      return true;
+    };
+    if (wait(q_full, 0) && wait_k(0)) {
+      tc_fence_after();
+      issue_s(0, 0);
+      issue_s(1, 0);
+      commit(&kv_empty[0]);
     }
+    for (int jj = 0; jj < n_tiles && ok; ++jj) {
+      const bool more = jj + 1 < n_tiles;
+      const uint32_t ph = jj & 1;
+      // tile A: P_A(jj) sits in S_A's columns; S_A(jj+1) may overwrite them
+      // only after O_A += P_A(jj) V_jj is issued (same-thread MMAs run in order)
+      if (!wait_v(jj) || !wait(&p_full[0], ph)) break;
+      tc_fence_after();
+      issue_pv(0, jj);
+      if (more) {
+        if (!wait_k(jj + 1)) break;
+        tc_fence_after();
+        issue_s(0, jj + 1);
+      }
+      if (!wait(&p_full[1], ph)) break;
+      tc_fence_after();
+      issue_pv(1, jj);
+      commit(&kv_empty[(2 * jj + 1) % kNS]);
+      if (more) {
+        issue_s(1, jj + 1);
+        commit(&kv_empty[(2 * (jj + 1)) % kNS]);
+      }
+    }
+    commit(drain);
+    __syncwarp();
+    drain_wait(drain, 0, a.err);
+    __syncwarp();
   } else {
     // ------------------------------------------------------------ softmax
     const int x = (warp - 2) >> 2;        // 0: tile A (warps 2-5), 1: tile B (warps 6-9)

@@ -7,6 +7,7 @@
 #include <string.h>
 
 #include <algorithm>
+#include <functional>
 #include <string>
 #include <vector>
 
@@ -66,9 +67,9 @@ aoh_status check_config(const aoh_config* cfg, const uint8_t* labels, int* n_r, 
 // heaviest first so the hardware block scheduler fills the machine
 // longest-processing-time first. The cost, the number of 128-key tiles visited,
 // is the same for all heads of a kind, so (b, pair, kind) entries are sorted and
-// then expanded into heads. *longest receives the first item's cost.
+// then expanded into heads. *costs receives each item's cost.
 std::vector<uint64_t> prefill_schedule(const CacheGeom& g, const std::vector<int32_t>& base,
-                                       const std::vector<int32_t>& lens, int* longest) {
+                                       const std::vector<int32_t>& lens, std::vector<int>* costs) {
   constexpr int BM = 256, BN = 128;
   struct Entry {
     int cost, b, pair, streaming;
@@ -98,24 +99,86 @@ std::vector<uint64_t> prefill_schedule(const CacheGeom& g, const std::vector<int
   std::stable_sort(entries.begin(), entries.end(), [](const Entry& x, const Entry& y) { return x.cost > y.cost; });
   std::vector<uint64_t> items;
   items.reserve(entries.size() * (size_t)g.Hq);
+  costs->reserve(entries.size() * (size_t)g.Hq);
   for (const Entry& e : entries)
     for (int i = 0; i < (e.streaming ? g.n_s : g.n_r); ++i) {
       const int kvh = e.streaming ? g.s_head[i] : g.r_head[i];
-      for (int h = kvh * g.G; h < (kvh + 1) * g.G; ++h) items.push_back(prefill_item(e.b, h, e.pair));
+      for (int h = kvh * g.G; h < (kvh + 1) * g.G; ++h) {
+        items.push_back(prefill_item(e.b, h, e.pair));
+        costs->push_back(e.cost);
+      }
     }
-  *longest = entries.empty() ? 0 : entries[0].cost;
   return items;
 }
 
-// Whether clusters of two CTAs halve each item's KV tiles: when every item's
-// cluster runs at once, the call lasts as long as its longest item.
-// Measured (8 heads of 128, one sequence, us of the kernel without / with):
-// 256 rows (2 tiles) 11.2 / 11.5, 384 11.8 / 13.4, 512 15.4 / 13.5, 1024 21.1 /
-// 17.5, 2048 34.8 / 24.4; heads of 64: 384 11.4 / 11.6, 512 13.9 / 11.7, 2048
-// 30.8 / 21.1. In more waves it does not pay: 4K rows after a long prefix (448
-// items) took 2% longer, the exchange of the states and the second start of a
-// pipeline costing more than the fuller last wave gives.
-bool prefill_split(size_t items, int longest, int num_sms) { return (int)items <= num_sms / 2 && longest >= 4; }
+// The work of clusters of two CTAs, two entries a cluster: two items, or one item
+// twice, with kPrefillHalf, that its CTAs share (kPrefillNone fills the last
+// cluster). Nothing when one CTA an item is as good.
+//
+// When every item's cluster runs at once, the call lasts as long as its longest
+// item, and sharing all halves that. Measured (8 heads of 128, one sequence, us of
+// the kernel without / with): 256 rows (2 tiles) 11.2 / 11.5, 384 11.8 / 13.4, 512
+// 15.4 / 13.5, 1024 21.1 / 17.5, 2048 34.8 / 24.4; heads of 64: 384 11.4 / 11.6,
+// 512 13.9 / 11.7, 2048 30.8 / 21.1.
+//
+// In a few waves, as in a chunk after a long prefix whose heavy items all read it,
+// a last wave of heavy items that leaves many SMs idle is shared, while the
+// lighter items behind it are not. k + 1 of the first k * num_sms + 1 items meet
+// on one SM; where that ends a tenth later than the work spread evenly, the ends
+// of longest-first schedules decide, in visited tiles, with 4 tiles' time added
+// to an item and 8 to a half: nothing shared, or half a wave or a whole one from
+// item k * num_sms on. Past four items an SM the last wave matters little. 28
+// heads of 128, half of them streaming (S = 128, W = 2048), us of a call without /
+// with: 4096 rows after 16K tokens 388 / 388 (not shared), 20K 471 / 461, 24K 555 /
+// 526, 28K 638 / 585; 1024 rows after 24K 272 / 151.
+std::vector<uint64_t> prefill_pairs(const std::vector<uint64_t>& items, const std::vector<int>& costs, int num_sms) {
+  const int n = (int)items.size(), slots = num_sms / 2;
+  int first = 0, last = 0;  // items [first, last) are shared
+  if (n <= slots) {
+    if (n > 0 && costs[0] >= 4) last = n;
+  } else if (n <= std::min(4 * num_sms, kPrefillSplitMost)) {
+    long long work = 0, meet = 0;
+    for (int c : costs) work += c + 4;
+    for (int a = 0; a < n; a += num_sms)
+      if ((a / num_sms + 1) * (long long)(costs[a] + 4) > meet) {
+        meet = (a / num_sms + 1) * (long long)(costs[a] + 4);
+        first = a;
+      }
+    if (meet * num_sms * 10 > work * 11) {
+      std::vector<int> free_at;  // a min-heap
+      auto end_of = [&](int count, int shared_end) {
+        free_at.assign(count, 0);
+        int end = 0;
+        for (int i = 0; i < n;) {
+          const bool half = i >= first && i < shared_end;
+          std::pop_heap(free_at.begin(), free_at.end(), std::greater<int>());
+          end = std::max(end, free_at.back() += half ? (costs[i] + 1) / 2 + 8 : costs[i] + 4);
+          std::push_heap(free_at.begin(), free_at.end(), std::greater<int>());
+          i += count == num_sms || half ? 1 : 2;
+        }
+        return end;
+      };
+      int best = end_of(num_sms, 0);
+      for (int window = slots; window <= 2 * slots; window += slots) {
+        const int end = end_of(slots, first + window);
+        if (end < best) {
+          best = end;
+          last = std::min(first + window, n);
+        }
+      }
+    }
+  }
+  std::vector<uint64_t> pairs;
+  if (last == 0) return pairs;
+  pairs.reserve(n + last - first + 2);
+  for (int i = 0; i < n; ++i) {
+    const bool half = i >= first && i < last;
+    if (half) pairs.push_back(items[i] | kPrefillHalf);
+    pairs.push_back(items[i] | (half ? kPrefillHalf : 0));
+  }
+  if (pairs.size() & 1) pairs.push_back(kPrefillNone);
+  return pairs;
+}
 
 size_t bytes_for(const aoh_config& c, int n_r, int n_s) {
   const size_t tokens = (size_t)n_r * c.max_seq + (size_t)n_s * (size_t)(c.sink + c.window);
@@ -417,8 +480,9 @@ aoh_status aoh_prefill(const void* q, const void* k, const void* v, int32_t T, c
   // positions its rows still read
   if (out) {
     const float scale_log2 = (float)(1.4426950408889634 / sqrt((double)g.D));
-    int longest = 0;
-    const std::vector<uint64_t> items = prefill_schedule(g, base, clen, &longest);
+    std::vector<int> costs;
+    const std::vector<uint64_t> items = prefill_schedule(g, base, clen, &costs);
+    const std::vector<uint64_t> pairs = prefill_pairs(items, costs, cache->num_sms);
     // up to kPrefillByValue items travel as kernel arguments: a copy from
     // pageable memory waits for the stream's earlier work, so the GPU would
     // stand idle from one call to the next
@@ -441,8 +505,7 @@ aoh_status aoh_prefill(const void* q, const void* k, const void* v, int32_t T, c
       return fail(AOH_ERR_CUDA, "cuTensorMapEncodeTiled failed for q/k/v");
     if (chunked && !prefill_tc_make_cache_maps(&pa, cache->kv))
       return fail(AOH_ERR_CUDA, "cuTensorMapEncodeTiled failed for the cache");
-    e = launch_prefill_tc(pa, items.data(), (int)items.size(),
-                          prefill_split(items.size(), longest, cache->num_sms), s);
+    e = launch_prefill_tc(pa, items, pairs, s);
     if (e != cudaSuccess) return cuda_fail(e, "prefill kernel launch");
   }
 

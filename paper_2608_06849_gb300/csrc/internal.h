@@ -7,6 +7,8 @@
 #include <stddef.h>
 #include <stdint.h>
 
+#include <vector>
+
 namespace aoh {
 
 constexpr int kMaxKvHeads = 64;
@@ -156,8 +158,12 @@ cudaError_t launch_wait_selftest(uint32_t* err, uint64_t limit_ns, unsigned long
 
 // A prefill work item: sequence b, query head h, rows 256 pair .. 256 pair + 255.
 inline uint64_t prefill_item(int b, int h, int pair) { return (uint64_t)b << 34 | (uint64_t)h << 24 | (uint32_t)pair; }
+// A half of an item that a cluster's two CTAs share, and an entry without work.
+constexpr uint64_t kPrefillHalf = 1ull << 63, kPrefillNone = ~0ull;
 // Work items that travel as kernel arguments (32 KB of them at most).
 constexpr int kPrefillByValue = 3840;
+// Most work items of a launch on clusters of two CTAs.
+constexpr int kPrefillSplitMost = 640;
 
 // cuTensorMapEncodeTiled from the driver (nullptr if unavailable).
 PFN_cuTensorMapEncodeTiled_v12000 encode_fn();
@@ -175,10 +181,11 @@ bool make_cache_region_maps(CUtensorMap* tcr, CUtensorMap* tcs, const CacheGeom&
 // The maps of a decode step on the tcgen05 kernel (DecodeArgs); at d_head 64
 // box [1][1][128][64] over every second row.
 bool make_decode_maps(DecodeArgs* a, const CacheGeom& g, const void* kv);
-// One CTA a work item, or a cluster of two that halve its KV tiles (`split`;
-// up to 256 items). `items` is host memory, a copy of a.work when there are more
-// than kPrefillByValue.
-cudaError_t launch_prefill_tc(const PrefillTcArgs& a, const uint64_t* items, int n_items, bool split, cudaStream_t s);
+// One CTA an entry of `pairs`, in clusters of two, or a work item when it is
+// empty. Host memory; the items are a copy of a.work when there are more than
+// kPrefillByValue.
+cudaError_t launch_prefill_tc(const PrefillTcArgs& a, const std::vector<uint64_t>& items,
+                              const std::vector<uint64_t>& pairs, cudaStream_t s);
 // The CUDA-core decode kernel: the H2Share reuse step of d_head 64, with its
 // CTA count.
 cudaError_t launch_decode_cc(const DecodeArgs& a, cudaStream_t s);

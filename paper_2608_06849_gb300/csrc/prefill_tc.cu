@@ -48,11 +48,12 @@ namespace {
 
 using namespace pf;
 
-// SPLIT: a cluster of two CTAs shares one work item. Each visits half of its KV
-// tiles; then each finishes one of the two query tiles: it receives the other
+// PAIRS: clusters of two CTAs, each with its entry of the list. Where both have the
+// same item's halves, each visits half of its KV tiles; then each finishes one of
+// the two query tiles: it receives the other
 // CTA's state of that tile (O, running max and sum) in shared memory that the
 // main loop no longer needs, adds its own and writes the rows.
-template <int D, bool SPLIT, int CAP>
+template <int D, bool PAIRS, int CAP>
 __global__ void __launch_bounds__(kThreads, 1)
     prefill_tc_kernel(const __grid_constant__ PrefillTcArgs a, const __grid_constant__ WorkList<CAP> wl) {
   using C = PfCfg<D>;
@@ -78,14 +79,16 @@ __global__ void __launch_bounds__(kThreads, 1)
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   // the append may start once the last CTAs of this grid run (append.cu)
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-  const int item_i = SPLIT ? blockIdx.x >> 1 : blockIdx.x;
-  const Item t(a, CAP > 0 ? wl.item[item_i] : a.work[item_i]);
+  const uint64_t code = CAP > 0 ? wl.item[blockIdx.x] : a.work[blockIdx.x];
+  if (PAIRS && code == kPrefillNone) return;
+  const bool half = PAIRS && code >= kPrefillHalf;  // alike in both CTAs of a cluster
+  const Item t(a, code & ~kPrefillHalf);
   const CacheGeom& g = a.geom;
   const int n_all = t.tiles();
   // this CTA visits tiles t0 .. t0 + n_tiles - 1 of the item's n_all
-  const int rank = SPLIT ? (int)cluster_rank() : 0;
+  const int rank = half ? (int)cluster_rank() : 0;
   const int t0 = rank * ((n_all + 1) / 2);
-  const int n_tiles = !SPLIT ? n_all : rank == 0 ? (n_all + 1) / 2 : n_all / 2;
+  const int n_tiles = !half ? n_all : rank == 0 ? (n_all + 1) / 2 : n_all / 2;
   if (threadIdx.x == 0) {
     mbar_init(q_full, 2);
     for (int s = 0; s < kNS; ++s) {
@@ -118,7 +121,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   tc_fence_after();
   const uint32_t tmem = *tmem_slot;
 
-  // SPLIT: a row's final softmax state (softmax warps)
+  // a half: a row's final softmax state (softmax warps)
   float end_m = -INFINITY, end_l = 0.f;
   bool end_ok = true;
   if (warp == 0) {
@@ -257,7 +260,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       ok = softmax_tile<D>(a, mask, tl, s_col, o_col, jj == 0, m, l, &pv_done[x], (jj - 1) & 1,
                            &p_full[2 * x], abort_flag);
     }
-    if constexpr (SPLIT) {
+    if (half) {
       end_m = m;
       end_l = l;
       end_ok = ok && (n_tiles == 0 ||
@@ -272,7 +275,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
-  if constexpr (SPLIT) {
+  if (half) {
     // both CTAs' copies and MMAs are done with their shared memory
     cluster_arrive();
     cluster_wait();
@@ -367,18 +370,20 @@ bool make_map(CUtensorMap* map, const void* base, int B, int T, int H, int D) {
   return r == CUDA_SUCCESS;
 }
 
-template <int D, bool SPLIT, int CAP>
-cudaError_t launch_cfg(const PrefillTcArgs& a, const uint64_t* items, int n_items, cudaStream_t s) {
+constexpr int kSmall = 640;  // items of a launch that copies 5 KB of arguments instead of 30
+
+template <int D, bool PAIRS, int CAP>
+cudaError_t launch_cfg(const PrefillTcArgs& a, const std::vector<uint64_t>& items, cudaStream_t s) {
   using C = PfCfg<D>;
   static bool attr_set = false;
   if (!attr_set) {
     cudaError_t e =
-        cudaFuncSetAttribute(prefill_tc_kernel<D, SPLIT, CAP>, cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM);
+        cudaFuncSetAttribute(prefill_tc_kernel<D, PAIRS, CAP>, cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM);
     if (e != cudaSuccess) return e;
     attr_set = true;
   }
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(SPLIT ? 2 * n_items : n_items);
+  cfg.gridDim = dim3((unsigned)items.size());
   cfg.blockDim = dim3(kThreads);
   cfg.dynamicSmemBytes = C::SMEM;
   cfg.stream = s;
@@ -387,19 +392,19 @@ cudaError_t launch_cfg(const PrefillTcArgs& a, const uint64_t* items, int n_item
   attr[0].val.clusterDim.x = 2;
   attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
   cfg.attrs = attr;
-  cfg.numAttrs = SPLIT ? 1 : 0;
+  cfg.numAttrs = PAIRS ? 1 : 0;
   WorkList<CAP> wl;
-  if (CAP > 0) memcpy(wl.item, items, n_items * sizeof(uint64_t));
-  return cudaLaunchKernelEx(&cfg, prefill_tc_kernel<D, SPLIT, CAP>, a, wl);
+  if (CAP > 0) memcpy(wl.item, items.data(), items.size() * sizeof(uint64_t));
+  return cudaLaunchKernelEx(&cfg, prefill_tc_kernel<D, PAIRS, CAP>, a, wl);
 }
 
 template <int D>
-cudaError_t launch_d(const PrefillTcArgs& a, const uint64_t* items, int n_items, bool split, cudaStream_t s) {
-  constexpr int kSmall = 256;
-  if (n_items <= kSmall)
-    return split ? launch_cfg<D, true, kSmall>(a, items, n_items, s) : launch_cfg<D, false, kSmall>(a, items, n_items, s);
-  if (n_items <= kPrefillByValue) return launch_cfg<D, false, kPrefillByValue>(a, items, n_items, s);
-  return launch_cfg<D, false, 0>(a, items, n_items, s);
+cudaError_t launch_d(const PrefillTcArgs& a, const std::vector<uint64_t>& items, const std::vector<uint64_t>& pairs,
+                     cudaStream_t s) {
+  if (!pairs.empty()) return launch_cfg<D, true, 2 * kPrefillSplitMost>(a, pairs, s);
+  if (items.size() <= kSmall) return launch_cfg<D, false, kSmall>(a, items, s);
+  if (items.size() <= kPrefillByValue) return launch_cfg<D, false, kPrefillByValue>(a, items, s);
+  return launch_cfg<D, false, 0>(a, items, s);
 }
 
 }  // namespace
@@ -459,10 +464,11 @@ bool prefill_tc_make_cache_maps(PrefillTcArgs* a, const void* kv) {
   return make_cache_region_maps(&a->tcr, &a->tcs, a->geom, kv);
 }
 
-cudaError_t launch_prefill_tc(const PrefillTcArgs& a, const uint64_t* items, int n_items, bool split, cudaStream_t s) {
-  if (n_items <= 0) return cudaSuccess;
-  if (a.geom.D == 128) return launch_d<128>(a, items, n_items, split, s);
-  if (a.geom.D == 64) return launch_d<64>(a, items, n_items, split, s);
+cudaError_t launch_prefill_tc(const PrefillTcArgs& a, const std::vector<uint64_t>& items,
+                              const std::vector<uint64_t>& pairs, cudaStream_t s) {
+  if (items.empty()) return cudaSuccess;
+  if (a.geom.D == 128) return launch_d<128>(a, items, pairs, s);
+  if (a.geom.D == 64) return launch_d<64>(a, items, pairs, s);
   return cudaErrorInvalidValue;
 }
 

@@ -1,7 +1,7 @@
 """Prefill calls small enough that clusters of two CTAs share each work item,
-around the rule's edges (four visited tiles, 76 items), against the oracle: odd
-lengths, a cached prefix, streaming heads whose halves see no key of some rows,
-the chunk-eviction rule."""
+around the rule's edges (four visited tiles, 76 items), and larger ones whose last
+wave is shared, against the oracle: odd lengths, a cached prefix, streaming heads
+whose halves see no key of some rows, the chunk-eviction rule."""
 
 import numpy as np
 import pytest
@@ -47,4 +47,35 @@ def test_after_a_cached_prefix(d, rule):
     want = oatt.prefill(qn, kn, vn, labels, S, W, **kw)
     mag = oatt.prefill(qn, kn, np.abs(vn), labels, S, W, **kw)
     assert_matches(np.concatenate(got), want, "two chunks", mag)
+    cache.close()
+
+
+@pytest.mark.parametrize("d,B,Hq,Hkv,light,T,prefix", [
+    (128, 20, 8, 1, 0, 256, 1280),   # 160 items: the 8 past the first wave are shared
+    (64, 33, 7, 1, 1, 200, 2048),    # 231: 76 shared, then three light ones and an entry without work
+    (128, 3, 32, 4, 0, 300, 1500),   # 192 items in two tiles a sequence, a wave of whole ones first
+    (128, 4, 25, 5, 1, 250, 2999),   # 100: the 75 heavy ones and one light one shared
+])
+def test_last_wave_shared(d, B, Hq, Hkv, light, T, prefix):
+    """Chunks after a long prefix whose last wave of items is shared; `light`
+    sequences have a prefix of one token."""
+    ensure_lib()
+    labels, S, W = [0] * Hkv, 4, 60
+    pk, pv, k, v = (randn_bf16((B, n, Hkv, d), 50 + i, "cuda") for i, n in enumerate((prefix, prefix, T, T)))
+    q = randn_bf16((B, T, Hq, d), 60, "cuda")
+    before = [prefix] * (B - light) + [1] * light
+    lens = [T - b % 3 for b in range(B)]
+    cache = aoh.Cache(B, Hq, Hkv, d, prefix + T, S, W, labels)
+    cache.prefill(None, pk, pv, seq_lens=before)
+    out = torch.full_like(q, float("nan"))
+    cache.prefill(q, k, v, out, seq_lens=lens)
+    cache.check()
+    for b in sorted({0, 152 // Hq, 228 // Hq, B - 1} & set(range(B))):
+        n = before[b] + lens[b]
+        rows = np.arange(before[b], n)
+        kn, vn = (np.concatenate([f64(x[b, :before[b]]), f64(y[b, :lens[b]])]) for x, y in ((pk, k), (pv, v)))
+        qn = np.concatenate([np.zeros((before[b], Hq, d)), f64(q[b, :lens[b]])])
+        want = oatt.prefill(qn, kn, vn, labels, S, W, rows=rows)
+        mag = oatt.prefill(qn, kn, np.abs(vn), labels, S, W, rows=rows)
+        assert_matches(f64(out[b, :lens[b]]), want, f"b={b}", mag)
     cache.close()

@@ -36,17 +36,21 @@ __device__ __forceinline__ int seq_len(const DecodeArgs& a, int b, const int* le
 // (the allocation-free entry point, e.g. replayed from a CUDA graph).
 __device__ __forceinline__ bool seq_full(const CacheGeom& g, int t) { return g.n_r > 0 && t >= g.max_seq; }
 
-// Rows of item `id`. Retrieval: t + 1 rows (min(top_k, t + 1) borrowed rows
-// in the H2Share reuse step); streaming: min(t + 1, S + W) ring rows;
-// t = tokens held before this step. 0 for every item of a full sequence.
-__device__ __forceinline__ int item_rows(const DecodeArgs& a, int id, const int* lens_s = nullptr) {
+// Rows of item `id`, item k of sequence b. Retrieval: t + 1 rows (min(top_k,
+// t + 1) borrowed rows in the H2Share reuse step); streaming: min(t + 1, S + W)
+// ring rows; t = tokens held before this step. 0 for every item of a full
+// sequence.
+__device__ __forceinline__ int item_rows(const DecodeArgs& a, int b, int k, const int* lens_s) {
   const CacheGeom& g = a.geom;
-  const int HK = g.n_r + g.n_s;
-  const int b = id / HK, k = id - b * HK;
   const int t = seq_len(a, b, lens_s);
   if (seq_full(g, t)) return 0;
   if (k < g.n_r) return a.idx ? min(a.top_k, t + 1) : t + 1;
   return min(t + 1, g.S + g.W);
+}
+__device__ __forceinline__ int item_rows(const DecodeArgs& a, int id, const int* lens_s = nullptr) {
+  const int HK = a.geom.n_r + a.geom.n_s;
+  const int b = id / HK;
+  return item_rows(a, b, id - b * HK, lens_s);
 }
 
 // Rows as the split counts them: a.row_keys cache rows each (2 where the
@@ -425,7 +429,8 @@ __device__ __forceinline__ void finish_launch(const DecodeArgs& a, const int* le
 constexpr int kClusterItems = 32;  // most items of a step on this split
 constexpr int kClusterMax = 16;    // most CTAs of a cluster
 // words of the plan in shared memory
-constexpr int kPlanItem = 0, kPlanFlag = 1, kPlanLo = 2, kPlanHi = 3, kPlanParts = 4, kPlanFirst = 5, kPlanKeys = 6;
+constexpr int kPlanItem = 0, kPlanFlag = 1, kPlanLo = 2, kPlanHi = 3, kPlanParts = 4, kPlanFirst = 5, kPlanKeys = 6,
+              kPlanSeq = 7;
 
 // Receive buffer: [C] values of the share, then [C][G] (m, l).
 __host__ __device__ constexpr int recv_floats(int G, int D) { return G * D + 2 * kClusterMax * G; }
@@ -436,51 +441,80 @@ __host__ __device__ constexpr int recv_floats(int G, int D) { return G * D + 2 *
 // between an even share and one that always fits is taken. Up to 8 tiles a
 // CTA, T and the CTA's rows are whole tiles (a started tile costs as much as a
 // full one); above that an equal share is better.
-__device__ __forceinline__ void plan_clusters(const DecodeArgs& a, const int* lens_s, int tile, int* plan) {
+//
+// Nothing is loaded before the plan is known, so its latency is part of every
+// step: what does not need the lengths is formed before the wait for the
+// previous kernel (PlanSetup), clusters are powers of two (shifts), the bounds of T
+// come from reciprocals (a T that does not fit is found out below), and the
+// division of a CTA's rows is left out where an item has one cluster: 1,600 clocks
+// for 4 items, 2,600 with integer divisions throughout.
+struct PlanSetup {
+  int lg, nc, c, rank;  // log2 of a cluster's CTAs; clusters; this CTA's cluster and place in it
+  int b, k;             // lane i: item i
+  float inv_nc;
+  __device__ __forceinline__ explicit PlanSetup(const CacheGeom& g) {
+    const int HK = g.n_r + g.n_s, lane = threadIdx.x & 31;
+    lg = __ffs((int)cluster_ctas()) - 1;
+    nc = (int)gridDim.x >> lg;
+    c = (int)blockIdx.x >> lg;
+    rank = (int)cluster_rank();
+    // lane / HK: both at most 64, so the half keeps the quotient clear of rounding
+    b = (int)(((float)lane + 0.5f) * __frcp_rn((float)HK));
+    k = lane - b * HK;
+    inv_nc = __frcp_rn((float)nc);
+  }
+};
+
+__device__ __forceinline__ void plan_clusters(const DecodeArgs& a, const PlanSetup& ps, const int* lens_s, int tile,
+                                              int* plan) {
   constexpr unsigned kAll = 0xffffffffu;
   const CacheGeom& g = a.geom;
   const int n_items = g.B * (g.n_r + g.n_s);
-  const int lane = threadIdx.x & 31;
-  const int C = (int)cluster_ctas(), nc = (int)gridDim.x / C, c = (int)blockIdx.x / C;
-  const int keys = lane < n_items ? item_rows(a, lane, lens_s) : 0;
+  const int lane = threadIdx.x & 31, lg = ps.lg, C = 1 << lg, nc = ps.nc;
+  const int keys = lane < n_items ? item_rows(a, ps.b, ps.k, lens_s) : 0;
   const int rows = split_rows(a, keys);
   const int total = __reduce_add_sync(kAll, rows), most = __reduce_max_sync(kAll, rows);
   const int active = __popc(__ballot_sync(kAll, rows > 0));
-  const int lo = max(1, (total + nc - 1) / nc);
-  const int hi = max(lo, nc > active ? min(most, (total + nc - active - 1) / (nc - active)) : most);
+  const int lo = max(1, (int)((float)total * ps.inv_nc));
+  const int hi = max(lo, nc > active ? min(most, (int)__fdividef((float)total * 1.000001f, (float)(nc - active)) + 1) : most);
   int T = lane == 31 ? hi : lo + (hi - lo) / 31 * lane;
-  const int unit = tile * C;
-  if (T <= 8 * unit) T = (T + unit - 1) / unit * unit;
+  const int unit = tile * C;  // a power of two
+  if (T <= 8 * unit) T = (T + unit - 1) & ~(unit - 1);
   // ceil(r / t); the half row keeps exact multiples clear of the rounding
   auto clusters = [](int r, int t, float rc) { return r > 0 ? max(1, (int)(((float)(r + t) - 0.5f) * rc)) : 0; };
-  const float rc = 1.f / (float)T;
+  const float rc = __fdividef(1.f, (float)T);
   int need = 0;
+#pragma unroll 4
   for (int j = 0; j < n_items; ++j) need += clusters(__shfl_sync(kAll, rows, j), T, rc);
   const unsigned fits = __ballot_sync(kAll, need <= nc);
   const int pick = fits ? __ffs(fits) - 1 : 0;
   const int Tp = __shfl_sync(kAll, T, pick);
-  const int n = fits ? clusters(rows, Tp, 1.f / (float)Tp) : (rows > 0 ? 1 : 0);
+  const float rcp = __shfl_sync(kAll, rc, pick);
+  const int n = fits ? clusters(rows, Tp, rcp) : (rows > 0 ? 1 : 0);
   int inc = n;
 #pragma unroll
   for (int o = 1; o < 32; o <<= 1) {
+    if (o >= n_items) break;
     const int y = __shfl_up_sync(kAll, inc, o);
     if (lane >= o) inc += y;
   }
-  const unsigned past = __ballot_sync(kAll, inc > c);
+  const unsigned past = __ballot_sync(kAll, lane < n_items && inc > ps.c);
   const int item = past ? __ffs(past) - 1 : n_items;
   const int src = item < 32 ? item : 31;
   const int first = __shfl_sync(kAll, inc - n, src), parts = __shfl_sync(kAll, n, src);
-  const int r = __shfl_sync(kAll, rows, src), rk = __shfl_sync(kAll, keys, src);
+  const int r = __shfl_sync(kAll, rows, src), rk = __shfl_sync(kAll, keys, src), rb = __shfl_sync(kAll, ps.b, src);
   if (lane == 0) {
     plan[kPlanItem] = item;
     plan[kPlanParts] = parts;
     plan[kPlanFirst] = first * C;
     plan[kPlanKeys] = rk;
+    plan[kPlanSeq] = rb;
     int l = 0, h = 0;
     if (item < n_items) {
-      int per = (r + parts * C - 1) / (parts * C);
-      if (per <= 8 * tile) per = (per + tile - 1) / tile * tile;
-      const int q = (c - first) * C + (int)cluster_rank();
+      int per = (r + C - 1) >> lg;
+      if (parts > 1) per = (int)((unsigned)(per + parts - 1) / (unsigned)parts);
+      if (per <= 8 * tile) per = (per + tile - 1) & ~(tile - 1);
+      const int q = (ps.c - first) * C + ps.rank;
       l = (int)min((long long)r, (long long)q * per);
       h = (int)min((long long)r, (long long)l + per);
     }
@@ -528,7 +562,7 @@ template <int G, int D, int NT>
 __device__ __forceinline__ void cluster_finish(const DecodeArgs& a, const float* recv, int* plan, __nv_bfloat16* out,
                                                float2* stats) {
   const int C = (int)cluster_ctas(), me = (int)cluster_rank(), t = threadIdx.x;
-  const int share = G * D / C, e0 = me * share;
+  const int share = G * D >> (__ffs(C) - 1), e0 = me * share;
   const float2* ml = reinterpret_cast<const float2*>(recv + G * D);
   const int parts = plan[kPlanParts], first = plan[kPlanFirst];
   float* mine = partial_slot(a, (int)blockIdx.x, 0, G, D);
@@ -539,19 +573,25 @@ __device__ __forceinline__ void cluster_finish(const DecodeArgs& a, const float*
   };
   for (int i = 2 * t; i < share; i += 2 * NT) {
     const int e = e0 + i, h = e / D;
-    float M = -INFINITY;
-    for (int c = 0; c < C; ++c) M = fmaxf(M, ml[c * G + h].x);
-    float L = 0.f;
+    // all loads at once, past C as states that weigh nothing
+    float2 st[kClusterMax], x[kClusterMax];
+#pragma unroll
+    for (int c = 0; c < kClusterMax; ++c) {
+      st[c] = c < C ? ml[c * G + h] : make_float2(-INFINITY, 0.f);
+      x[c] = c < C ? *reinterpret_cast<const float2*>(recv + c * share + i) : make_float2(0.f, 0.f);
+    }
+    float M = st[0].x, L = 0.f;
+#pragma unroll
+    for (int c = 1; c + 1 < kClusterMax; c += 2) M = fmax3f(M, st[c].x, st[c + 1].x);
+    M = fmaxf(M, st[kClusterMax - 1].x);
     float2 o = make_float2(0.f, 0.f);
-#pragma unroll 4
-    for (int c = 0; c < C; ++c) {
-      const float2 s = ml[c * G + h];
-      if (s.x == -INFINITY) continue;
-      const float w = fast_exp2(s.x - M);
-      const float2 x = *reinterpret_cast<const float2*>(recv + c * share + i);
-      L += w * s.y;
-      o.x += w * x.x;
-      o.y += w * x.y;
+#pragma unroll
+    for (int c = 0; c < kClusterMax; ++c) {
+      const bool any = st[c].x != -INFINITY;  // else its values were never written
+      const float w = any ? fast_exp2(st[c].x - M) : 0.f;
+      L += w * st[c].y;
+      o.x += any ? w * x[c].x : 0.f;
+      o.y += any ? w * x[c].y : 0.f;
     }
     if (parts == 1) {
       store(e, M, L, o);

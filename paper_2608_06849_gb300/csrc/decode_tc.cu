@@ -51,16 +51,19 @@ long long clusters_for(long long n, long long rows, int C, int k) {
 // length update at its end, worth about kSpared tiles (a tile is 0.8-1.4 us);
 // with more items the whole clusters fit the rows less evenly. Measured, B=1
 // and 28/4 heads of which 2 stream (S = 128, W = 2048), us a step as a layer
-// of a graph, stream-K / clusters of 2 / 4 / 8 / 16: 1K 14.9 / 9.0 / 8.5 /
-// 6.9 / 7.4, 2K 15.4 / 10.5 / 9.0 / 9.0 / 8.1, 4K 13.6 / 11.6 / 9.5 / 9.1 /
-// 9.5, 16K 18.9 / 15.5 / 13.0 / 12.6 / 13.4, 32K 19.2 / 18.5 / 15.0 / 15.0 /
-// 18.7, 128K 36.1 / 35.0 / 33.4 / 34.3 / 43.6, 256K 55.3 / 54.2 / 52.5 / 56.0 /
-// 75.1; B=4, 16 items: 1K 15.9 / 9.7 / 9.0 / - / -, 16K 27.0 / 22.7 / 22.0; B=4,
-// 32 items: 1K 18.2 / 11.1 / 9.7, 4K 17.0 / 15.7 / 17.4, 16K 34.6 / 34.1 / 40.7.
+// of a graph, stream-K / clusters of 2 / 4 / 8 / 16: 1K 13.9 / 8.5 / 6.4 / 6.1 /
+// 6.2, 2K 13.1 / 9.5 / 7.8 / 7.7 / 6.7, 4K 12.5 / 10.5 / 8.7 / 8.2 / 7.4, 16K
+// 17.2 / 13.4 / 11.3 / 10.8 / 11.9, 32K 18.6 / 17.8 / 14.1 / 13.9 / 16.1, 128K
+// 35.1 / 34.0 / 31.4 / - / -, 256K (W = 4096) 54.0 / 52.7 / 50.2 / - / -; B=4, 16
+// items: 1K 14.3 / 9.0 / 7.0, 16K 25.6 / 20.7 / 20.5; B=4, 32/8 heads, 32 items: 1K
+// 15.6 / 10.5 / 9.0, 4K 15.9 / 14.9 / 15.3, 16K 33.0 / - / - (-: not taken, the
+// clusters that run at once do not hold the rows within kSpared tiles).
 //
-// Among the sizes: a step costs k tiles (0.8 us each here), a global exchange
-// (2 tiles) unless one cluster holds each item, and another round trip (1
-// tile) for every eight clusters of an item beyond eight. Clusters of 2 leave
+// Among the sizes and tiles a CTA: a step costs its k tiles (0.8 us each here), a
+// global exchange (1.3 us, 2 tiles) unless one cluster holds each item, and
+// another round trip (1 tile) for every eight clusters of an item beyond eight; a
+// tile more is cheaper than the exchange (4,097 rows on 16 CTAs: 9.0 us with two
+// clusters of 2 tiles, 8.7 with one of 3). Clusters of 2 leave
 // more of them to that exchange, and are taken only above 16 items, where the
 // larger sizes run out of clusters.
 void decode_tc_split(DecodeArgs& a, const CacheGeom& g, long long longest, long long total_rows, int num_sms) {
@@ -91,7 +94,6 @@ void decode_tc_split(DecodeArgs& a, const CacheGeom& g, long long longest, long 
         a.cluster = C;
         a.n_ctas = C * (int)need;
       }
-      break;
     }
   }
 }

@@ -117,7 +117,7 @@ struct Lay {
   static constexpr int OFF_KV = 0;
   static constexpr int OFF_Q = OFF_KV + kNS * kStage;
   static constexpr int OFF_P = OFF_Q + 2 * QBUF;
-  static constexpr int OFF_RED = OFF_P + NPB * PBUF;           // [2][4][16] warp maxima, [4][16] warp sums
+  static constexpr int OFF_RED = OFF_P + NPB * PBUF;           // [2][16][4] warp maxima, [4][16] warp sums
   static constexpr int OFF_MS = OFF_RED + (2 * 64 + 64) * 4;
   static constexpr int MS_FLOATS = 1024;                       // merge scratch; the odd keys' O at d_head 64
   static constexpr int OFF_BAR = OFF_MS + MS_FLOATS * 4;
@@ -174,19 +174,20 @@ struct Walk {
     return false;
   }
   __device__ __forceinline__ int keys() const { return sp.keys; }
+  __device__ __forceinline__ int seq(int HK) const { return id / HK; }
   // another item of the range may follow: it starts at its row 0
   __device__ __forceinline__ bool more() const { return off < end && id + 1 < n_items; }
 };
 // In the cluster split a CTA holds rows of one item at most (dec::ClusterPlan).
 template <>
 struct Walk<true> {
-  int id;
+  int id, b;
   bool left;
   long long item_off = 0;
   dec::Span sp;
   __device__ __forceinline__ Walk(const DecodeArgs&, const int*, int, long long, long long, int first, long long,
                                   const int* plan)
-      : id(first) {
+      : id(first), b(plan[dec::kPlanSeq]) {
     sp.keys = plan[dec::kPlanKeys];
     sp.lo = plan[dec::kPlanLo];
     sp.hi = plan[dec::kPlanHi];
@@ -198,6 +199,7 @@ struct Walk<true> {
     return r;
   }
   __device__ __forceinline__ int keys() const { return sp.keys; }
+  __device__ __forceinline__ int seq(int) const { return b; }
   __device__ __forceinline__ bool more() const { return false; }
 };
 
@@ -225,7 +227,7 @@ __global__ void __launch_bounds__(kThreads + 32 * gather_warps(G, MODE), 1)
   uint8_t* sKV = smem + C::OFF_KV;
   uint8_t* sQ = smem + C::OFF_Q;
   uint8_t* sP = smem + C::OFF_P;
-  float* red = reinterpret_cast<float*>(smem + C::OFF_RED);  // [2][4][16]
+  float* red = reinterpret_cast<float*>(smem + C::OFF_RED);  // [2][16][4]
   float* lsum = red + 2 * 64;                             // [4][16]
   float* ms = reinterpret_cast<float*>(smem + C::OFF_MS);
   uint64_t* full = reinterpret_cast<uint64_t*>(smem + C::OFF_BAR);  // [kNS] a TMA-loaded tile landed
@@ -274,6 +276,12 @@ __global__ void __launch_bounds__(kThreads + 32 * gather_warps(G, MODE), 1)
     *abort_flag = 0;
     fence_mbar_init();
   }
+  if (warp == 4 && lane == 0) {
+    if (g.n_r > 0) prefetch_tmap(&a.tcr);
+    if (g.n_s > 0) prefetch_tmap(&a.tcs);
+    if (PAIR && g.n_r > 0) prefetch_tmap(&a.tcr_odd);
+    if (PAIR && g.n_s > 0) prefetch_tmap(&a.tcs_odd);
+  }
   if (warp == 5) {
     tmem_alloc(tmem_slot, C::TMEM_COLS);
     tmem_relinquish();
@@ -282,6 +290,7 @@ __global__ void __launch_bounds__(kThreads + 32 * gather_warps(G, MODE), 1)
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = *tmem_slot;
+  const dec::PlanSetup plan_setup(g);
   // a CTA writes into its cluster's shared memory only once every CTA of it runs
   if constexpr (CLUSTER) cluster_arrive();
   // everything the previous kernels wrote (lengths, cache, inputs, counters)
@@ -297,7 +306,7 @@ __global__ void __launch_bounds__(kThreads + 32 * gather_warps(G, MODE), 1)
   }
   long long total = 0, start = 0, end = 0, first_off = 0;
   if constexpr (CLUSTER) {
-    if (warp == 0) dec::plan_clusters(a, lens_s, kBN, sh32);
+    if (warp == 0) dec::plan_clusters(a, plan_setup, lens_s, kBN, sh32);
     __syncthreads();
     cluster_wait();
   } else {
@@ -317,15 +326,11 @@ __global__ void __launch_bounds__(kThreads + 32 * gather_warps(G, MODE), 1)
     // the cache regions, 128-byte swizzle). In the reuse variant the gather
     // warps issue every tile instead (see below) and this warp idles.
     if (!GATHER && lane == 0) {
-      if (g.n_r > 0) prefetch_tmap(&a.tcr);
-      if (g.n_s > 0) prefetch_tmap(&a.tcs);
-      if (PAIR && g.n_r > 0) prefetch_tmap(&a.tcr_odd);
-      if (PAIR && g.n_s > 0) prefetch_tmap(&a.tcs_odd);
       int it = 0;
       bool ok = true;
       while (ok && walk.next()) {
         const int id = walk.id, lo = walk.sp.lo, hi = walk.sp.hi;
-        const int b = id / HK, k = id - b * HK;
+        const int b = walk.seq(HK), k = id - b * HK;
         const bool strm = k >= g.n_r;
         const int region = strm ? b * g.n_s + (k - g.n_r) : b * g.n_r + k;
         const CUtensorMap* map = strm ? &a.tcs : &a.tcr;
@@ -374,7 +379,6 @@ __global__ void __launch_bounds__(kThreads + 32 * gather_warps(G, MODE), 1)
     const uint32_t dst_lane = half * kTile + (ch >> 3) * kBox;
     const uint32_t swz = ch & 7;
     const bool loader = gw == 0 && lane == 0;  // issues the TMA tiles
-    if (loader && g.n_s > 0) prefetch_tmap(&a.tcs);
     int it = 0;
     bool ok = true;
     uint32_t fpar = 0;  // loader: bit st, parity of stage st's next full[] phase
@@ -386,7 +390,7 @@ __global__ void __launch_bounds__(kThreads + 32 * gather_warps(G, MODE), 1)
     };
     while (ok && walk.next()) {
       const int id = walk.id, lo = walk.sp.lo, hi = walk.sp.hi;
-      const int b = id / HK, k = id - b * HK;
+      const int b = walk.seq(HK), k = id - b * HK;
       if (k >= g.n_r) {
         const int region = b * g.n_s + (k - g.n_r);
         for (int row0 = lo; row0 < hi; row0 += kBN, ++it) {
@@ -516,12 +520,9 @@ __global__ void __launch_bounds__(kThreads + 32 * gather_warps(G, MODE), 1)
     uint4 nvr;
     const int ch = lane % CPR;
     const bool new_v = lane >= CPR, new_lane = lane < 2 * CPR;
-    auto kv_head_of = [&](int id) {
-      const int k = id % HK;
-      return k >= g.n_r ? (int)g.s_head[k - g.n_r] : (int)g.r_head[k];
-    };
     auto fetch_inputs = [&](int id) {
-      const int b = id / HK, kvh = kv_head_of(id);
+      const int b = CLUSTER ? walk.seq(HK) : id / HK, k = id - b * HK;
+      const int kvh = k >= g.n_r ? (int)g.s_head[k - g.n_r] : (int)g.r_head[k];
       const bf16* qg = static_cast<const bf16*>(a.q) + ((size_t)b * g.Hq + (size_t)kvh * G) * D;
 #pragma unroll
       for (int i = 0; i < QV; ++i) {
@@ -539,7 +540,7 @@ __global__ void __launch_bounds__(kThreads + 32 * gather_warps(G, MODE), 1)
 
     while (ok && walk.next()) {
       const int id = walk.id, lo = walk.sp.lo, hi = walk.sp.hi;
-      const int b = id / HK, k = id - b * HK;
+      const int b = walk.seq(HK), k = id - b * HK;
       const bool strm = k >= g.n_r;
       const int hi_idx = strm ? k - g.n_r : k;
       const int t = dec::seq_len(a, b, ls);
@@ -666,7 +667,7 @@ __global__ void __launch_bounds__(kThreads + 32 * gather_warps(G, MODE), 1)
     }
     while (ok && walk.next()) {
       const int id = walk.id, lo = walk.sp.lo, hi = walk.sp.hi;
-      const int b = id / HK, k = id - b * HK;
+      const int b = walk.seq(HK), k = id - b * HK;
       const bool strm = k >= g.n_r;
       const int kvh = strm ? g.s_head[k - g.n_r] : g.r_head[k];
 
@@ -724,27 +725,36 @@ __global__ void __launch_bounds__(kThreads + 32 * gather_warps(G, MODE), 1)
           const float r = warp_max(PAIR ? fmaxf(s[0][h], s[NK - 1][h]) : s[0][h]);
           wm = (lane == h) ? r : wm;
         }
-        if (lane < G) rx[warp * 16 + lane] = wm;
+        if (lane < G) rx[lane * 4 + warp] = wm;
         ok = named_barrier_and(1, kSoftmaxThreads, local_ok);
         if (!ok) break;
+        // one 16-byte load a head, and a single uniform branch past the first tile
         bool resc = false;
-        float alpha[G];
+        float alpha[G], tm[G];
 #pragma unroll
         for (int h = 0; h < G; ++h) {
-          const float tm = fmaxf(fmax3f(rx[h], rx[16 + h], rx[32 + h]), rx[48 + h]);
-          const float mn = fmaxf(m[h], tm);
+          const float4 w4 = *reinterpret_cast<const float4*>(rx + h * 4);
+          tm[h] = fmaxf(fmax3f(w4.x, w4.y, w4.z), w4.w);
           alpha[h] = 1.f;
-          if (mn > m[h] + kRescaleThreshold) {
-            alpha[h] = (m[h] == -INFINITY) ? 0.f : fast_exp2(m[h] - mn);
-            m[h] = mn;
-            l[h] *= alpha[h];
-            resc = true;
+          if (row0 == lo)
+            m[h] = fmaxf(m[h], tm[h]);
+          else
+            resc = resc || tm[h] > m[h] + kRescaleThreshold;
+        }
+        if (resc) {
+#pragma unroll
+          for (int h = 0; h < G; ++h) {
+            if (tm[h] > m[h] + kRescaleThreshold) {
+              alpha[h] = (m[h] == -INFINITY) ? 0.f : fast_exp2(m[h] - tm[h]);
+              m[h] = tm[h];
+              l[h] *= alpha[h];
+            }
           }
         }
         // the P buffer is free once O += P(it - NPB) V is done
         if (it >= C::NPB)
           local_ok = wait_bar(&p_free[(it - C::NPB) & 1], ((it - C::NPB) >> 1) & 1, a.err, abort_flag) && local_ok;
-        if (resc && row0 != lo) {
+        if (resc) {
           // rescale row t of O^T; O += P(it - 1) V must have landed first
           local_ok = wait_bar(&p_free[x ^ 1], ((it - 1) >> 1) & 1, a.err, abort_flag) && local_ok;
           tc_fence_after();
@@ -768,15 +778,18 @@ __global__ void __launch_bounds__(kThreads + 32 * gather_warps(G, MODE), 1)
             pr[y][h] = valid[y] ? fast_exp2(s[y][h] - m[h]) : 0.f;
             l[h] += pr[y][h];
           }
-        if (!valid[NK - 1]) {
+        if (!__all_sync(0xffffffffu, valid[NK - 1])) {
           // the tile has landed (its S is complete); zero the V rows of this
-          // thread's keys that the item does not hold (d_head 128: both halves)
+          // warp's keys that the item does not hold (d_head 128: both halves).
+          // The lanes' chunks lie side by side: each lane zeroing its own row
+          // met bank conflicts, 2,100 clocks at a step's last tile
           wait_bar(gathered ? &gfull[st] : &full[st], land_par, a.err, abort_flag);
-          uint8_t* vr = sKV + st * kStage + kTile + t * 128;
+          const int end = (warp + 1) * 32;
 #pragma unroll
-          for (int c = 0; c < 8; ++c) {
-            if (!valid[0]) reinterpret_cast<uint4*>(vr)[c] = make_uint4(0, 0, 0, 0);
-            reinterpret_cast<uint4*>(vr + kBox)[c] = make_uint4(0, 0, 0, 0);
+          for (int box = 0; box < 2; ++box) {
+            const int first = max(warp * 32, PAIR ? (kv + 1 - box) / 2 : kv);  // first row to zero
+            uint4* v4 = reinterpret_cast<uint4*>(sKV + st * kStage + kTile + box * kBox);
+            for (int c = first * 8 + lane; c < end * 8; c += 32) v4[c] = make_uint4(0, 0, 0, 0);
           }
         }
         // P^T row t -> column t of the K-major [NPV][128 rows] buffer
@@ -892,13 +905,14 @@ __global__ void __launch_bounds__(kThreads + 32 * gather_warps(G, MODE), 1)
     // every CTA's state has arrived; the waits of an aborted CTA are bounded,
     // so it comes here too
     cluster_arrive();
+    const bool any = first_id < n_items;
+    const int b = any ? walk.seq(HK) : 0, k = any ? first_id - b * HK : 0;
+    const bool strm = k >= g.n_r;
+    const int kvh = strm ? g.s_head[k - g.n_r] : g.r_head[k];
+    bf16* outp = static_cast<bf16*>(a.out) + ((size_t)b * g.Hq + (size_t)kvh * G) * D;
+    float2* st = (a.scores != nullptr && !strm) ? a.score_stats + (size_t)(b * g.n_r + k) * G : nullptr;
     cluster_wait();
-    if (warp < 4 && first_id < n_items) {
-      const int b = first_id / HK, k = first_id - b * HK;
-      const bool strm = k >= g.n_r;
-      const int kvh = strm ? g.s_head[k - g.n_r] : g.r_head[k];
-      bf16* outp = static_cast<bf16*>(a.out) + ((size_t)b * g.Hq + (size_t)kvh * G) * D;
-      float2* st = (a.scores != nullptr && !strm) ? a.score_stats + (size_t)(b * g.n_r + k) * G : nullptr;
+    if (warp < 4 && any) {
       dec::cluster_finish<G, D, kSoftmaxThreads>(a, recv, sh32, outp, st);
     }
   }

@@ -35,6 +35,21 @@ def test_split(name):
     run_case(B, Hq, Hkv, 128, T, S, W, labels, seq_lens=lens, decode_steps=2, check_prefill_out=False)
 
 
+@pytest.mark.parametrize("batch", [8, 40])  # clusters, stream-K
+def test_last_tile_of_every_warp_edge(batch, monkeypatch):
+    """A last tile of 1 to 128 rows: cache rows past it hold NaNs, which a weight
+    of zero would not hide."""
+    init = aoh.Cache.__init__
+
+    def filled(self, *args, **kw):
+        init(self, *args, **kw)
+        self.buffer.fill_(0xFF)  # every bf16 a NaN
+
+    monkeypatch.setattr(aoh.Cache, "__init__", filled)
+    lens = [(256 + r if i % 2 else r) for i, r in enumerate([30, 31, 32, 62, 63, 94, 126, 127] * (batch // 8))]
+    run_case(batch, 7, 1, 128, 400, 4, 60, [0], seq_lens=lens, decode_steps=2, check_prefill_out=False)
+
+
 def test_stream_k_two_merge_levels():
     """One item of 3.1M rows: past the length where whole clusters fit the rows
     as evenly as the stream-K split, whose 152 parts merge in two levels."""

@@ -76,44 +76,48 @@ __global__ void __launch_bounds__(256) row_exp_kernel(const bf16* wq, const bf16
 // 7-bit digits d_1 .. d_8 (a bf16 value's 8 bits fall into two neighbouring
 // digits), and digit matrices are exact in bf16, so W W^T is the sum over
 // digit pairs of D_i D_j^T 2^(-7 (i + j)). Pairs with the same i + j = c share
-// a TMEM accumulator: at most 8 pairs times 128 columns times 2^14 stay below
-// 2^24, so every fp32 accumulation is exact, and after every 128 columns the
-// accumulators are added into 64-bit integers. Products below 2^-63 of the
+// a TMEM accumulator, and before one holds more than kGramExact digit products
+// (each below 2^14) the accumulators are added into 64-bit integers: every fp32
+// accumulation is exact. Products below 2^-63 of the
 // two rows' scale (c > 9) are left out; fp64 sums round at 2^-53 of it. The
 // result rounds once, when it becomes a double.
 //
 // The 8 accumulators (c = 2 .. 9) do not fit TMEM at once, so
 // blockIdx.z = 0 takes c = 2 .. 5 (digits 1-4, 10 pairs) and 1 takes c = 6 .. 9
-// (26 pairs), each writing its own part. For 896 matrices of 128 x 3584 this
-// takes 4.8 ms, and the row exponents 0.12 ms (7.1 TB/s); the plain fp64 Gram
-// took 88.6 ms (105 GFLOP at 1.19 TFLOP/s, the fp64 pipe's two FMAs a clock
-// and SM). It is bound by the tensor cores (36 digit products of 128 x 128 x
-// 64 a step) plus the digit production, which alternate.
+// (26 pairs), each writing its own part. Four digits hold every weight down to
+// 2^-20 of its row's largest, so a step of 64 columns whose weights have no
+// digit past the fourth (nearly all) is narrow: 4 digit tiles, and 6 pairs for
+// c = 6 .. 9. Narrow steps alternate between the halves of the 8 tiles, so that
+// one's digits are formed while the other's products run.
+//
+// For 896 matrices of 128 x 3584 this takes 2.57 ms, and the row exponents 0.11 ms
+// (7.1 TB/s); with all 8 digits formed and multiplied in every step, one after the
+// other, it took 4.8 ms, and the plain fp64 Gram 88.6 ms (105 GFLOP at 1.19
+// TFLOP/s, the fp64 pipe's two FMAs a clock and SM). It is bound by the
+// digit production, about 25 instructions a weight.
 //
 // One CTA: 128 rows (one matrix at d_head 128, two at 64, whose off-diagonal
 // blocks are dropped), 512 threads. Each thread turns 16 weights of a
 // 64-column step into digits (128-byte-swizzled K-major tiles, one per digit),
-// one thread issues the step's MMAs, and the next step's weights are loaded
-// meanwhile.
+// one thread issues the step's MMAs, and the weights of the step after the next
+// are loaded meanwhile.
 constexpr int kDigits = 8;
+constexpr int kNarrow = 4;  // digits of a step without deep weights
 constexpr int kDigitTile = 128 * 64 * 2;
 constexpr int kGramTcThreads = 512;
 constexpr int kGramTcSmem = kDigits * kDigitTile + 1024;
-constexpr int kGramChunk = 128;  // columns between two reads of the accumulators
+// Digit products that an accumulator takes between two reads: 127^2 times as many
+// stay below 2^24.
+constexpr int kGramExact = 1040;
+constexpr int kGramSpan = 128;  // a split takes a multiple of these columns
 constexpr uint32_t kGramIdesc = idesc_bf16(128, 128, false);
-
-// bf16 bits of +-d, 0 <= d < 256.
-__device__ __forceinline__ uint32_t digit_bf16(uint32_t d, uint32_t sign) {
-  const float f = __uint_as_float(0x4B000000u | d) - 8388608.f;
-  return (__float_as_uint(f) >> 16) | sign;
-}
 
 __global__ void __launch_bounds__(kGramTcThreads, 1)
     gram_tc_kernel(const bf16* wq, const bf16* wk, int Hq, int Hkv, int nall, int dh, int dm, int span, int vec,
                    const int* row_exp, double* part, uint32_t* err) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = smem_raw + ((1024 - (smem_u32(smem_raw) & 1023)) & 1023);
-  __shared__ uint64_t done;
+  __shared__ uint64_t done[2];  // step n's MMAs complete on done[n & 1]
   __shared__ uint32_t tmem_slot;
   __shared__ int s_abort, col_exp[128];
   const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
@@ -121,7 +125,8 @@ __global__ void __launch_bounds__(kGramTcThreads, 1)
   const int split = blockIdx.y, high = blockIdx.z;
   const int k0 = split * span, k1 = min(dm, k0 + span);
   if (t == 0) {
-    mbar_init(&done, 1);
+    mbar_init(&done[0], 1);
+    mbar_init(&done[1], 1);
     s_abort = 0;
     fence_mbar_init();
   }
@@ -146,8 +151,8 @@ __global__ void __launch_bounds__(kGramTcThreads, 1)
       has ? reinterpret_cast<const uint16_t*>(weight_of(wq, wk, pm, Hq, Hkv, dh, dm)) + (size_t)(prow % dh) * dm
           : nullptr;
   const int pexp = col_exp[prow];
-  uint32_t w[8];
-  auto load = [&](int kc) {
+  uint32_t w[8] = {}, next[8] = {};  // this step's weights and the next one's, two a word
+  auto load = [&](int kc, uint32_t (&w)[8]) {
     const int c0 = kc + (t & 3) * 16;
 #pragma unroll
     for (int i = 0; i < 8; ++i) w[i] = 0u;
@@ -168,54 +173,73 @@ __global__ void __launch_bounds__(kGramTcThreads, 1)
         if (c0 + i < k1) w[i >> 1] |= (uint32_t)wrow[c0 + i] << ((i & 1) * 16);
     }
   };
-  const int n_dig = high ? kDigits : 4;
-  auto digits = [&]() {
+  // a weight's two digits, first | second << 8, and the place of the first
+  auto two_digits = [&](int i, int& s0) {
+    const uint32_t h = (w[i >> 1] >> ((i & 1) * 16)) & 0x7fffu;
+    const int ef = (int)(h >> 7);
+    const uint32_t mant = (h & 127u) | (ef ? 128u : 0u);
+    const int p = min(pexp - max(ef, 1), 63);  // leading bit at 2^(-1 - p)
+    s0 = (p * 37) >> 8;                         // p / 7
+    const uint32_t y = mant << (6 - (p - 7 * s0));
+    return (y >> 7) | (y & 127u) << 8;
+  };
+  uint32_t x[16];  // digits 1-4 of each weight, a byte each
+  auto first_digits = [&]() {  // whether a weight has digits past the fourth
+    uint32_t deep = 0;
+#pragma unroll
+    for (int i = 0; i < 16; ++i) {
+      int s0;
+      const uint32_t d = two_digits(i, s0);
+      x[i] = __funnelshift_lc(0u, d, 8 * s0);
+      deep |= __funnelshift_lc(d, 0u, 8 * s0);
+    }
+    return deep != 0u;
+  };
+  // four digit tiles from x: 128 + d is a bf16 value's bits 0x4300 | d, and
+  // +-(128 + d) -+ 128 is exact
+  auto emit = [&](uint8_t* tiles) {
 #pragma unroll
     for (int half = 0; half < 2; ++half) {
-      uint32_t hi[8], lo[8];
-      int s0[8];
+      uint8_t* dst = tiles + prow * 128 + (((pch + half) ^ (prow & 7)) << 4);
 #pragma unroll
-      for (int i = 0; i < 8; ++i) {
-        const uint32_t h = (w[4 * half + (i >> 1)] >> ((i & 1) * 16)) & 0xffffu;
-        const int ef = (int)((h >> 7) & 255u);
-        const uint32_t mant = (h & 127u) | (ef ? 128u : 0u);
-        const int p = min(pexp - max(ef, 1), 63);  // leading bit at 2^(-1 - p)
-        s0[i] = (p * 37) >> 8;                      // p / 7
-        const uint32_t y = mant << (6 - (p - 7 * s0[i]));
-        const uint32_t sign = h & 0x8000u;
-        hi[i] = digit_bf16(y >> 7, sign);
-        lo[i] = digit_bf16(y & 127u, sign);
-      }
-      uint8_t* dst = smem + prow * 128 + (((pch + half) ^ (prow & 7)) << 4);
-#pragma unroll
-      for (int s = 0; s < kDigits; ++s) {
-        if (s >= n_dig) break;
+      for (int s = 0; s < 4; ++s) {
         uint32_t o[4];
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
-          const uint32_t a = s == s0[2 * i] ? hi[2 * i] : s == s0[2 * i] + 1 ? lo[2 * i] : 0u;
-          const uint32_t b = s == s0[2 * i + 1] ? hi[2 * i + 1] : s == s0[2 * i + 1] + 1 ? lo[2 * i + 1] : 0u;
-          o[i] = a | (b << 16);
+          const int e = 8 * half + 2 * i;
+          const uint32_t sign = w[e >> 1] & 0x80008000u;
+          const uint32_t d = (__byte_perm(x[e], x[e + 1], s * 0x1111 + 0x4400) & 0x007f007fu) | 0x43004300u;
+          o[i] = bf16x2_fma(d, 0x3f803f80u | sign, 0xc300c300u ^ sign);
         }
         *reinterpret_cast<uint4*>(dst + s * kDigitTile) = make_uint4(o[0], o[1], o[2], o[3]);
       }
     }
   };
-  auto issue = [&](bool fresh) {  // one elected lane: the step's digit pairs
-    const uint64_t base = sdesc_sw128(smem_u32(smem), 16, 1024);
+  auto last_digits = [&]() {  // x: digits 5-8
+#pragma unroll
+    for (int i = 0; i < 16; ++i) {
+      int s0;
+      const uint32_t d = two_digits(i, s0);
+      x[i] = s0 < 4 ? __funnelshift_lc(d, 0u, 8 * s0) : __funnelshift_lc(0u, d, 8 * s0 - 32);
+    }
+  };
+  // one elected lane: the step's digit pairs; accumulators not in `started` are
+  // overwritten
+  auto issue = [&](int n_dig, const uint8_t* tiles, int started, uint64_t* bar) {
+    const uint64_t base = sdesc_sw128(smem_u32(tiles), 16, 1024);
     for (int a = 0; a < 4; ++a) {
       const int c = a + (high ? 6 : 2);
-      const int i0 = max(1, c - kDigits), i1 = min(c - 1, kDigits);
+      const int i0 = max(1, c - n_dig), i1 = min(c - 1, n_dig);
       for (int i = i0; i <= i1; ++i) {
         const uint64_t da = base + (uint32_t)((i - 1) * sdesc_step(kDigitTile));
         const uint64_t db = base + (uint32_t)((c - i - 1) * sdesc_step(kDigitTile));
 #pragma unroll
         for (int kk = 0; kk < 4; ++kk)
           tc_mma(tmem + a * 128, da + sdesc_step(kk * 32), db + sdesc_step(kk * 32), kGramIdesc,
-                 (fresh && i == i0 && kk == 0) ? 0u : 1u);
+                 (!(started >> a & 1) && i == i0 && kk == 0) ? 0u : 1u);
       }
     }
-    tc_commit(&done);
+    tc_commit(bar);
   };
 
   // accumulators: row 32 (warp % 4) + lane, columns 32 (warp / 4) .. + 31
@@ -224,7 +248,7 @@ __global__ void __launch_bounds__(kGramTcThreads, 1)
   long long acc[32];
 #pragma unroll
   for (int i = 0; i < 32; ++i) acc[i] = 0;
-  auto flush = [&]() {
+  auto flush = [&](int started) {
     if (!wanted) return;
     const uint32_t tl = tmem + ((uint32_t)((warp & 3) * 32) << 16) + cg * 32;
 #pragma unroll
@@ -235,6 +259,10 @@ __global__ void __launch_bounds__(kGramTcThreads, 1)
       tmem_ld8(tl + 256 + q * 8, v2);
       tmem_ld8(tl + 384 + q * 8, v3);
       tmem_ld_wait();
+      if (!(started >> 3)) {  // only c = 9 can be without a product
+#pragma unroll
+        for (int i = 0; i < 8; ++i) v3[i] = 0u;
+      }
 #pragma unroll
       for (int i = 0; i < 8; ++i) {
         const int a = __float2int_rn(__uint_as_float(v0[i])) * 128 + __float2int_rn(__uint_as_float(v1[i]));
@@ -245,32 +273,57 @@ __global__ void __launch_bounds__(kGramTcThreads, 1)
   };
 
   int step = 0;
-  bool ok = true;
-  load(k0);
+  int started = 0, taken = 0;  // accumulators with products since the last flush, and the most of one
+  bool ok = true, wide_before = false;
+  auto wait_step = [&](int n) {
+    ok = __all_sync(0xffffffffu, wait_bar(&done[n & 1], (n >> 1) & 1, err, &s_abort)) && ok;
+    tc_fence_after();
+  };
+  load(k0, w);
+  load(k0 + 64, next);
   for (int kc = k0; kc < k1; kc += 64, ++step) {
-    const bool fresh = (step * 64) % kGramChunk == 0;
-    if (step > 0) {
-      ok = wait_bar(&done, (step - 1) & 1, err, &s_abort);  // the digit tiles are free
-      tc_fence_after();
-      ok = __all_sync(0xffffffffu, ok);
-      if (ok && fresh) flush();
+    const bool deep = first_digits();
+    const bool wide = high && __syncthreads_or(deep);
+    // all 8 tiles (wide), or the half that step - 2 used
+    uint8_t* tiles = smem + (wide ? 0 : (step & 1) * kNarrow * kDigitTile);
+    const bool all_done = wide || wide_before;
+    if (step > 0 && all_done)
+      wait_step(step - 1);
+    else if (step > 1)
+      wait_step(step - 2);
+    if (ok) {
+      emit(tiles);
+      if (wide) {
+        last_digits();
+        emit(tiles + kNarrow * kDigitTile);
+      }
     }
-    if (ok) digits();
-    if (kc + 64 < k1) load(kc + 64);
+#pragma unroll
+    for (int i = 0; i < 8; ++i) w[i] = next[i];
+    load(kc + 128, next);
+    const int products = 64 * (wide ? 8 : high ? 3 : 4);  // of the pair sum with the most pairs
+    if (taken + products > kGramExact) {
+      if (!all_done) wait_step(step - 1);
+      if (ok) flush(started);
+      started = taken = 0;
+    }
+    taken += products;
+    wide_before = wide;
     fence_proxy_async_smem();
     tc_fence_before();
     ok = __syncthreads_and(ok);
     if (!ok) break;
     if (warp == 0) {
       tc_fence_after();
-      if (elect_one()) issue(fresh);
+      if (elect_one()) issue(wide ? kDigits : kNarrow, tiles, started, &done[step & 1]);
     }
     __syncwarp();
+    started |= high && !wide ? 7 : 15;
   }
   if (step > 0) {  // every issued MMA ends before TMEM is freed
-    ok = drain_wait(&done, (step - 1) & 1, err) && ok;
+    ok = drain_wait(&done[(step - 1) & 1], ((step - 1) >> 1) & 1, err) && ok;
     tc_fence_after();
-    if (__all_sync(0xffffffffu, ok)) flush();
+    if (__all_sync(0xffffffffu, ok)) flush(started);
   }
   const int m = blockIdx.x * per + row / dh;
   if (wanted && m < nall) {
@@ -691,7 +744,7 @@ extern "C" aoh_status aoh_classify(const void* w_q, const void* w_k, int32_t n_l
   int nsplit = (sms + groups - 1) / groups;
   nsplit = std::max(1, std::min(nsplit, std::max(1, d_model / 256)));
   nsplit = std::min(nsplit, 16);
-  const int span = ((d_model + nsplit - 1) / nsplit + kGramChunk - 1) / kGramChunk * kGramChunk;
+  const int span = ((d_model + nsplit - 1) / nsplit + kGramSpan - 1) / kGramSpan * kGramSpan;
   nsplit = (d_model + span - 1) / span;
   const int nparts = 2 * nsplit;
   const size_t n2 = (size_t)dh * dh;

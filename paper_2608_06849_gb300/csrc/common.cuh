@@ -188,6 +188,13 @@ __device__ __forceinline__ float fast_exp2(float x) {
   return y;
 }
 
+// a * b + c of two bf16 pairs.
+__device__ __forceinline__ uint32_t bf16x2_fma(uint32_t a, uint32_t b, uint32_t c) {
+  uint32_t r;
+  asm("fma.rn.bf16x2 %0, %1, %2, %3;" : "=r"(r) : "r"(a), "r"(b), "r"(c));
+  return r;
+}
+
 // max(a, b, c) in one instruction (three-input max.f32, sm_100 and later).
 __device__ __forceinline__ float fmax3f(float a, float b, float c) {
   float d;

@@ -222,3 +222,23 @@ def test_gram_digits_at_column_edges(dh, dm, offset):
 
     _, er = aoh.aoh_classify(place(wq), place(wk), Hkv, 50)
     np.testing.assert_allclose(er, _er_by_svd(wq, wk), rtol=1e-10)
+
+
+@pytest.mark.parametrize("dh,dm,deep", [(128, 1024, [0]), (128, 1152, [3, 4, 9, 17]), (64, 900, [14]),
+                                        (128, 3584, list(range(1, 56, 3)))])
+def test_gram_steps_with_and_without_deep_digits(dh, dm, deep):
+    """64-column steps in `deep` hold weights down to 2^-50 of the row's largest
+    (all 8 digits), the others down to 2^-20 of it (4 digits), the last bit of
+    the fourth included. Bound as in test_gram_digits_at_column_edges."""
+    ensure_lib()
+    rng = np.random.default_rng(dm + len(deep))
+    Hq, Hkv = 3, 1
+    wq, wk = (_bf16(rng.choice([-1.0, 1.0], size=(h, dh, dm)) * rng.uniform(1.0, 2.0, size=(h, dh, dm))
+                    * 2.0 ** -rng.integers(0, 21, size=(h, dh, dm))) for h in (Hq, Hkv))
+    for x in (wq, wk):
+        x[:, :, dm // 2] = 1.9921875  # the row's largest: bits 1 to 8
+        x[:, 0, 5] = 1.9921875 * 2.0 ** -20  # bits 21 to 28
+        for s in deep:
+            x[:, ::3, 64 * s:64 * s + 2] *= 2.0 ** -30
+    _, er = aoh.aoh_classify(_dev(wq), _dev(wk), Hkv, 50)
+    np.testing.assert_allclose(er, _er_by_svd(wq, wk), rtol=1e-10)

@@ -63,16 +63,24 @@ aoh_status check_config(const aoh_config* cfg, const uint8_t* labels, int* n_r, 
   return AOH_OK;
 }
 
-// Prefill work: one item per (b, query head, pair of 128-row query tiles),
-// heaviest first so the hardware block scheduler fills the machine
-// longest-processing-time first. The cost, the number of 128-key tiles visited,
-// is the same for all heads of a kind, so (b, pair, kind) entries are sorted and
-// then expanded into heads. *costs receives each item's cost.
+// Prefill work: items of two 128-row query tiles, heaviest first so the
+// hardware block scheduler fills the machine longest-processing-time first. An
+// item is one query tile of two heads of a group, or, for the last head of an
+// odd group, two consecutive tiles of that head. Two heads see the same keys;
+// two tiles visit the union of their KV tiles, so that each pair of tiles has one
+// KV tile that the first does not see, and a sequence's last pair may lack the
+// second: 8 ragged sequences of up to 2,999 tokens, 32/8 heads of 128 of which
+// half stream (S = 64, W = 512), 298 -> 277 us; 32K tokens of 28/4 streaming heads
+// (S = 128, W = 1024) 517 -> 480, 32K with half of them retrieval 2504 -> 2468.
+// The cost, the number of KV tiles visited, is the same for all items of a kind,
+// so (b, index, kind) entries are sorted and then expanded. *costs receives each
+// item's cost.
 std::vector<uint64_t> prefill_schedule(const CacheGeom& g, const std::vector<int32_t>& base,
                                        const std::vector<int32_t>& lens, std::vector<int>* costs) {
-  constexpr int BM = 256, BN = 128;
+  constexpr int BM = 128, BN = 128;
   struct Entry {
-    int cost, b, pair, streaming;
+    int cost, b, index;
+    bool streaming, two_heads;
   };
   std::vector<Entry> entries;
   for (int b = 0; b < g.B; ++b) {
@@ -81,30 +89,36 @@ std::vector<uint64_t> prefill_schedule(const CacheGeom& g, const std::vector<int
     for (int streaming = 0; streaming < 2; ++streaming) {
       if ((streaming ? g.n_s : g.n_r) == 0) continue;
       const int n_c = Lb == 0 ? 0 : ((streaming ? std::min(Lb, g.S + g.W) : Lb) + BN - 1) / BN;
-      for (int q0 = 0; q0 < lens[b]; q0 += BM) {
-        const int q_end = std::min(q0 + BM, (int)lens[b]);
-        int n;
-        if (!streaming) {
-          n = (q_end + BN - 1) / BN;
-        } else {
-          const int a_end = (std::min(std::max(S_rel, 0), q_end) + BN - 1) / BN;
-          const int c_begin = std::max(a_end, std::max(0, g.wstart(q0)) / BN);
-          const int c_end = std::max(c_begin, (q_end + BN - 1) / BN);
-          n = a_end + (c_end - c_begin);
+      for (int two_heads = 0; two_heads < 2; ++two_heads) {
+        if ((two_heads ? g.G / 2 : g.G % 2) == 0) continue;
+        const int rows = two_heads ? BM : 2 * BM;
+        for (int q0 = 0; q0 < lens[b]; q0 += rows) {
+          const int q_end = std::min(q0 + rows, (int)lens[b]);
+          int n;
+          if (!streaming) {
+            n = (q_end + BN - 1) / BN;
+          } else {
+            const int a_end = (std::min(std::max(S_rel, 0), q_end) + BN - 1) / BN;
+            const int c_begin = std::max(a_end, std::max(0, g.wstart(q0)) / BN);
+            const int c_end = std::max(c_begin, (q_end + BN - 1) / BN);
+            n = a_end + (c_end - c_begin);
+          }
+          entries.push_back({n_c + n, b, q0 / rows, streaming != 0, two_heads != 0});
         }
-        entries.push_back({n_c + n, b, q0 / BM, streaming});
       }
     }
   }
   std::stable_sort(entries.begin(), entries.end(), [](const Entry& x, const Entry& y) { return x.cost > y.cost; });
   std::vector<uint64_t> items;
-  items.reserve(entries.size() * (size_t)g.Hq);
-  costs->reserve(entries.size() * (size_t)g.Hq);
+  const size_t most = entries.size() * (size_t)(g.Hq / 2 + g.Hkv);
+  items.reserve(most);
+  costs->reserve(most);
   for (const Entry& e : entries)
     for (int i = 0; i < (e.streaming ? g.n_s : g.n_r); ++i) {
       const int kvh = e.streaming ? g.s_head[i] : g.r_head[i];
-      for (int h = kvh * g.G; h < (kvh + 1) * g.G; ++h) {
-        items.push_back(prefill_item(e.b, h, e.pair));
+      const int first = e.two_heads ? 0 : g.G - 1, step = e.two_heads ? 2 : 1;
+      for (int h = first; h + step <= g.G; h += step) {
+        items.push_back(prefill_item(e.b, kvh * g.G + h, e.index) | (e.two_heads ? kPrefillTwoHeads : 0));
         costs->push_back(e.cost);
       }
     }
@@ -230,8 +244,8 @@ cudaError_t reserve_work(aoh_cache* h, size_t n) {
   return e;
 }
 
-// Work items of a prefill call whose chunks hold up to `tokens` rows: one per
-// (sequence, query head, 256-row pair of query tiles).
+// Work items of a prefill call whose chunks hold up to `tokens` rows, at most: 256
+// rows of a head each, or 128 of two.
 size_t work_items_for(const CacheGeom& g, long long tokens) {
   return (size_t)g.B * g.Hq * (size_t)((tokens + 255) / 256);
 }

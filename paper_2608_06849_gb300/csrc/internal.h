@@ -157,7 +157,10 @@ struct PrefillTcArgs {
 cudaError_t launch_wait_selftest(uint32_t* err, uint64_t limit_ns, unsigned long long* elapsed_ns, cudaStream_t s);
 
 // A prefill work item: sequence b, query head h, rows 256 pair .. 256 pair + 255.
-inline uint64_t prefill_item(int b, int h, int pair) { return (uint64_t)b << 34 | (uint64_t)h << 24 | (uint32_t)pair; }
+inline uint64_t prefill_item(int b, int h, int index) { return (uint64_t)b << 34 | (uint64_t)h << 24 | (uint32_t)index; }
+// An item of 128 rows of heads h and h + 1 (the 128 index-th), instead of 256 rows
+// of head h (the 256 index-th).
+constexpr uint64_t kPrefillTwoHeads = 1ull << 62;
 // A half of an item that a cluster's two CTAs share, and an entry without work.
 constexpr uint64_t kPrefillHalf = 1ull << 63, kPrefillNone = ~0ull;
 // Work items that travel as kernel arguments (32 KB of them at most).

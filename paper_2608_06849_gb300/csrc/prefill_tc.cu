@@ -6,12 +6,12 @@
 // slots) before the chunk's own keys; the cache is appended after this
 // kernel, so the ring still holds the positions the chunk's rows need.
 //
-// One CTA computes two consecutive 128-row query tiles (A = rows q0..q0+127,
-// B = rows q0+128..q0+255) of one query head against the same stream of
-// 128-key K/V tiles. The KV tiles visited come from a per-head schedule: a
+// One CTA computes two 128-row query tiles (A, B) against the same stream of
+// 128-key K/V tiles: the same rows of two heads of a group, or two consecutive
+// tiles of one head. The KV tiles visited come from a per-head schedule: a
 // retrieval head visits tiles 0 .. causal end; a streaming head only the
 // tiles holding its S sinks and the tiles that intersect the W-token window
-// of some row, so its cost is O(S + W) per row instead of O(T). Both query
+// of some row, so its cost is O(S + W) per row instead of O(T). Consecutive
 // tiles visit the union of their tile sets; a tile hidden from every row of
 // one query tile contributes zero weights there. Tiles fully visible to every
 // row of a query tile skip the mask.
@@ -245,7 +245,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     const int x = (warp - 2) >> 2;        // 0: tile A (warps 2-5), 1: tile B (warps 6-9)
     const int q4 = warp & 3;              // TMEM lane quarter this warp may access
     const int r = q4 * 32 + lane;
-    const int qx0 = t.q0 + x * kBM;       // first row of this query tile
+    const int qx0 = t.row0(x);            // first row of this query tile
     const int i = qx0 + r;
     const uint32_t tl = tmem + ((uint32_t)(q4 * 32) << 16);
     const uint32_t s_col = x * 128, o_col = 256 + x * D;
@@ -268,7 +268,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     } else if (ok && __all_sync(0xffffffffu, wait_bar(&pv_done[x], (n_tiles - 1) & 1, a.err, abort_flag))) {
       tc_fence_after();
       // Q_X is free: the last S_X was done before the last P V
-      store_o<D>(a, t, qx0 + q4 * 32, tl + o_col, 1.f / l, sQ + x * C::QBYTES + q4 * (C::QBYTES / 4), lane);
+      store_o<D>(a, t, x, qx0 + q4 * 32, tl + o_col, 1.f / l, sQ + x * C::QBYTES + q4 * (C::QBYTES / 4), lane);
     }
   }
 
@@ -330,7 +330,7 @@ __global__ void __launch_bounds__(kThreads, 1)
           put_row<D>(stage, lane, c * 4 + e / 8, y);
         }
       }
-      write_rows<D>(a, t, t.q0 + x * kBM + q4 * 32, stage, lane);
+      write_rows<D>(a, t, x, t.row0(x) + q4 * 32, stage, lane);
       tc_fence_before();
     }
     __syncthreads();

@@ -52,23 +52,26 @@ struct WorkList {
   uint64_t item[CAP > 0 ? CAP : 1];
 };
 
-// A work item: query rows q0 .. q0 + 255 of query head h of sequence b, and the
-// KV tiles it visits: the n_c tiles of cached rows, then chunk tiles [0, a_end)
-// and [c_begin, c_end).
+// A work item: two query tiles of sequence b, 0 and 1 (A and B), and the KV tiles
+// they visit: the n_c tiles of cached rows, then chunk tiles [0, a_end)
+// and [c_begin, c_end). Rows q0 .. q0 + 127 of heads h and h + 1, or rows q0 ..
+// q0 + 255 of head h.
 struct Item {
   int b, h, kvh, q0, len, Lb, S_rel, n_c, a_end, c_begin, c_end;
-  bool streaming;
+  bool streaming, two_heads;
   __device__ __forceinline__ Item(const PrefillTcArgs& a, uint64_t code) {
     const CacheGeom& g = a.geom;
+    two_heads = (code & kPrefillTwoHeads) != 0;
+    code &= ~kPrefillTwoHeads;
     b = (int)(code >> 34);
     h = (int)(code >> 24) & 1023;
-    q0 = (int)(code & 0xffffffu) * 2 * kBM;
+    q0 = (int)(code & 0xffffffu) * (two_heads ? kBM : 2 * kBM);
     kvh = h / g.G;
     streaming = g.kind[kvh] != 0;
     const int2 chunk = a.chunk.of(b);
     len = chunk.x;
     Lb = chunk.y;
-    const int q_end = min(q0 + 2 * kBM, len);
+    const int q_end = min(q0 + (two_heads ? kBM : 2 * kBM), len);
     S_rel = g.S - Lb;
     n_c = Lb == 0 ? 0 : ((streaming ? min(Lb, g.S + g.W) : Lb) + kBN - 1) / kBN;
     if (!streaming) {
@@ -80,6 +83,9 @@ struct Item {
       c_end = max(c_begin, (q_end + kBN - 1) / kBN);
     }
   }
+  // query tile x: its first row and its head
+  __device__ __forceinline__ int row0(int x) const { return two_heads ? q0 : q0 + x * kBM; }
+  __device__ __forceinline__ int head(int x) const { return two_heads ? h + x : h; }
   __device__ __forceinline__ int tiles() const { return n_c + a_end + (c_end - c_begin); }
   // visited tile i: the chunk tile, for i >= n_c
   __device__ __forceinline__ int chunk_tile(int i) const { return i - n_c < a_end ? i - n_c : c_begin + (i - n_c - a_end); }
@@ -115,7 +121,7 @@ __device__ __forceinline__ void load_q(const PrefillTcArgs& a, const Item& t, in
   using C = PfCfg<D>;
   mbar_arrive_expect_tx(bar, C::QBYTES);
   for (int db = 0; db < C::DBLK; ++db)
-    tma_load_4d(dst + db * C::BOX, &a.tq, db * 64, t.h, t.q0 + x * kBM, t.b, bar);
+    tma_load_4d(dst + db * C::BOX, &a.tq, db * 64, t.head(x), t.row0(x), t.b, bar);
 }
 
 // Zero the rows of a landed V tile past its valid keys; one warp.
@@ -354,13 +360,15 @@ __device__ __forceinline__ void put_row(uint8_t* stage, int lane, int chunk, con
   *reinterpret_cast<uint4*>(stage + lane * (D * 2) + ((chunk ^ (lane % CH)) << 4)) = w;
 }
 
-// Rows i0 .. i0 + 31 of the chunk (those below len) from the warp's `stage`.
+// Rows i0 .. i0 + 31 of the chunk (those below len), query tile x's head, from the
+// warp's `stage`.
 template <int D>
-__device__ __forceinline__ void write_rows(const PrefillTcArgs& a, const Item& t, int i0, const uint8_t* stage, int lane) {
+__device__ __forceinline__ void write_rows(const PrefillTcArgs& a, const Item& t, int x, int i0, const uint8_t* stage,
+                                           int lane) {
   constexpr int CH = D / 8, RPI = 32 / CH;  // chunks a row, rows a step
   __syncwarp();
   const int c = lane % CH;
-  bf16* out = static_cast<bf16*>(a.out) + ((size_t)t.b * a.T * a.geom.Hq + t.h) * D + c * 8;
+  bf16* out = static_cast<bf16*>(a.out) + ((size_t)t.b * a.T * a.geom.Hq + t.head(x)) * D + c * 8;
 #pragma unroll
   for (int r0 = 0; r0 < 32; r0 += RPI) {
     const int r = r0 + lane / CH;
@@ -369,10 +377,10 @@ __device__ __forceinline__ void write_rows(const PrefillTcArgs& a, const Item& t
   }
 }
 
-// Write a warp's 32 finished rows of O (each lane's times its inv), the first of
-// them row i0 of the chunk. taddr: O's first column, stage: 32 * D * 2 bytes.
+// Write a warp's 32 finished rows of query tile x's O (each lane's times its inv), the
+// first of them row i0 of the chunk. taddr: O's first column, stage: 32 * D * 2 bytes.
 template <int D>
-__device__ __forceinline__ void store_o(const PrefillTcArgs& a, const Item& t, int i0, uint32_t taddr, float inv,
+__device__ __forceinline__ void store_o(const PrefillTcArgs& a, const Item& t, int x, int i0, uint32_t taddr, float inv,
                                         uint8_t* stage, int lane) {
 #pragma unroll
   for (int c = 0; c < D / 32; ++c) {
@@ -387,7 +395,7 @@ __device__ __forceinline__ void store_o(const PrefillTcArgs& a, const Item& t, i
       put_row<D>(stage, lane, c * 4 + e / 8, y);
     }
   }
-  write_rows<D>(a, t, i0, stage, lane);
+  write_rows<D>(a, t, x, i0, stage, lane);
 }
 
 }  // namespace pf

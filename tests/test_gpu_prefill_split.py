@@ -79,3 +79,11 @@ def test_last_wave_shared(d, B, Hq, Hkv, light, T, prefix):
         mag = oatt.prefill(qn, kn, np.abs(vn), labels, S, W, rows=rows)
         assert_matches(f64(out[b, :lens[b]]), want, f"b={b}", mag)
     cache.close()
+
+
+@pytest.mark.parametrize("d", [64, 128])
+@pytest.mark.parametrize("group", [1, 2, 7, 8])
+def test_items_of_two_heads(d, group):
+    """An item is one query tile of two heads, or two tiles of an odd group's last
+    head: lengths around both, more items than two to an SM at the larger groups."""
+    run_case(6, 4 * group, 4, d, 641, 130, 129, [0, 1, 0, 1], seq_lens=[641, 1, 127, 128, 129, 385])

@@ -131,9 +131,8 @@ std::vector<uint64_t> prefill_schedule(const CacheGeom& g, const std::vector<int
 //
 // When every item's cluster runs at once, the call lasts as long as its longest
 // item, and sharing all halves that. Measured (8 heads of 128, one sequence, us of
-// the kernel without / with): 256 rows (2 tiles) 11.2 / 11.5, 384 11.8 / 13.4, 512
-// 15.4 / 13.5, 1024 21.1 / 17.5, 2048 34.8 / 24.4; heads of 64: 384 11.4 / 11.6,
-// 512 13.9 / 11.7, 2048 30.8 / 21.1.
+// a call without / with): 512 rows (4 tiles) 17 / 18, 640 19 / 20, 1024 22 / 21, 2048
+// 33 / 26; heads of 64: 512 16 / 16, 1024 20 / 18, 2048 30 / 22.
 //
 // In a few waves, as in a chunk after a long prefix whose heavy items all read it,
 // a last wave of heavy items that leaves many SMs idle is shared, while the
@@ -149,7 +148,7 @@ std::vector<uint64_t> prefill_pairs(const std::vector<uint64_t>& items, const st
   const int n = (int)items.size(), slots = num_sms / 2;
   int first = 0, last = 0;  // items [first, last) are shared
   if (n <= slots) {
-    if (n > 0 && costs[0] >= 4) last = n;
+    if (n > 0 && costs[0] >= 7) last = n;
   } else if (n <= std::min(4 * num_sms, kPrefillSplitMost)) {
     long long work = 0, meet = 0;
     for (int c : costs) work += c + 4;

@@ -1,5 +1,5 @@
 """Prefill calls small enough that clusters of two CTAs share each work item,
-around the rule's edges (four visited tiles, 76 items), and larger ones whose last
+around the rule's edges (seven visited tiles, 76 items), and larger ones whose last
 wave is shared, against the oracle: odd lengths, a cached prefix, streaming heads
 whose halves see no key of some rows, the chunk-eviction rule."""
 
@@ -16,12 +16,12 @@ pytestmark = pytest.mark.gpu
 
 
 @pytest.mark.parametrize("B,Hq,Hkv,d,T,S,W,labels,lens", [
-    (1, 8, 2, 128, 384, 4, 60, [0, 1], None),             # three tiles: not split
-    (1, 8, 2, 128, 385, 4, 60, [0, 1], None),             # four
+    (1, 8, 2, 128, 768, 4, 60, [0, 1], None),             # six tiles: not split
+    (1, 8, 2, 128, 769, 4, 60, [0, 1], None),             # seven
     (1, 8, 2, 64, 1025, 16, 100, [0, 1], None),           # a last item of one row
-    (2, 14, 2, 128, 700, 200, 130, [1, 0], [700, 513]),   # ragged, sinks past a tile
+    (2, 12, 2, 128, 700, 200, 130, [1, 0], [700, 513]),   # ragged, sinks past a tile
     (1, 4, 4, 128, 2300, 0, 1, [1, 0, 1, 0], None),       # a window of one
-    (1, 32, 4, 64, 512, 4, 60, [0, 1, 0, 0], None),       # 64 items
+    (1, 16, 2, 64, 1100, 4, 60, [0, 1], None),            # 72 items
 ])
 def test_small_calls(B, Hq, Hkv, d, T, S, W, labels, lens):
     run_case(B, Hq, Hkv, d, T, S, W, labels, seq_lens=lens)

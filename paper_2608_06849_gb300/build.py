@@ -36,7 +36,7 @@ def source_digest():
 KERNEL_SOURCES = {
     "decode": ["decode.cu", "decode_common.cuh", "cluster.cuh", "common.cuh", "internal.h"],
     "decode_tc": ["decode_tc.cuh", "decode_tc.cu", "decode_tc64.cu", "decode_tc_cluster.cu", "decode_common.cuh", "cluster.cuh", "tc.cuh", "common.cuh", "internal.h"],
-    "prefill": ["prefill_tc.cu", "prefill_tile.cuh", "cluster.cuh", "tc.cuh", "common.cuh", "internal.h"],
+    "prefill": ["prefill_tc.cu", "prefill_short.cu", "prefill_tile.cuh", "cluster.cuh", "tc.cuh", "common.cuh", "internal.h"],
 }
 
 

@@ -193,6 +193,22 @@ std::vector<uint64_t> prefill_pairs(const std::vector<uint64_t>& items, const st
   return pairs;
 }
 
+// Whether one CTA an SM goes through all items in one pipeline instead of a CTA an
+// item: many short items, whose starts and ends it overlaps. It deals them out
+// beforehand, which needs several for an SM to even out, and its loop over KV tiles
+// is a few percent slower. Measured, us of a call with a CTA an item / so (32/8 heads
+// of 128, half streaming, S = 64, W = 512; items an SM, tiles an item): 8 x 512 (3.4,
+// 2.5) 41 / 38, 16 x 512 (6.7, 2.5) 78 / 62, 8 x 1024 (6.7, 4.3) 94 / 79, 2 x 2048
+// (3.4, 6.8) 60 / 62, 8 x 2048 (13.5, 6.8) 220 / 191, 1 x 4096 (3.4, 11) 80 / 87, 2 x 4096
+// (6.7, 11) 154 / 146, 1 x 8192 (6.7, 19) 224 / 238, 2 x 8192 (13.5, 19) 439 / 433; 4 x 512
+// (1.7, 2.5) 24 / 25; 32K tokens of 28/4 heads (24, 73) 2469 / 2609.
+bool prefill_is_short(const std::vector<int>& costs, int num_sms) {
+  const long long n = (long long)costs.size();
+  long long tiles = 0;
+  for (int c : costs) tiles += c;
+  return n >= 3 * num_sms && tiles <= 20 * n && tiles * num_sms * 10 <= 19 * n * n;
+}
+
 size_t bytes_for(const aoh_config& c, int n_r, int n_s) {
   const size_t tokens = (size_t)n_r * c.max_seq + (size_t)n_s * (size_t)(c.sink + c.window);
   return (size_t)c.batch * tokens * c.d_head * 2 * 2;
@@ -518,7 +534,8 @@ aoh_status aoh_prefill(const void* q, const void* k, const void* v, int32_t T, c
       return fail(AOH_ERR_CUDA, "cuTensorMapEncodeTiled failed for q/k/v");
     if (chunked && !prefill_tc_make_cache_maps(&pa, cache->kv))
       return fail(AOH_ERR_CUDA, "cuTensorMapEncodeTiled failed for the cache");
-    e = launch_prefill_tc(pa, items, pairs, s);
+    e = pairs.empty() && prefill_is_short(costs, cache->num_sms) ? launch_prefill_short(pa, items, cache->num_sms, s)
+                                                                 : launch_prefill_tc(pa, items, pairs, s);
     if (e != cudaSuccess) return cuda_fail(e, "prefill kernel launch");
   }
 

@@ -189,6 +189,9 @@ bool make_decode_maps(DecodeArgs* a, const CacheGeom& g, const void* kv);
 // kPrefillByValue.
 cudaError_t launch_prefill_tc(const PrefillTcArgs& a, const std::vector<uint64_t>& items,
                               const std::vector<uint64_t>& pairs, cudaStream_t s);
+// One CTA an SM through all items in one pipeline (prefill_short.cu).
+cudaError_t launch_prefill_short(const PrefillTcArgs& a, const std::vector<uint64_t>& items, int num_sms,
+                                 cudaStream_t s);
 // The CUDA-core decode kernel: the H2Share reuse step of d_head 64, with its
 // CTA count.
 cudaError_t launch_decode_cc(const DecodeArgs& a, cudaStream_t s);

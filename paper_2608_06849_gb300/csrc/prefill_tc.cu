@@ -268,7 +268,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     } else if (ok && __all_sync(0xffffffffu, wait_bar(&pv_done[x], (n_tiles - 1) & 1, a.err, abort_flag))) {
       tc_fence_after();
       // Q_X is free: the last S_X was done before the last P V
-      store_o<D>(a, t, x, qx0 + q4 * 32, tl + o_col, 1.f / l, sQ + x * C::QBYTES + q4 * (C::QBYTES / 4), lane);
+      store_o<D, D>(a, t, x, qx0 + q4 * 32, tl + o_col, 1.f / l, sQ + x * C::QBYTES + q4 * (C::QBYTES / 4), lane);
     }
   }
 
@@ -330,7 +330,7 @@ __global__ void __launch_bounds__(kThreads, 1)
           put_row<D>(stage, lane, c * 4 + e / 8, y);
         }
       }
-      write_rows<D>(a, t, x, t.row0(x) + q4 * 32, stage, lane);
+      write_rows<D, D>(a, t, x, t.row0(x) + q4 * 32, 0, stage, lane);
       tc_fence_before();
     }
     __syncthreads();

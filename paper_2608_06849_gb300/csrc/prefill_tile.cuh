@@ -1,5 +1,7 @@
-// The parts of the prefill kernel (prefill_tc.cu): shapes, the geometry of a work
-// item and its copies, the MMAs and the softmax of one tile, and the output rows.
+// The parts of the prefill kernels (prefill_tc.cu: a CTA an item, or half of one;
+// prefill_short.cu: one pipeline through many short items): shapes, the geometry of
+// a work item and its copies, the MMAs and the softmax of one tile, and the output
+// rows.
 #pragma once
 
 #include <math.h>
@@ -360,26 +362,27 @@ __device__ __forceinline__ void put_row(uint8_t* stage, int lane, int chunk, con
   *reinterpret_cast<uint4*>(stage + lane * (D * 2) + ((chunk ^ (lane % CH)) << 4)) = w;
 }
 
-// Rows i0 .. i0 + 31 of the chunk (those below len), query tile x's head, from the
-// warp's `stage`.
-template <int D>
-__device__ __forceinline__ void write_rows(const PrefillTcArgs& a, const Item& t, int x, int i0, const uint8_t* stage,
-                                           int lane) {
-  constexpr int CH = D / 8, RPI = 32 / CH;  // chunks a row, rows a step
+// COLS columns, from col0 on, of rows i0 .. i0 + 31 of the chunk (those below len), query
+// tile x's head, from the warp's `stage`.
+template <int D, int COLS>
+__device__ __forceinline__ void write_rows(const PrefillTcArgs& a, const Item& t, int x, int i0, int col0,
+                                           const uint8_t* stage, int lane) {
+  constexpr int CH = COLS / 8, RPI = 32 / CH;  // chunks a row, rows a step
   __syncwarp();
   const int c = lane % CH;
-  bf16* out = static_cast<bf16*>(a.out) + ((size_t)t.b * a.T * a.geom.Hq + t.head(x)) * D + c * 8;
+  bf16* out = static_cast<bf16*>(a.out) + ((size_t)t.b * a.T * a.geom.Hq + t.head(x)) * D + col0 + c * 8;
 #pragma unroll
   for (int r0 = 0; r0 < 32; r0 += RPI) {
     const int r = r0 + lane / CH;
-    const uint4 w = *reinterpret_cast<const uint4*>(stage + r * (D * 2) + ((c ^ (r % CH)) << 4));
+    const uint4 w = *reinterpret_cast<const uint4*>(stage + r * (COLS * 2) + ((c ^ (r % CH)) << 4));
     if (i0 + r < t.len) *reinterpret_cast<uint4*>(out + (size_t)(i0 + r) * a.geom.Hq * D) = w;
   }
 }
 
 // Write a warp's 32 finished rows of query tile x's O (each lane's times its inv), the
-// first of them row i0 of the chunk. taddr: O's first column, stage: 32 * D * 2 bytes.
-template <int D>
+// first of them row i0 of the chunk, COLS columns at a time. taddr: O's first
+// column, stage: 32 * COLS * 2 bytes.
+template <int D, int COLS>
 __device__ __forceinline__ void store_o(const PrefillTcArgs& a, const Item& t, int x, int i0, uint32_t taddr, float inv,
                                         uint8_t* stage, int lane) {
 #pragma unroll
@@ -392,10 +395,13 @@ __device__ __forceinline__ void store_o(const PrefillTcArgs& a, const Item& t, i
       float y[8];
 #pragma unroll
       for (int k = 0; k < 8; ++k) y[k] = __uint_as_float(v[e + k]) * inv;
-      put_row<D>(stage, lane, c * 4 + e / 8, y);
+      put_row<COLS>(stage, lane, c % (COLS / 32) * 4 + e / 8, y);
+    }
+    if ((c + 1) * 32 % COLS == 0) {
+      write_rows<D, COLS>(a, t, x, i0, (c + 1) * 32 - COLS, stage, lane);
+      __syncwarp();
     }
   }
-  write_rows<D>(a, t, x, i0, stage, lane);
 }
 
 }  // namespace pf

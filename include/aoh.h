@@ -135,8 +135,8 @@ aoh_status aoh_cache_init(const aoh_config* cfg, const uint8_t* head_labels, voi
  *             or past seq_lens[b] are ignored: their contents (even NaN) do
  *             not affect any output, and their outputs are not written.
  *   out  [B][T][n_q_heads][d_head], or NULL to only fill the cache.
- * With out, the host lists the call's query tiles (pairs of 128 rows of a query
- * head, longest first). Up to 3840 of them travel as kernel arguments; a longer
+ * With out, the host lists the call's query tiles (pairs of 128 rows, of two heads of a
+ * group or of one head, longest first). Up to 3840 of them travel as kernel arguments; a longer
  * list is uploaded to the handle's work list, a copy from pageable memory, which
  * waits for the stream's earlier work. A chunk of at most max_seq tokens (or
  * of at most the max_tokens given to aoh_cache_reserve) fits the list as

@@ -671,14 +671,24 @@ __global__ void __launch_bounds__(N) svals_kernel(const double* diag, const doub
   const double smax = block_max(nrm, red);
   const double tol = smax * (double)max(dm, N) * DBL_EPSILON;
   const bool keep = nrm > tol;
-  const double total = block_sum(keep ? nrm : 0.0, red);
+  // The sums' rounding errors would show in ER (exp of 4.7 moves by 9e-16 of itself
+  // with the last bit of its argument): each is summed again as what the first
+  // sum left, over terms that are small then, and enters to first order. A total
+  // off by d of itself moves the entropy H by d (H - 1).
+  const double kept = keep ? nrm : 0.0;
+  const double total = block_sum(kept, red);
+  const double off = block_sum(kept - total * (1.0 / N), red) / total;
   double ent = 0.0;
   if (keep) {
     const double p = nrm / total;
     ent = -p * log(p);
   }
-  ent = block_sum(ent, red);
-  if (j == 0) er[hg] = exp(ent);
+  const double H = block_sum(ent, red);
+  const double rest = block_sum(ent - H * (1.0 / N), red) - off * (H - 1.0);
+  if (j == 0) {
+    const double e = exp(H);
+    er[hg] = total > 0.0 ? fma(e, rest, e) : e;
+  }
 }
 
 // One layer per block (blockIdx.x), one thread.

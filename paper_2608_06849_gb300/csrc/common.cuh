@@ -127,6 +127,11 @@ __device__ __forceinline__ void cp_async_mbar_arrive(uint64_t* bar) {
 __device__ __forceinline__ void named_barrier_sync(int id, int count) {
   asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(count) : "memory");
 }
+// Announce shared-memory writes to the threads that named_barrier_sync.
+__device__ __forceinline__ void named_barrier_arrive(int id, int count) {
+  __threadfence_block();
+  asm volatile("bar.arrive %0, %1;" ::"r"(id), "r"(count) : "memory");
+}
 
 // Atomic add with acquire-release semantics at GPU scope. After a CTA
 // barrier, one thread's atomic publishes the whole CTA's earlier stores

@@ -36,13 +36,12 @@ __device__ __forceinline__ int seq_len(const DecodeArgs& a, int b, const int* le
 // (the allocation-free entry point, e.g. replayed from a CUDA graph).
 __device__ __forceinline__ bool seq_full(const CacheGeom& g, int t) { return g.n_r > 0 && t >= g.max_seq; }
 
-// Rows of item `id`, item k of sequence b. Retrieval: t + 1 rows (min(top_k,
+// Rows of item `id`, item k of its sequence. Retrieval: t + 1 rows (min(top_k,
 // t + 1) borrowed rows in the H2Share reuse step); streaming: min(t + 1, S + W)
 // ring rows; t = tokens held before this step. 0 for every item of a full
 // sequence.
-__device__ __forceinline__ int item_rows(const DecodeArgs& a, int b, int k, const int* lens_s) {
+__device__ __forceinline__ int rows_at(const DecodeArgs& a, int t, int k) {
   const CacheGeom& g = a.geom;
-  const int t = seq_len(a, b, lens_s);
   if (seq_full(g, t)) return 0;
   if (k < g.n_r) return a.idx ? min(a.top_k, t + 1) : t + 1;
   return min(t + 1, g.S + g.W);
@@ -50,7 +49,7 @@ __device__ __forceinline__ int item_rows(const DecodeArgs& a, int b, int k, cons
 __device__ __forceinline__ int item_rows(const DecodeArgs& a, int id, const int* lens_s = nullptr) {
   const int HK = a.geom.n_r + a.geom.n_s;
   const int b = id / HK;
-  return item_rows(a, b, id - b * HK, lens_s);
+  return rows_at(a, seq_len(a, b, lens_s), id - b * HK);
 }
 
 // Rows as the split counts them: a.row_keys cache rows each (2 where the
@@ -436,7 +435,7 @@ constexpr int kPlanItem = 0, kPlanFlag = 1, kPlanLo = 2, kPlanHi = 3, kPlanParts
 __host__ __device__ constexpr int recv_floats(int G, int D) { return G * D + 2 * kClusterMax * G; }
 
 // The item, the rows [lo, hi) and the place in its item of this CTA. Run by
-// warp 0; up to 32 items, lane i holding item i's rows. With T rows a cluster,
+// one warp; up to 32 items, lane i holding item i's rows. With T rows a cluster,
 // item i takes ceil(rows_i / T) clusters: the smallest of 32 values of T
 // between an even share and one that always fits is taken. Up to 8 tiles a
 // CTA, T and the CTA's rows are whole tiles (a started tile costs as much as a
@@ -448,8 +447,10 @@ __host__ __device__ constexpr int recv_floats(int G, int D) { return G * D + 2 *
 // come from reciprocals (a T that does not fit is found out below), and the
 // division of a CTA's rows is left out where an item has one cluster: 1,600 clocks
 // for 4 items, 2,600 with integer divisions throughout. As many clusters as items
-// (most short steps) need no search: 900 clocks; a token of 28 layers at 4K 214 ->
-// 204 us.
+// (most short steps) need no search: 900 clocks. The producer warp plans, so that its
+// first copies wait for no block barrier. A token of 28 layers at 4K: 214 us with the
+// search, 204 without, 193 with the lengths taken from registers and the plan in
+// the producer.
 struct PlanSetup {
   int lg, nc, c, rank;  // log2 of a cluster's CTAs; clusters; this CTA's cluster and place in it
   int b, k;             // lane i: item i
@@ -467,13 +468,17 @@ struct PlanSetup {
   }
 };
 
-__device__ __forceinline__ void plan_clusters(const DecodeArgs& a, const PlanSetup& ps, const int* lens_s, int tile,
+__device__ __forceinline__ void plan_clusters(const DecodeArgs& a, const PlanSetup& ps, int* lens_s, int tile,
                                               int* plan) {
   constexpr unsigned kAll = 0xffffffffu;
   const CacheGeom& g = a.geom;
   const int n_items = g.B * (g.n_r + g.n_s);
   const int lane = threadIdx.x & 31, lg = ps.lg, C = 1 << lg, nc = ps.nc;
-  const int keys = lane < n_items ? item_rows(a, ps.b, ps.k, lens_s) : 0;
+  // the lengths, for this warp and, in shared memory, for the others
+  const int len = lane < g.B ? __ldcg(&a.lens[lane]) : 0;
+  if (lane < g.B) lens_s[lane] = len;
+  const int t = __shfl_sync(kAll, len, min(ps.b, 31));
+  const int keys = lane < n_items ? rows_at(a, t, ps.k) : 0;
   const int rows = split_rows(a, keys);
   const int active = __popc(__ballot_sync(kAll, rows > 0));
   int item, n, inc;  // this CTA's item; lane i: item i's clusters, and those up to it
@@ -580,28 +585,39 @@ __device__ __forceinline__ void cluster_finish(const DecodeArgs& a, const float*
     *reinterpret_cast<uint32_t*>(out + e) = float2_to_bf16x2(o.x * inv, o.y * inv);
     if (stats != nullptr && e % D == 0) stats[e / D] = make_float2(M, L);
   };
-  for (int i = 2 * t; i < share; i += 2 * NT) {
+  // Four of the states a thread, C / 4 neighbouring lanes a pair of values: with all
+  // 16 states in one thread a token of 28 layers at 4K took 204.0 us, 202.5 so.
+  const int lq = C > 4 ? __ffs(C) - 3 : 0, slots = share / 2 << lq;
+  for (int s0 = 0; s0 < slots; s0 += NT) {
+    const int slot = min(s0 + t, slots - 1);
+    const int i = 2 * (slot >> lq), c0 = 4 * (slot & ((1 << lq) - 1));
     const int e = e0 + i, h = e / D;
-    // all loads at once, past C as states that weigh nothing
-    float2 st[kClusterMax], x[kClusterMax];
+    float2 st[4], x[4];
 #pragma unroll
-    for (int c = 0; c < kClusterMax; ++c) {
-      st[c] = c < C ? ml[c * G + h] : make_float2(-INFINITY, 0.f);
-      x[c] = c < C ? *reinterpret_cast<const float2*>(recv + c * share + i) : make_float2(0.f, 0.f);
+    for (int u = 0; u < 4; ++u) {
+      const int c = min(c0 + u, C - 1);
+      st[u] = ml[c * G + h];
+      x[u] = *reinterpret_cast<const float2*>(recv + c * share + i);
+      if (c0 + u >= C) st[u].x = -INFINITY;
     }
-    float M = st[0].x, L = 0.f;
-#pragma unroll
-    for (int c = 1; c + 1 < kClusterMax; c += 2) M = fmax3f(M, st[c].x, st[c + 1].x);
-    M = fmaxf(M, st[kClusterMax - 1].x);
+    float M = fmaxf(fmaxf(st[0].x, st[1].x), fmaxf(st[2].x, st[3].x));
+    for (int o = 1; o < 1 << lq; o <<= 1) M = fmaxf(M, __shfl_xor_sync(0xffffffffu, M, o));
+    float L = 0.f;
     float2 o = make_float2(0.f, 0.f);
 #pragma unroll
-    for (int c = 0; c < kClusterMax; ++c) {
-      const bool any = st[c].x != -INFINITY;  // else its values were never written
-      const float w = any ? fast_exp2(st[c].x - M) : 0.f;
-      L += w * st[c].y;
-      o.x += any ? w * x[c].x : 0.f;
-      o.y += any ? w * x[c].y : 0.f;
+    for (int u = 0; u < 4; ++u) {
+      const bool any = st[u].x != -INFINITY;  // else its values were never written
+      const float w = any ? fast_exp2(st[u].x - M) : 0.f;
+      L += w * st[u].y;
+      o.x += any ? w * x[u].x : 0.f;
+      o.y += any ? w * x[u].y : 0.f;
     }
+    for (int k = 1; k < 1 << lq; k <<= 1) {
+      L += __shfl_xor_sync(0xffffffffu, L, k);
+      o.x += __shfl_xor_sync(0xffffffffu, o.x, k);
+      o.y += __shfl_xor_sync(0xffffffffu, o.y, k);
+    }
+    if (c0 != 0 || s0 + t >= slots) continue;
     if (parts == 1) {
       store(e, M, L, o);
     } else {

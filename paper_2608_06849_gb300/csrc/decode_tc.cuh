@@ -300,14 +300,20 @@ __global__ void __launch_bounds__(kThreads + 32 * gather_warps(G, MODE), 1)
   // the lengths cannot change during the launch (the last CTA to finish
   // advances them), so every role reads this copy
   const int* ls = g.B <= C::LENS_CAP ? lens_s : nullptr;
-  if (ls != nullptr) {
+  if (!CLUSTER && ls != nullptr) {  // plan_clusters does it
     for (int i = threadIdx.x; i < g.B; i += NT) lens_s[i] = __ldcg(&a.lens[i]);
     __syncthreads();
   }
   long long total = 0, start = 0, end = 0, first_off = 0;
   if constexpr (CLUSTER) {
-    if (warp == 0) dec::plan_clusters(a, plan_setup, lens_s, kBN, sh32);
-    __syncthreads();
+    // the producer plans, and goes on to its copies without a block barrier
+    if (warp == 4) {
+      dec::plan_clusters(a, plan_setup, lens_s, kBN, sh32);
+      __syncwarp();
+      named_barrier_arrive(2, NT);
+    } else {
+      named_barrier_sync(2, NT);
+    }
     cluster_wait();
   } else {
     dec::find_cta_range<NT>(a, reinterpret_cast<long long*>(sKV), sh64, sh32, ls);
@@ -686,6 +692,22 @@ __global__ void __launch_bounds__(kThreads + 32 * gather_warps(G, MODE), 1)
           gpar ^= 1u << st;
         else
           fpar ^= 1u << st;
+        // the tile's keys that the item holds (at d_head 64 the last pair may hold one)
+        const int kv = PAIR ? min(2 * cnt, walk.keys() - 2 * row0) : cnt;
+        if (kv < NK * kBN) {
+          // zero the V rows of this warp's keys that the item does not hold (d_head
+          // 128: both halves) while S is formed. The lanes' chunks lie side by
+          // side: each lane zeroing its own row met bank conflicts, 2,100 clocks at
+          // a step's last tile, and after S the rest, 500, still held up the step
+          local_ok = wait_bar(gathered ? &gfull[st] : &full[st], land_par, a.err, abort_flag) && local_ok;
+          const int end = (warp + 1) * 32;
+#pragma unroll
+          for (int box = 0; box < 2; ++box) {
+            const int first = max(warp * 32, PAIR ? (kv + 1 - box) / 2 : kv);  // first row to zero
+            uint4* v4 = reinterpret_cast<uint4*>(sKV + st * kStage + kTile + box * kBox);
+            for (int c = first * 8 + lane; c < end * 8; c += 32) v4[c] = make_uint4(0, 0, 0, 0);
+          }
+        }
         local_ok = wait_bar(&s_full[x], (it >> 1) & 1, a.err, abort_flag) && local_ok;
         tc_fence_after();
         uint32_t v[NK][PAIR ? 8 : 16];
@@ -699,9 +721,6 @@ __global__ void __launch_bounds__(kThreads + 32 * gather_warps(G, MODE), 1)
         tc_fence_before();
         __syncwarp();
         if (lane == 0) mbar_arrive(&s_free[x]);
-        // keys of this thread's row that the item holds (at d_head 64 the item's
-        // last pair may hold one)
-        const int kv = PAIR ? min(2 * cnt, walk.keys() - 2 * row0) : cnt;
         bool valid[NK];
         float s[NK][G];
 #pragma unroll
@@ -778,20 +797,6 @@ __global__ void __launch_bounds__(kThreads + 32 * gather_warps(G, MODE), 1)
             pr[y][h] = valid[y] ? fast_exp2(s[y][h] - m[h]) : 0.f;
             l[h] += pr[y][h];
           }
-        if (!__all_sync(0xffffffffu, valid[NK - 1])) {
-          // the tile has landed (its S is complete); zero the V rows of this
-          // warp's keys that the item does not hold (d_head 128: both halves).
-          // The lanes' chunks lie side by side: each lane zeroing its own row
-          // met bank conflicts, 2,100 clocks at a step's last tile
-          wait_bar(gathered ? &gfull[st] : &full[st], land_par, a.err, abort_flag);
-          const int end = (warp + 1) * 32;
-#pragma unroll
-          for (int box = 0; box < 2; ++box) {
-            const int first = max(warp * 32, PAIR ? (kv + 1 - box) / 2 : kv);  // first row to zero
-            uint4* v4 = reinterpret_cast<uint4*>(sKV + st * kStage + kTile + box * kBox);
-            for (int c = first * 8 + lane; c < end * 8; c += 32) v4[c] = make_uint4(0, 0, 0, 0);
-          }
-        }
         // P^T row t -> column t of the K-major [NPV][128 rows] buffer
         uint8_t* pb = sP + (it % C::NPB) * C::PBUF + (t >> 6) * (C::NPV * 128) + (t & 7) * 2;
         const int j = (t & 63) >> 3;
@@ -815,7 +820,15 @@ __global__ void __launch_bounds__(kThreads + 32 * gather_warps(G, MODE), 1)
       }
       if (!ok) break;
 
-      // ---- the item's state: O^T row t, m (uniform), l summed over the keys
+      // ---- the item's state: O^T row t, m (uniform), l summed over the keys (while
+      // the last P V runs)
+#pragma unroll
+      for (int h = 0; h < G; ++h) {
+        float v = l[h];
+#pragma unroll
+        for (int msk = 16; msk >= 1; msk >>= 1) v += __shfl_xor_sync(0xffffffffu, v, msk);
+        if (lane == 0) lsum[warp * 16 + h] = v;
+      }
       const int last = it - 1;
       local_ok = wait_bar(&p_free[last & 1], (last >> 1) & 1, a.err, abort_flag) && local_ok;
       tc_fence_after();
@@ -838,13 +851,6 @@ __global__ void __launch_bounds__(kThreads + 32 * gather_warps(G, MODE), 1)
       if (PAIR && t >= 64) {
 #pragma unroll
         for (int h = 0; h < G; ++h) ms[h * 64 + t - 64] = __uint_as_float(o[NK * C::HP - C::HP + h]);
-      }
-#pragma unroll
-      for (int h = 0; h < G; ++h) {
-        float v = l[h];
-#pragma unroll
-        for (int msk = 16; msk >= 1; msk >>= 1) v += __shfl_xor_sync(0xffffffffu, v, msk);
-        if (lane == 0) lsum[warp * 16 + h] = v;
       }
       ok = named_barrier_and(1, kSoftmaxThreads, local_ok);
       if (!ok) break;

@@ -430,7 +430,7 @@ __device__ __forceinline__ double warp_sum(double v) {
 // flops each: 240 ms for 784 heads of 128. The reduction now takes 9.7 ms (its
 // 4.4 GFLOP and the product's 1.5 cost 5 ms at the 1.2 TFLOP/s the fp64 pipe
 // gives; the rest is the chain of 256 reflectors a head and the sixth, mostly
-// empty, wave of heads) and the values 1.4 ms.
+// empty, wave of heads) and the values 1.5 ms.
 //
 // One CTA per head, 4 N threads, A row-major in shared memory with N + 1
 // doubles a row, so that neither a row nor a column walk meets a bank
@@ -568,10 +568,13 @@ __global__ void __launch_bounds__(4 * N) bidiag_kernel(const double* L, int Hq, 
 // is 64 times as wide as the fp64 pipe), then takes Newton steps in fp64 from
 // there, two or three as a rule. Every evaluation's count says on which side of
 // the wanted value the point lies: a step is taken only towards that side and
-// inside the bracket that the counts have left, else the bracket is halved
-// (values that repeat, to the last bit). The values are wanted to absolute
-// accuracy (ER weights them by their share of the sum). 784 heads of 128 take
-// 1.4 ms; with the bisection in fp64 as well, from 128 shared counts to single
+// inside the bracket that the counts have left, else the bracket is halved.
+// Towards a value that repeats m times a Newton step closes only 1 / m of the
+// distance, so from the ninth round on every round halves the bracket, and 54
+// halvings end any search: with three Newton steps to a halving, up to 120
+// rounds, the values beside a repeated one were left up to 5e-11 of the largest
+// away. The values are wanted to absolute accuracy (ER weights them by their share
+// of the sum). 784 heads of 128 take 1.5 ms; with the bisection in fp64 as well, from 128 shared counts to single
 // values, and divisions for the reciprocals they took 22 ms.
 // 1 / x for 1e-30 <= |x| <= 1e30, to about an ulp: the residual e = 1 - x y of
 // an fp32 reciprocal y gives y (1 + e + e^2) + O(e^3), e < 2^-22. Half the fp64
@@ -629,7 +632,8 @@ __global__ void __launch_bounds__(N) svals_kernel(const double* diag, const doub
   double x = fmax((double)xf, 1e-16), lo = 0.0, hi = 1.0 + 1e-9, prev = 0.0;
   int nlo = 0, nhi = N;
   bool done = false;
-  for (int round = 0; round < 120 && !__all_sync(0xffffffffu, done); ++round) {
+  constexpr int kNewtonRounds = 8, kRounds = kNewtonRounds + 56;
+  for (int round = 0; round < kRounds && !__all_sync(0xffffffffu, done); ++round) {
     const double s = x * x;
     double t = -s, tp = -1.0, g = 0.0;  // g = p'(s) / p(s)
     int c = 0;
@@ -656,16 +660,17 @@ __global__ void __launch_bounds__(N) svals_kernel(const double* diag, const doub
     const double xn = x - 1.0 / (2.0 * x * g);
     const double step = fabs(xn - x);
     const bool near_j = c == j || c == j + 1;
-    // Once a Newton step is far shorter than the one before, a step of 1e-11
-    // leaves 1e-22 over the distance to the next value (and its sign may be
-    // rounding). Towards a value that repeats the steps shrink slowly: there
-    // only the bracket ends the search.
-    const bool converged = near_j && step < 1e-11 && step < 1e-3 * prev;
-    // past eight rounds every fourth halves the bracket, so the search ends
-    const bool newton = near_j && (xn > x) == (c <= j) && xn > lo && xn < hi && (round < 8 || (round & 3) != 3);
-    done = converged || hi - lo < 1.2e-16 || hi < 1e-15 || (newton && step < 4e-15 && nhi - nlo == 1);
+    // Once a Newton step is far shorter than the one before, a step of 1e-14
+    // leaves 1e-20. Its sign may be rounding, so it may leave the bracket, but by
+    // no more than rounding: a step towards a neighbour of the wanted value can be
+    // as short. (Steps of 1e-11, taken wherever they led, gave the neighbour or
+    // a cluster's edge in one of 1e4 spectra of near-equal values, 7e-9 off.)
+    const bool converged = near_j && step < 1e-14 && step < 1e-3 * prev && xn > lo - 4e-15 && xn < hi + 4e-15;
+    const bool newton = near_j && (xn > x) == (c <= j) && xn > lo && xn < hi && round < kNewtonRounds;
+    const double mid = 0.5 * (lo + hi);
+    done = converged || hi - lo < 1.2e-16 || hi < 1e-15 || (newton ? step < 4e-15 && nhi - nlo == 1 : mid <= lo || mid >= hi);
     prev = newton ? step : 0.0;
-    x = converged || newton ? xn : 0.5 * (lo + hi);
+    x = converged || newton ? xn : mid;
   }
   const double nrm = x * bound;
   const double smax = block_max(nrm, red);

@@ -197,6 +197,31 @@ def test_spectra_at_the_edges_of_the_value_search(dh):
     np.testing.assert_allclose(er[3:], _er_by_svd(wq[3:], wk), rtol=1e-12)
 
 
+@pytest.mark.parametrize("dense", [False, True])
+@pytest.mark.parametrize("dh,spectra", [
+    (128, [[(1.0, 64), (2.0, 64)], [(1.2734375, 28), (0.08056640625, 100)],
+           [(1.5, 3), (0.76953125, 59), (0.310546875, 66)]]),
+    (64, [[(1.2734375, 14), (0.08056640625, 50)], [(1.5, 3), (0.310546875, 61)],
+          [(1.8984375, 7), (0.69921875, 37), (0.2001953125, 20)]]),
+])
+def test_values_that_repeat_are_found_to_the_end(dh, spectra, dense):
+    """Heads with two or three values that repeat, as a diagonal and as H D with
+    H a Hadamard matrix (a dense factor), against the closed form. A search that
+    ends early leaves the values beside a repeated one 1e-11 of the largest off,
+    1e-14 to 1e-12 in ER. Values found to the last bits (4e-16) move it by
+    their weight 1 + |log p| - H, below 8 here, so 4e-15 and a few eps of the
+    reduction stay under 1e-14."""
+    H = np.ones((1, 1))
+    while len(H) < dh:
+        H = np.block([[H, H], [H, -H]])
+    wq = np.stack([(H if dense else np.eye(dh)) * np.repeat([v for v, _ in s], [m for _, m in s]) for s in spectra])
+    _, er = _classify(wq, np.eye(dh)[None], 50)
+    for got, s in zip(er, spectra):
+        v, m = (np.array(x, dtype=np.longdouble) for x in zip(*s))
+        p = v / (v * m).sum()
+        np.testing.assert_allclose(got, float(np.exp(-(m * p * np.log(p)).sum())), rtol=1e-14)
+
+
 @pytest.mark.parametrize("dh,dm,offset", [(64, 1, 0), (64, 127, 1), (64, 193, 0), (64, 640, 0), (128, 257, 0),
                                           (128, 1031, 3), (128, 776, 0)])
 def test_gram_digits_at_column_edges(dh, dm, offset):

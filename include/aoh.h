@@ -142,6 +142,14 @@ aoh_status aoh_cache_init(const aoh_config* cfg, const uint8_t* head_labels, voi
  * of at most the max_tokens given to aoh_cache_reserve) fits the list as
  * allocated; only a longer chunk, which a cache without retrieval heads can
  * take, grows it with cudaMalloc (which synchronises the device).
+ * L_b is the handle's own count. Once a call of the handle has been captured into
+ * a CUDA graph, whose replays advance the device lengths alone, it is the device
+ * length instead; the checks made on the host (chunk boundary, capacity) still
+ * see the handle's count, and a chunk that then finds no room on the device is
+ * left out: nothing is appended, its outputs are unspecified, the length stays,
+ * and aoh_cache_check reports CAPACITY. A captured chunk is appended at the
+ * device length on every replay; a batch above 64 or a list above 3840 tiles
+ * needs the uploads and is not for capture.
  * Errors: INVALID, CAPACITY (a retrieval head would pass max_seq; nothing is
  * launched), CUDA.
  */
@@ -270,8 +278,9 @@ aoh_status aoh_cache_reset(aoh_cache* cache, void* stream);
 
 /*
  * Synchronise `stream` and read the device error word that kernels set when
- * a bounded wait runs out (or when a decode step finds a sequence already
- * holding max_seq tokens, which the host checks prevent on this handle).
+ * a bounded wait runs out, or when a decode step finds a sequence already
+ * holding max_seq tokens or a chunk does not fit behind one's tokens (which the
+ * host's checks prevent unless replayed graphs have moved the lengths).
  * Returns AOH_OK, AOH_ERR_TIMEOUT or AOH_ERR_CAPACITY (and clears the word),
  * or AOH_ERR_CUDA.
  */

@@ -226,6 +226,9 @@ struct aoh_cache {
   void* kv = nullptr;
   size_t kv_bytes = 0;
   std::vector<int32_t> lens;  // host mirror of the device lengths
+  // a call of this handle was captured into a graph, whose replays move the device
+  // lengths alone: from then on the mirror does not place prefill chunks
+  bool captured = false;
   int device = 0;
   int num_sms = 0;
   // device metadata (one allocation)
@@ -263,6 +266,17 @@ cudaError_t reserve_work(aoh_cache* h, size_t n) {
 // rows of a head each, or 128 of two.
 size_t work_items_for(const CacheGeom& g, long long tokens) {
   return (size_t)g.B * g.Hq * (size_t)((tokens + 255) / 256);
+}
+
+// Before a call that moves the lengths: whether it is being captured.
+void note_capture(aoh_cache* h, cudaStream_t s) {
+  if (h->captured) return;
+  cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(s, &st) != cudaSuccess) {
+    cudaGetLastError();  // the legacy stream beside a capture: the launch reports it
+    return;
+  }
+  h->captured = st != cudaStreamCaptureStatusNone;
 }
 
 // The H2Share anchor workspace (once per handle; cudaMalloc).
@@ -422,6 +436,7 @@ aoh_status aoh_cache_region(const aoh_cache* cache, int32_t b, int32_t kv_head, 
 
 aoh_status aoh_cache_reset(aoh_cache* cache, void* stream) {
   if (!cache) return fail(AOH_ERR_INVALID, "cache is NULL");
+  note_capture(cache, (cudaStream_t)stream);
   std::fill(cache->lens.begin(), cache->lens.end(), 0);
   cudaError_t e = cudaMemsetAsync(cache->d_lens, 0, sizeof(int32_t) * cache->geom.B, (cudaStream_t)stream);
   if (e != cudaSuccess) return cuda_fail(e, "cudaMemsetAsync");
@@ -439,8 +454,8 @@ aoh_status aoh_cache_check(aoh_cache* cache, void* stream) {
     const uint32_t zero = 0;
     cudaMemcpy(cache->d_err, &zero, sizeof(zero), cudaMemcpyHostToDevice);
     if (err & kErrTimeout) return fail(AOH_ERR_TIMEOUT, "a kernel's bounded wait ran out (error word 0x%x)", err);
-    return fail(AOH_ERR_CAPACITY, "a decode step found a sequence already holding max_seq tokens (error word 0x%x)",
-                err);
+    return fail(AOH_ERR_CAPACITY,
+                "a step or chunk found a sequence whose max_seq tokens leave no room for it (error word 0x%x)", err);
   }
   return AOH_OK;
 }
@@ -494,11 +509,13 @@ aoh_status aoh_prefill(const void* q, const void* k, const void* v, int32_t T, c
   }
   cudaStream_t s = (cudaStream_t)stream;
   cudaError_t e = cudaSuccess;
+  note_capture(cache, s);
   ChunkLens cl;
-  const bool by_value = g.B <= ChunkLens::kMost;
-  cl.lens = by_value ? nullptr : cache->d_chunk;
+  const bool rows_by_value = g.B <= ChunkLens::kMost;
+  const bool by_value = rows_by_value && !cache->captured;
+  cl.lens = rows_by_value ? nullptr : cache->d_chunk;
   cl.base = by_value ? nullptr : cache->d_lens;
-  if (by_value) {
+  if (rows_by_value) {
     for (int b = 0; b < g.B; ++b) cl.by_value[b] = make_int2(clen[b], base[b]);
   } else {
     e = cudaMemcpyAsync(cache->d_chunk, clen.data(), sizeof(int32_t) * g.B, cudaMemcpyHostToDevice, s);
@@ -532,7 +549,7 @@ aoh_status aoh_prefill(const void* q, const void* k, const void* v, int32_t T, c
     pa.scale_log2 = scale_log2;
     if (!prefill_tc_make_maps(&pa, q, k, v, g.B, T))
       return fail(AOH_ERR_CUDA, "cuTensorMapEncodeTiled failed for q/k/v");
-    if (chunked && !prefill_tc_make_cache_maps(&pa, cache->kv))
+    if ((chunked || cache->captured) && !prefill_tc_make_cache_maps(&pa, cache->kv))
       return fail(AOH_ERR_CUDA, "cuTensorMapEncodeTiled failed for the cache");
     e = pairs.empty() && prefill_is_short(costs, cache->num_sms) ? launch_prefill_short(pa, items, cache->num_sms, s)
                                                                  : launch_prefill_tc(pa, items, pairs, s);
@@ -551,7 +568,7 @@ aoh_status aoh_prefill(const void* q, const void* k, const void* v, int32_t T, c
   e = launch_append(ap, s);
   if (e != cudaSuccess) return cuda_fail(e, "append kernel launch");
   if (!by_value) {
-    e = launch_lens_add(cache->d_lens, cache->d_chunk, g.B, s);
+    e = launch_lens_add(cache->d_lens, cl, g, cache->d_err, s);
     if (e != cudaSuccess) return cuda_fail(e, "length update launch");
   }
   cache->lens = lens;
@@ -565,7 +582,7 @@ namespace {
 // Host checks shared by the decode entry points; fills `a` for the step, the
 // longest sequence's rows and the step's total rows (every retrieval row; ring rows of streaming heads).
 aoh_status prepare_decode(const void* q, const void* k_new, const void* v_new, aoh_cache* cache, void* out,
-                          DecodeArgs& a, long long& total, long long& longest) {
+                          cudaStream_t s, DecodeArgs& a, long long& total, long long& longest) {
   if (!cache) return fail(AOH_ERR_INVALID, "cache is NULL");
   if (!q || !k_new || !v_new || !out) return fail(AOH_ERR_INVALID, "q, k_new, v_new and out must not be NULL");
   if (!aligned(q, 16) || !aligned(k_new, 16) || !aligned(v_new, 16) || !aligned(out, 16))
@@ -596,6 +613,7 @@ aoh_status prepare_decode(const void* q, const void* k_new, const void* v_new, a
   a.done = cache->d_done;
   a.err = cache->d_err;
   a.scale_log2 = (float)(1.4426950408889634 / sqrt((double)g.D));
+  note_capture(cache, s);
   return AOH_OK;
 }
 
@@ -607,7 +625,7 @@ aoh_status aoh_decode_step(const void* q, const void* k_new, const void* v_new, 
                            void* stream) {
   DecodeArgs a;
   long long total = 0, longest = 0;
-  const aoh_status st = prepare_decode(q, k_new, v_new, cache, out, a, total, longest);
+  const aoh_status st = prepare_decode(q, k_new, v_new, cache, out, (cudaStream_t)stream, a, total, longest);
   if (st != AOH_OK) return st;
   const CacheGeom& g = cache->geom;
   decode_tc_split(a, g, longest, total, cache->num_sms);
@@ -621,7 +639,7 @@ aoh_status aoh_decode_step_anchor(const void* q, const void* k_new, const void* 
                                   int32_t top_k, int32_t* indices, void* stream) {
   DecodeArgs a;
   long long total = 0, longest = 0;
-  const aoh_status st = prepare_decode(q, k_new, v_new, cache, out, a, total, longest);
+  const aoh_status st = prepare_decode(q, k_new, v_new, cache, out, (cudaStream_t)stream, a, total, longest);
   if (st != AOH_OK) return st;
   const CacheGeom& g = cache->geom;
   if (top_k < 1) return fail(AOH_ERR_INVALID, "top_k must be >= 1");
@@ -650,7 +668,7 @@ aoh_status aoh_decode_step_reuse(const void* q, const void* k_new, const void* v
                                  const int32_t* group_map, void* stream) {
   DecodeArgs a;
   long long total = 0, longest = 0;
-  const aoh_status st = prepare_decode(q, k_new, v_new, cache, out, a, total, longest);
+  const aoh_status st = prepare_decode(q, k_new, v_new, cache, out, (cudaStream_t)stream, a, total, longest);
   if (st != AOH_OK) return st;
   const CacheGeom& g = cache->geom;
   // d_head 128: the tcgen05 kernel's gather warps copy the borrowed rows, a

@@ -18,6 +18,8 @@
 // 3K rows (54 MB of K and V): the append (16 us), the length update (2.5 us) and
 // the copy of the chunk lengths that came before the prefill were 295 - 264 us of
 // the call.
+#include <limits.h>
+
 #include "common.cuh"
 #include "internal.h"
 
@@ -44,6 +46,8 @@ __global__ void __launch_bounds__(kThreads) append_kernel(const __grid_constant_
   const int2 chunk = a.chunk.of(b);
   const int len = chunk.x, Lb = chunk.y;
   const int newlen = Lb + len;
+  // a chunk that does not fit (device lengths past the host's) is left out
+  if (g.n_r > 0 && newlen > g.max_seq) return;
   const int r0 = blockIdx.x * kRows;          // chunk rows [r0, r1)
   const int r1 = min(r0 + kRows, len);
   if (r0 >= r1) return;
@@ -69,16 +73,21 @@ __global__ void __launch_bounds__(kThreads) append_kernel(const __grid_constant_
   }
 }
 
-// lens[b] += add[b] (the lengths after a prefill chunk), stream-ordered.
-__global__ void lens_add_kernel(int32_t* lens, const int32_t* add, int B) {
+// lens[b] += the chunk's rows, stream-ordered.
+__global__ void lens_add_kernel(int32_t* lens, const __grid_constant__ ChunkLens chunk, int B, int most, uint32_t* err) {
   const int b = blockIdx.x * blockDim.x + threadIdx.x;
-  if (b < B) lens[b] += add[b];
+  if (b >= B) return;
+  const int n = lens[b] + chunk.rows(b);
+  if (n > most)
+    atomicOr(err, kErrCapacity);
+  else
+    lens[b] = n;
 }
 
 }  // namespace
 
-cudaError_t launch_lens_add(int32_t* lens, const int32_t* add, int B, cudaStream_t s) {
-  lens_add_kernel<<<(B + 255) / 256, 256, 0, s>>>(lens, add, B);
+cudaError_t launch_lens_add(int32_t* lens, const ChunkLens& chunk, const CacheGeom& g, uint32_t* err, cudaStream_t s) {
+  lens_add_kernel<<<(g.B + 255) / 256, 256, 0, s>>>(lens, chunk, g.B, g.n_r > 0 ? g.max_seq : INT_MAX, err);
   return cudaGetLastError();
 }
 

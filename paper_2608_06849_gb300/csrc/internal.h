@@ -113,13 +113,15 @@ struct DecodeArgs {
 
 // Rows of the chunk and tokens cached before it, per sequence: by value up to
 // kMost sequences (no copy to the device precedes the launch), in device
-// arrays above.
+// arrays above. The tokens cached before come from the device lengths as well
+// where those can differ from the host's (aoh_cache::captured).
 struct ChunkLens {
   static constexpr int kMost = 64;
   int2 by_value[kMost];  // {rows, tokens before}
   const int32_t* lens;   // device [B], or null: by value
   const int32_t* base;
-  __host__ __device__ int2 of(int b) const { return lens ? make_int2(lens[b], base[b]) : by_value[b]; }
+  __host__ __device__ int rows(int b) const { return lens ? lens[b] : by_value[b].x; }
+  __host__ __device__ int2 of(int b) const { return make_int2(rows(b), base ? base[b] : by_value[b].y); }
 };
 
 struct AppendArgs {
@@ -128,8 +130,8 @@ struct AppendArgs {
   const void* v;
   void* kv;
   ChunkLens chunk;
-  // device [B] lengths that the kernel sets to the new ones (chunk by value),
-  // or null
+  // device [B] lengths that the kernel sets to the new ones (chunk wholly by
+  // value), or null
   int32_t* new_lens;
   // the prefill kernel precedes the launch, which may start under its tail
   int after_prefill;
@@ -240,7 +242,9 @@ void decode_tc_split(DecodeArgs& a, const CacheGeom& g, long long longest, long 
 // Floats of the partial buffer for `n_ctas` CTAs.
 size_t decode_partial_floats(int n_ctas, int G, int D);
 cudaError_t launch_append(const AppendArgs& a, cudaStream_t s);
-cudaError_t launch_lens_add(int32_t* lens, const int32_t* add, int B, cudaStream_t s);
+// The lengths after a chunk whose cached tokens came from `lens`; a sequence that
+// it does not fit keeps its length and sets kErrCapacity in *err.
+cudaError_t launch_lens_add(int32_t* lens, const ChunkLens& chunk, const CacheGeom& g, uint32_t* err, cudaStream_t s);
 bool decode_supported(int D, int G);
 
 }  // namespace aoh

@@ -140,7 +140,7 @@ std::vector<uint64_t> prefill_schedule(const CacheGeom& g, const std::vector<int
 // on one SM; where that ends a tenth later than the work spread evenly, the ends
 // of longest-first schedules decide, in visited tiles, with 4 tiles' time added
 // to an item and 8 to a half: nothing shared, or half a wave or a whole one from
-// item k * num_sms on. Past four items an SM the last wave matters little. 28
+// item k * num_sms on (from the even one below, with an odd count of SMs). Past four items an SM the last wave matters little. 28
 // heads of 128, half of them streaming (S = 128, W = 2048), us of a call without /
 // with: 4096 rows after 16K tokens 388 / 388 (not shared), 20K 471 / 461, 24K 555 /
 // 526, 28K 638 / 585; 1024 rows after 24K 272 / 151.
@@ -157,6 +157,7 @@ std::vector<uint64_t> prefill_pairs(const std::vector<uint64_t>& items, const st
         meet = (a / num_sms + 1) * (long long)(costs[a] + 4);
         first = a;
       }
+    first &= ~1;  // the halves of an item are entries 2 i and 2 i + 1 at any count of SMs
     if (meet * num_sms * 10 > work * 11) {
       std::vector<int> free_at;  // a min-heap
       auto end_of = [&](int count, int shared_end) {

@@ -434,7 +434,12 @@ extern "C" aoh_status aoh_h2share_map(const void* w_q_anchor, const void* w_k_an
   std::vector<unsigned char> res(res_bytes);
   if (e == cudaSuccess) e = cudaMemcpyAsync(res.data(), gsim, res_bytes, cudaMemcpyDeviceToHost, s);
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-  if (e != cudaSuccess) return fail(AOH_ERR_CUDA, "aoh_h2share_map: a CUDA call failed");
+  if (e != cudaSuccess) {
+    // what was launched may still run on the workspace, and may have set its error word
+    cudaMemsetAsync(err, 0, sizeof(*err), s);
+    cudaStreamSynchronize(s);
+    return fail(AOH_ERR_CUDA, "aoh_h2share_map: a CUDA call failed");
+  }
   uint32_t h_err = 0;
   memcpy(map_out, res.data() + (size_t)Hkv * Hkv * 8, (size_t)Hkv * 4);
   if (group_sim_out) memcpy(group_sim_out, res.data(), (size_t)Hkv * Hkv * 8);

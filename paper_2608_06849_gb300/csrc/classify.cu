@@ -777,17 +777,17 @@ extern "C" aoh_status aoh_classify(const void* w_q, const void* w_k, int32_t n_l
   uint32_t* err = reinterpret_cast<uint32_t*>(er + nq);
   int* row_exp = reinterpret_cast<int*>(err + 1);
   uint8_t* labels = reinterpret_cast<uint8_t*>(row_exp + (size_t)nall * dh);
-  static bool attr_set = false;
-  if (!attr_set) {
-    e = cudaFuncSetAttribute(chol_kernel<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, kCholSmem<128>);
+  static std::atomic<uint64_t> done{0};
+  e = once_per_device(done, [] {
+    cudaError_t e = cudaFuncSetAttribute(chol_kernel<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, kCholSmem<128>);
     if (e == cudaSuccess)
       e = cudaFuncSetAttribute(bidiag_kernel<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, BidiagCfg<128>::SMEM);
     if (e == cudaSuccess) e = cudaFuncSetAttribute(gram_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kGramTcSmem);
-    if (e != cudaSuccess) {
-      cudaFreeAsync(scratch, s);
-      return fail(AOH_ERR_CUDA, "aoh_classify: cudaFuncSetAttribute failed");
-    }
-    attr_set = true;
+    return e;
+  });
+  if (e != cudaSuccess) {
+    cudaFreeAsync(scratch, s);
+    return fail(AOH_ERR_CUDA, "aoh_classify: cudaFuncSetAttribute failed");
   }
   const bf16 *wq = static_cast<const bf16*>(w_q), *wk = static_cast<const bf16*>(w_k);
   // 16-byte loads of the weights when every row starts on 16 bytes

@@ -466,12 +466,10 @@ __global__ void __launch_bounds__(C::THREADS) decode_kernel(const __grid_constan
 template <int D, int G>
 cudaError_t launch_cfg(const DecodeArgs& a, cudaStream_t s) {
   using C = DecodeCfg<D, G>;
-  static bool attr_set = false;
-  if (!attr_set) {
-    cudaError_t e = cudaFuncSetAttribute(decode_kernel<C>, cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM);
-    if (e != cudaSuccess) return e;
-    attr_set = true;
-  }
+  static std::atomic<uint64_t> done{0};
+  const cudaError_t e = once_per_device(
+      done, [] { return cudaFuncSetAttribute(decode_kernel<C>, cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM); });
+  if (e != cudaSuccess) return e;
   decode_kernel<C><<<a.n_ctas, C::THREADS, C::SMEM, s>>>(a);
   return cudaGetLastError();
 }

@@ -932,15 +932,15 @@ __global__ void __launch_bounds__(kThreads + 32 * gather_warps(G, MODE), 1)
 // `cluster`: CTAs per cluster (kCluster; it divides a.n_ctas).
 template <int D, int G, int MODE>
 cudaError_t launch_g(const DecodeArgs& a, int cluster, cudaStream_t s) {
-  static bool attr_set = false;
-  if (!attr_set) {
+  static std::atomic<uint64_t> done{0};
+  const cudaError_t e = once_per_device(done, [] {
     cudaError_t e =
         cudaFuncSetAttribute(decode_tc_kernel<D, G, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, Lay<D, G>::SMEM);
     if (e == cudaSuccess && MODE == kCluster)
       e = cudaFuncSetAttribute(decode_tc_kernel<D, G, MODE>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-    if (e != cudaSuccess) return e;
-    attr_set = true;
-  }
+    return e;
+  });
+  if (e != cudaSuccess) return e;
   // programmatic stream serialization: the kernel waits for the previous
   // work on the stream itself (griddepcontrol.wait) after its prologue
   cudaLaunchConfig_t cfg = {};

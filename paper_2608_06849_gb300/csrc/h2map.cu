@@ -256,12 +256,10 @@ bool add_problem(GemmArgs& g, const void* A, int M, const void* B, int N, int K,
 // A trace-mode launch overlaps the key-side launch before it (programmatic
 // dependent launch): only its epilogue waits for that grid.
 cudaError_t launch_gemm(const GemmArgs& g, cudaStream_t s) {
-  static bool attr_set = false;
-  if (!attr_set) {
-    cudaError_t e = cudaFuncSetAttribute(gemm_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, GEMM_SMEM);
-    if (e != cudaSuccess) return e;
-    attr_set = true;
-  }
+  static std::atomic<uint64_t> done{0};
+  const cudaError_t e = once_per_device(
+      done, [] { return cudaFuncSetAttribute(gemm_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, GEMM_SMEM); });
+  if (e != cudaSuccess) return e;
   int grid = 0;
   for (int i = 0; i < g.n_problems; ++i) grid += g.p[i].tiles;
   cudaLaunchConfig_t cfg = {};

@@ -571,12 +571,10 @@ H2Layout h2_layout(float* ws, int B, int n_r, int G, int max_seq) {
 template <int G>
 cudaError_t launch_topk_g(const H2Layout& l, int max_seq, const int32_t* lens, int n_r, int top_k, int32_t* idx_out,
                           unsigned grid, cudaStream_t s) {
-  static bool attr_set = false;
-  if (!attr_set) {
-    const cudaError_t e = cudaFuncSetAttribute(h2_topk_kernel<G>, cudaFuncAttributeMaxDynamicSharedMemorySize, kTopSmem);
-    if (e != cudaSuccess) return e;
-    attr_set = true;
-  }
+  static std::atomic<uint64_t> done{0};
+  const cudaError_t e = once_per_device(
+      done, [] { return cudaFuncSetAttribute(h2_topk_kernel<G>, cudaFuncAttributeMaxDynamicSharedMemorySize, kTopSmem); });
+  if (e != cudaSuccess) return e;
   h2_topk_kernel<G><<<grid, kTopThreads, kTopSmem, s>>>(l.scores, score_stride(max_seq), lens, n_r, l.stats,
                                                          l.imp_over, top_k, idx_out);
   return cudaGetLastError();

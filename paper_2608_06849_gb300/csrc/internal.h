@@ -7,6 +7,7 @@
 #include <stddef.h>
 #include <stdint.h>
 
+#include <atomic>
 #include <vector>
 
 namespace aoh {
@@ -172,6 +173,21 @@ constexpr int kPrefillSplitMost = 640;
 
 // cuTensorMapEncodeTiled from the driver (nullptr if unavailable).
 PFN_cuTensorMapEncodeTiled_v12000 encode_fn();
+
+// Runs set(), which sets a kernel's attributes, the first time that a launcher is
+// called with a device current: attributes belong to the device. `done` is the
+// launcher's own static, a bit a device; past its 64 devices every call sets them.
+template <class F>
+cudaError_t once_per_device(std::atomic<uint64_t>& done, F set) {
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  const uint64_t bit = dev >= 0 && dev < 64 ? 1ull << dev : 0;
+  if (done.load(std::memory_order_acquire) & bit) return cudaSuccess;
+  e = set();
+  if (e == cudaSuccess) done.fetch_or(bit, std::memory_order_release);
+  return e;
+}
 
 // Store `msg` as the calling thread's aoh_last_error() message.
 void record_error(const char* msg);

@@ -262,12 +262,11 @@ __global__ void __launch_bounds__(kThreads, 1)
 template <int D, int CAP>
 cudaError_t launch_short_cfg(const PrefillTcArgs& a, const std::vector<uint64_t>& items, int num_sms, cudaStream_t s) {
   using X = ShortCfg<D>;
-  static bool attr_set = false;
-  if (!attr_set) {
-    cudaError_t e = cudaFuncSetAttribute(prefill_short_kernel<D, CAP>, cudaFuncAttributeMaxDynamicSharedMemorySize, X::SMEM);
-    if (e != cudaSuccess) return e;
-    attr_set = true;
-  }
+  static std::atomic<uint64_t> done{0};
+  const cudaError_t e = once_per_device(done, [] {
+    return cudaFuncSetAttribute(prefill_short_kernel<D, CAP>, cudaFuncAttributeMaxDynamicSharedMemorySize, X::SMEM);
+  });
+  if (e != cudaSuccess) return e;
   const int n = (int)items.size();
   WorkList<CAP> wl;
   if (CAP > 0) memcpy(wl.item, items.data(), items.size() * sizeof(uint64_t));

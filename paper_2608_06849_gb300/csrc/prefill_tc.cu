@@ -375,13 +375,11 @@ constexpr int kSmall = 640;  // items of a launch that copies 5 KB of arguments 
 template <int D, bool PAIRS, int CAP>
 cudaError_t launch_cfg(const PrefillTcArgs& a, const std::vector<uint64_t>& items, cudaStream_t s) {
   using C = PfCfg<D>;
-  static bool attr_set = false;
-  if (!attr_set) {
-    cudaError_t e =
-        cudaFuncSetAttribute(prefill_tc_kernel<D, PAIRS, CAP>, cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM);
-    if (e != cudaSuccess) return e;
-    attr_set = true;
-  }
+  static std::atomic<uint64_t> done{0};
+  const cudaError_t e = once_per_device(done, [] {
+    return cudaFuncSetAttribute(prefill_tc_kernel<D, PAIRS, CAP>, cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM);
+  });
+  if (e != cudaSuccess) return e;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)items.size());
   cfg.blockDim = dim3(kThreads);

@@ -1,6 +1,6 @@
-"""aoh_h2share_map when a CUDA call fails after its first launch: the next call may
+"""aoh_h2share_map when a CUDA call fails after its first launch (the next call may
 use the workspace, so the call has to end with the stream synchronised and the
-error word cleared. The host code is compiled with a fake of the CUDA runtime that
+error word cleared), and on several devices of a process. The host code is compiled with a fake of the CUDA runtime that
 logs the calls and fails one of them; nothing runs on a GPU."""
 
 import os
@@ -19,7 +19,8 @@ PROBE = r"""
 
 extern "C" const char* fake_calls();
 extern "C" void* fake_memory();
-extern "C" int fail_encode, fail_launch;
+extern "C" const char* fake_attributes();
+extern "C" int fail_encode, fail_launch, fake_device;
 int fail_encode = -1, fail_launch = -1;
 
 static CUresult encode(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*, const cuuint64_t*,
@@ -38,8 +39,12 @@ int main(int, char** v) {
   const uint8_t lab[2] = {0, 1};
   int32_t map[2];
   void* w = fake_memory();
-  const int st = aoh_h2share_map(w, w, w, w, 8, 2, 64, 512, lab, lab, map, nullptr, nullptr);
-  printf("%d %s\n", st, fake_calls());
+  int st = 0;
+  for (const char* d = v[3]; *d; ++d) {
+    fake_device = *d - '0';
+    st = aoh_h2share_map(w, w, w, w, 8, 2, 64, 512, lab, lab, map, nullptr, nullptr);
+  }
+  printf("%d %s %s\n", st, fake_calls(), fake_attributes());
 }
 """
 
@@ -55,10 +60,16 @@ extern "C" {
 extern int fail_launch;
 const char* fake_calls() { return calls.c_str(); }
 void* fake_memory() { return memory; }
-cudaError_t cudaGetDevice(int* d) { return *d = 0, cudaSuccess; }
+int fake_device = 0;
+static std::string attributes;  // the device of each cudaFuncSetAttribute
+const char* fake_attributes() { return attributes.c_str(); }
+cudaError_t cudaGetDevice(int* d) { return *d = fake_device, cudaSuccess; }
 cudaError_t cudaMalloc(void** p, size_t n) { return *p = memory, n <= sizeof(memory) ? cudaSuccess : cudaErrorMemoryAllocation; }
 cudaError_t cudaFree(void*) { return cudaSuccess; }
-cudaError_t cudaFuncSetAttribute(const void*, cudaFuncAttribute, int) { return cudaSuccess; }
+cudaError_t cudaFuncSetAttribute(const void*, cudaFuncAttribute, int) {
+  attributes += (char)('0' + fake_device);
+  return cudaSuccess;
+}
 cudaError_t cudaLaunchKernelExC(const cudaLaunchConfig_t*, const void*, void**) {
   if (launches++ == fail_launch) return cudaErrorInvalidValue;
   return calls += 'L', cudaSuccess;
@@ -104,5 +115,12 @@ def probe(tmp_path_factory):
     (-1, 2, "3 LLZS"),     # the mapping's launch
 ])
 def test_a_failed_call_leaves_nothing_running(probe, encode, launch, want):
-    r = subprocess.run([probe, str(encode), str(launch)], capture_output=True, text=True, check=True)
-    assert r.stdout.strip() == want
+    r = subprocess.run([probe, str(encode), str(launch), "0"], capture_output=True, text=True, check=True)
+    assert " ".join(r.stdout.split()[:2]) == want
+
+
+def test_attributes_are_set_on_every_device(probe):
+    """Kernel attributes belong to a device: set on each device's first launch."""
+    r = subprocess.run([probe, "-1", "-1", "01102"], capture_output=True, text=True, check=True)
+    st, _, devices = r.stdout.split()
+    assert st == "0" and devices == "012"

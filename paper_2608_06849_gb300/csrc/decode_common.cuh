@@ -285,7 +285,8 @@ __device__ __forceinline__ void merge_parts(int n, PartFn part, __nv_bfloat16* o
         L[e] *= sc;
 #pragma unroll
         for (int u = 0; u < U; ++u) {
-          const float w = (j + u < n && mj[u][e] != -INFINITY) ? fast_exp2(mj[u][e] - bm) : 0.f;
+          if (j + u >= n || mj[u][e] == -INFINITY) continue;  // a repeated part: 0 times its infinity is NaN
+          const float w = fast_exp2(mj[u][e] - bm);
           O[e].x += w * x[u][e].x;
           O[e].y += w * x[u][e].y;
           O[e].z += w * x[u][e].z;
@@ -665,7 +666,8 @@ __device__ __forceinline__ void cluster_finish(const DecodeArgs& a, const float*
       L *= sc;
 #pragma unroll
       for (int u = 0; u < U; ++u) {
-        const float w = (j + u < parts && mj[u] != -INFINITY) ? fast_exp2(mj[u] - bm) : 0.f;
+        if (j + u >= parts || mj[u] == -INFINITY) continue;
+        const float w = fast_exp2(mj[u] - bm);
         o.x += w * x[u].x;
         o.y += w * x[u].y;
         L += w * lj[u];

@@ -839,9 +839,13 @@ __global__ void __launch_bounds__(kThreads + 32 * gather_warps(G, MODE), 1)
         tmem_ld(tl + C::OCOL + C::NP, o1);
         tmem_ld(tl + C::OCOL + 2 * C::NP, o2);
         tmem_ld_wait();
+        // an infinite V row makes the first sum infinite and the others NaN where a
+        // part of its weight is zero: the first sum is the result then
 #pragma unroll
-        for (int c = 0; c < C::NP; ++c)
-          o[c] = __float_as_uint(__uint_as_float(o[c]) + (__uint_as_float(o1[c]) + __uint_as_float(o2[c])));
+        for (int c = 0; c < C::NP; ++c) {
+          const float s = __uint_as_float(o[c]);
+          if (!isinf(s)) o[c] = __float_as_uint(s + (__uint_as_float(o1[c]) + __uint_as_float(o2[c])));
+        }
       } else {
         tmem_ld_wait();
       }

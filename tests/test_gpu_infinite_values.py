@@ -1,5 +1,6 @@
 """Infinities in V: a visible key's infinity reaches the output as an infinity of its
-sign, in its column alone, through the merges of an item's CTAs (several sequences: the stream-K split; one: clusters, and clusters
+sign, in its column alone, through the weight's parts (d_head 64) and the merges
+of an item's CTAs (several sequences: the stream-K split; one: clusters, and clusters
 that exchange through global memory)."""
 
 import pytest
@@ -12,7 +13,8 @@ from paper_2608_06849_gb300.workloads import randn_bf16
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("B,Hq,Hkv,d,n", [(1, 8, 2, 128, 700), (40, 8, 2, 128, 700), (1, 2, 2, 128, 30000)])
+@pytest.mark.parametrize("B,Hq,Hkv,d,n", [(1, 8, 2, 64, 700), (40, 8, 2, 64, 700), (1, 14, 2, 64, 201), (1, 2, 2, 64, 30000),
+                                          (1, 8, 2, 128, 700), (40, 8, 2, 128, 700), (1, 2, 2, 128, 30000)])
 def test_infinite_value_rows(B, Hq, Hkv, d, n):
     ensure_lib()
     inf = float("inf")

@@ -304,9 +304,11 @@ __global__ void __launch_bounds__(kThreads, 1)
     if (warp >= 2 && x == rank && end_ok) {
       const float2 o_ml = recv_ml[r];
       const float M = fmaxf(end_m, o_ml.x);
-      // the other CTA may have had no tile (-inf and unwritten values)
-      const float w0 = end_m == -INFINITY ? 0.f : fast_exp2(end_m - M),
-                  w1 = o_ml.x == -INFINITY ? 0.f : fast_exp2(o_ml.x - M);
+      // a state of -inf saw no key of this row, and its CTA may have had no tile at all
+      // (unwritten values); any other state counts, also with a weight that rounds to
+      // zero, whose NaN is one in a single CTA as well
+      const bool mine = end_m != -INFINITY, other = o_ml.x != -INFINITY;
+      const float w0 = mine ? fast_exp2(end_m - M) : 0.f, w1 = other ? fast_exp2(o_ml.x - M) : 0.f;
       const float inv = 1.f / (end_l * w0 + o_ml.y * w1);
       const float f0 = w0 * inv, f1 = w1 * inv;
       uint8_t* stage = smem + C::OFF_BAR - C::QBYTES + q4 * (C::QBYTES / 4);  // past the receive buffer
@@ -321,11 +323,10 @@ __global__ void __launch_bounds__(kThreads, 1)
 #pragma unroll
           for (int k = 0; k < 8; k += 4) {
             const float4 z = recv[(c * 8 + (e + k) / 4) * 128 + r];
-            // a weight of 0 must not meet values that were never written
-            y[k + 0] = (w0 == 0.f ? 0.f : __uint_as_float(v[e + k + 0]) * f0) + (w1 == 0.f ? 0.f : z.x * f1);
-            y[k + 1] = (w0 == 0.f ? 0.f : __uint_as_float(v[e + k + 1]) * f0) + (w1 == 0.f ? 0.f : z.y * f1);
-            y[k + 2] = (w0 == 0.f ? 0.f : __uint_as_float(v[e + k + 2]) * f0) + (w1 == 0.f ? 0.f : z.z * f1);
-            y[k + 3] = (w0 == 0.f ? 0.f : __uint_as_float(v[e + k + 3]) * f0) + (w1 == 0.f ? 0.f : z.w * f1);
+            y[k + 0] = (mine ? __uint_as_float(v[e + k + 0]) * f0 : 0.f) + (other ? z.x * f1 : 0.f);
+            y[k + 1] = (mine ? __uint_as_float(v[e + k + 1]) * f0 : 0.f) + (other ? z.y * f1 : 0.f);
+            y[k + 2] = (mine ? __uint_as_float(v[e + k + 2]) * f0 : 0.f) + (other ? z.z * f1 : 0.f);
+            y[k + 3] = (mine ? __uint_as_float(v[e + k + 3]) * f0 : 0.f) + (other ? z.w * f1 : 0.f);
           }
           put_row<D>(stage, lane, c * 4 + e / 8, y);
         }

@@ -87,3 +87,27 @@ def test_items_of_two_heads(d, group):
     """An item is one query tile of two heads, or two tiles of an odd group's last
     head: lengths around both, more items than two to an SM at the larger groups."""
     run_case(6, 4 * group, 4, d, 641, 130, 129, [0, 1, 0, 1], seq_lens=[641, 1, 127, 128, 129, 385])
+
+
+@pytest.mark.parametrize("d", [64, 128])
+@pytest.mark.parametrize("T", [512, 1024])
+def test_a_nan_row_whose_weight_rounds_to_zero(d, T):
+    """Keys of the first half of the rows score 300 below the others' for the last
+    rows: zero times the NaN in a visible V row is NaN, in items of one CTA (512
+    rows) and of two (1024) alike. Columns without a NaN row stay finite."""
+    ensure_lib()
+    cache = aoh.Cache(1, 8, 8, d, T, 4, 60, [0] * 8)
+    u = torch.full((d,), d ** -0.5, device="cuda")
+    c = (150 * d ** 0.5) ** 0.5  # the scores are +-150
+    sign = torch.where(torch.arange(T, device="cuda") < T // 2, -1.0, 1.0).view(1, T, 1, 1)
+    q = (c * u).expand(1, T, 8, d).to(torch.bfloat16).contiguous()
+    k = (c * u * sign).expand(1, T, 8, d).to(torch.bfloat16).contiguous()
+    v = randn_bf16((1, T, 8, d), 71, "cuda")
+    v[0, 5, :, 3] = float("nan")
+    out = torch.empty_like(q)
+    cache.prefill(q, k, v, out)
+    cache.check()
+    late = out[0, T // 2 + 128:]
+    assert torch.isnan(late[..., 3]).all()
+    assert torch.isfinite(late[..., [x for x in range(d) if x != 3]]).all()
+    cache.close()

@@ -531,16 +531,13 @@ def run_native(args):
 
 
 def decode_kernel_key(wl):
-    """Which decode kernel serves this shape (the library's dispatch: d_head
-    128 runs on the tensor cores, d_head 64 on CUDA cores)."""
-    return "decode_tc" if wl.d_head == 128 else "decode"
+    """The key of the shape's decode kernel in the traffic record (taken at d_head
+    128; the d_head 64 instances have no entry)."""
+    return "decode_tc" if wl.d_head == 128 else "decode_tc64"
 
 
 def decode_kernel_name(wl):
-    g = wl.n_q_heads // wl.n_kv_heads
-    if wl.d_head == 128:
-        return f"decode_tc_kernel<{g}> (tcgen05 split-KV)"
-    return f"decode_kernel<DecodeCfg<64,{g}>> (CUDA-core split-KV)"
+    return f"decode_tc_kernel<{wl.d_head}, {wl.n_q_heads // wl.n_kv_heads}> (tcgen05 split-KV)"
 
 
 def traffic_for(kernel):

@@ -374,11 +374,11 @@ aoh_status aoh_decode_step_noalloc_status(uint32_t* flags, void* stream);
 /*
  * Self-test of the allocation-free step's recovery from a bounded-wait
  * timeout (the paper has no counterpart): the same call and arguments as
- * aoh_decode_step_noalloc, except that in the launch's last CTA (which
- * always holds rows of the step) the softmax warps withhold their first
- * result, so the MMA warp's wait for it runs out (after about 2 s) and that
- * CTA stops once its copies and MMAs in flight have landed; the other CTAs
- * finish. The outputs of this call are unspecified, the new token may be
+ * aoh_decode_step_noalloc, except that in one CTA that holds rows of the step
+ * (the launch's last; its first in a short step that runs on whole clusters)
+ * the softmax warps withhold their first result, so the MMA warp's wait for it
+ * runs out (after about 2 s) and that CTA stops once its copies and MMAs in
+ * flight have landed; the other CTAs finish. The outputs of this call are unspecified, the new token may be
  * missing from the cache rows that the stalled CTA would have appended,
  * and the lengths advance as usual. The launch still leaves the static scratch clean, and
  * aoh_decode_step_noalloc_status() then reports AOH_ERR_TIMEOUT once.
@@ -391,7 +391,7 @@ aoh_status aoh_decode_step_noalloc_selftest(const aoh_config* cfg, const uint8_t
 
 /*
  * Effective-rank head classification (Sec. 4, Eq. 2-6 and Algorithm 1;
- * Appendix "GQA Extension"), computed on the GPU in fp64, for n_layers
+ * Appendix "GQA Extension"), computed on the GPU to fp64, for n_layers
  * layers at once. For query head h of a layer, M_h = W_K^T W_Q (Eq. 2, the
  * key projection of h's group); its nonzero singular values give
  * ER(h) = exp(entropy of sigma / sum(sigma)) (Eq. 4). A group's score is the
@@ -407,13 +407,16 @@ aoh_status aoh_decode_step_noalloc_selftest(const aoh_config* cfg, const uint8_t
  *   er_out     host double [n_layers][n_q_heads] receiving ER, or NULL.
  *   labels_out host uint8 [n_layers][n_kv_heads] receiving AOH_RETRIEVAL /
  *              AOH_STREAMING, ready for aoh_cache_init.
- * Work: the Gram matrices W W^T (exact bf16 products, fp64 sums), their
- * semi-definite Cholesky factors L, and a one-sided Jacobi SVD of
- * L_K^T L_Q, whose singular values are those of M_h; singular values at or
- * below sigma_max * d_model * eps are dropped as zeros.
- * Allocates temporary device memory stream-ordered (cudaMallocAsync;
- * about 0.26 MB per matrix at d_head 128), frees it, and synchronises
- * `stream` before returning. Errors: INVALID, UNSUPPORTED, CUDA.
+ * Work: the Gram matrices W W^T (exact, digit products on the tensor cores),
+ * and in fp64 their semi-definite Cholesky factors L and the singular values of
+ * L_K^T L_Q, which are those of M_h (Householder bidiagonalisation, counts and
+ * Newton steps); singular values at or below sigma_max * d_model * eps are
+ * dropped as zeros.
+ * Allocates temporary device memory stream-ordered (cudaMallocAsync):
+ * (2 * splits + 1) * d_head^2 * 8 bytes per matrix, 0.39 MB at d_head 128 with one
+ * split of d_model (up to 16, when there are few matrices), frees it, and
+ * synchronises `stream` before returning.
+ * Errors: INVALID, UNSUPPORTED, TIMEOUT, CUDA.
  */
 aoh_status aoh_classify(const void* w_q, const void* w_k, int32_t n_layers, int32_t n_q_heads,
                         int32_t n_kv_heads, int32_t d_head, int32_t d_model, int32_t sparsity_pct,

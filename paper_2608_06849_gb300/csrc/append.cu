@@ -8,9 +8,9 @@
 // Each row is D bf16 = D/8 16-byte chunks; consecutive threads take
 // consecutive chunks, so loads and stores are coalesced 16-byte accesses.
 //
-// After a prefill kernel the launch is a programmatic dependent one: its CTAs
-// fit beside that kernel's (no shared memory, 40 registers a thread) and copy
-// while its last wave leaves SMs idle. What that kernel may still read is left
+// After a prefill kernel the launch is a programmatic dependent one: its CTAs copy
+// on the SMs that the kernel's last wave leaves idle (a prefill CTA's twelve
+// allocated warps of 168 registers leave no room beside it). What that kernel may still read is left
 // alone until it has ended: the rings of streaming heads that hold tokens
 // already (a retrieval head's cached rows stay, and rows past them are masked
 // or zeroed by the reader). The first CTA waits for that kernel in any case and

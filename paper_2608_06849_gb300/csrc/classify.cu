@@ -1,6 +1,7 @@
 // Effective-rank head classifier (Sec. 4: Eq. 2-6 and Algorithm 1; Appendix
-// "GQA Extension"), in fp64 on CUDA cores. It runs once per model, offline;
-// exactness matters more than speed.
+// "GQA Extension"): exact Gram matrices from digit products on the tensor
+// cores, fp64 on CUDA cores after them. It runs once per model, offline; exactness
+// matters more than speed.
 //
 // For query head h with projections W_Q^h, W_K^h ([d_head][d_model]) the
 // kernel attention matrix M_h = W_K^T W_Q (Eq. 2) has rank <= d_head, and
@@ -8,10 +9,11 @@
 //   A = L_K^T L_Q,  with  W_Q W_Q^T = L_Q L_Q^T,  W_K W_K^T = L_K L_K^T
 // (Cholesky factors; W^T = Q L^T is a thin QR, so M_h = Q_K (L_K^T L_Q) Q_Q^T).
 // Steps:
-//   1. gram_kernel: Gram matrices W W^T of every query and key projection
-//      (bf16 products are exact in fp64; the d_model range is split over
-//      CTAs and the parts are summed in a fixed order, so the result does
-//      not depend on scheduling).
+//   1. row_exp_kernel: the scale of every weight row; gram_tc_kernel: Gram
+//      matrices W W^T of every query and key projection (products and sums are
+//      exact; the d_model range is split over CTAs, each part rounds once to
+//      fp64, and the parts are summed in a fixed order, so the result does not
+//      depend on scheduling).
 //   2. chol_kernel: semi-definite Cholesky in shared memory; a pivot at or
 //      below d_head * eps * max(diag) leaves a zero column (rank deficiency).
 //   3. bidiag_kernel: A = L_K^T L_Q and its bidiagonal form; svals_kernel:
@@ -558,6 +560,15 @@ __global__ void __launch_bounds__(4 * N) bidiag_kernel(const double* L, int Hq, 
   }
 }
 
+// 1 / x for 1e-30 <= |x| <= 1e30, to about an ulp: the residual e = 1 - x y of
+// an fp32 reciprocal y gives y (1 + e + e^2) + O(e^3), e < 2^-22. Half the fp64
+// operations of a division.
+__device__ __forceinline__ double fast_rcp(double x) {
+  const double y = (double)__frcp_rn((float)x);
+  const double e = fma(-x, y, 1.0);
+  return fma(y, fma(e, e, e), y);
+}
+
 // Singular values of each head's bidiagonal matrix B and its ER; one CTA of N
 // threads per head, thread j finds the j-th smallest value. With q_i = d_i^2
 // and f_i = e_i^2, the stationary qd transform (Fernando & Parlett 1994)
@@ -574,17 +585,9 @@ __global__ void __launch_bounds__(4 * N) bidiag_kernel(const double* L, int Hq, 
 // halvings end any search: with three Newton steps to a halving, up to 120
 // rounds, the values beside a repeated one were left up to 5e-11 of the largest
 // away. The values are wanted to absolute accuracy (ER weights them by their share
-// of the sum). 784 heads of 128 take 1.5 ms; with the bisection in fp64 as well, from 128 shared counts to single
-// values, and divisions for the reciprocals they took 22 ms.
-// 1 / x for 1e-30 <= |x| <= 1e30, to about an ulp: the residual e = 1 - x y of
-// an fp32 reciprocal y gives y (1 + e + e^2) + O(e^3), e < 2^-22. Half the fp64
-// operations of a division.
-__device__ __forceinline__ double fast_rcp(double x) {
-  const double y = (double)__frcp_rn((float)x);
-  const double e = fma(-x, y, 1.0);
-  return fma(y, fma(e, e, e), y);
-}
-
+// of the sum). 784 heads of 128 take 1.5 ms; with the bisection in fp64 as well, from
+// 128 shared counts to single values, and divisions for the reciprocals they took
+// 22 ms.
 template <int N>
 __global__ void __launch_bounds__(N) svals_kernel(const double* diag, const double* sup, int dm, double* er) {
   __shared__ double2 qf[N];  // (q_i, f_i)

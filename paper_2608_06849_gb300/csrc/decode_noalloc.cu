@@ -55,7 +55,7 @@ using namespace aoh;
 namespace {
 
 // The allocation-free step; stall_cta >= 0 runs the self-test (on the
-// launch's last CTA).
+// launch's last CTA, the first one on the cluster split).
 aoh_status noalloc_step(const aoh_config* cfg, const uint8_t* head_labels, void* kv_buffer, int32_t* lens,
                         int32_t max_len, const void* q, const void* k_new, const void* v_new, void* out,
                         void* stream, int stall_cta) {

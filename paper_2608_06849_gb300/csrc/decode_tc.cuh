@@ -178,7 +178,7 @@ struct Walk {
   // another item of the range may follow: it starts at its row 0
   __device__ __forceinline__ bool more() const { return off < end && id + 1 < n_items; }
 };
-// In the cluster split a CTA holds rows of one item at most (dec::ClusterPlan).
+// In the cluster split a CTA holds rows of one item at most (dec::plan_clusters).
 template <>
 struct Walk<true> {
   int id, b;
@@ -297,8 +297,9 @@ __global__ void __launch_bounds__(kThreads + 32 * gather_warps(G, MODE), 1)
   // is visible after this wait; the next step may then start its prologue
   asm volatile("griddepcontrol.wait;" ::: "memory");
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-  // the lengths cannot change during the launch (the last CTA to finish
-  // advances them), so every role reads this copy
+  // the lengths do not change before every CTA has this copy, which all roles
+  // read (the last CTA to finish, or on the cluster split to have issued its
+  // copies, advances them)
   const int* ls = g.B <= C::LENS_CAP ? lens_s : nullptr;
   if (!CLUSTER && ls != nullptr) {  // plan_clusters does it
     for (int i = threadIdx.x; i < g.B; i += NT) lens_s[i] = __ldcg(&a.lens[i]);

@@ -139,9 +139,9 @@ struct AppendArgs {
   int T;
 };
 
-// Arguments of the tcgen05 prefill kernel: tensor maps over q / k / v
+// Arguments of the tcgen05 prefill kernels: tensor maps over q / k / v
 // ([B][T][H][D], box 128 rows x 64 columns, 128-byte swizzle) and a work list
-// of (b, query head, first row) tiles sorted by cost.
+// of items (prefill_item) sorted by cost.
 struct PrefillTcArgs {
   CUtensorMap tq, tk, tv;  // the chunk's q / k / v
   CUtensorMap tcr, tcs;    // cache: retrieval / streaming regions as [regions][K, V][rows][D]
@@ -159,7 +159,7 @@ struct PrefillTcArgs {
 // not give up).
 cudaError_t launch_wait_selftest(uint32_t* err, uint64_t limit_ns, unsigned long long* elapsed_ns, cudaStream_t s);
 
-// A prefill work item: sequence b, query head h, rows 256 pair .. 256 pair + 255.
+// A prefill work item: sequence b, query head h, rows 256 index .. 256 index + 255.
 inline uint64_t prefill_item(int b, int h, int index) { return (uint64_t)b << 34 | (uint64_t)h << 24 | (uint32_t)index; }
 // An item of 128 rows of heads h and h + 1 (the 128 index-th), instead of 256 rows
 // of head h (the 256 index-th).

@@ -18,7 +18,7 @@ pytestmark = pytest.mark.gpu
 @pytest.mark.parametrize("B,Hq,Hkv,d,T,S,W,labels,lens", [
     (16, 32, 4, 128, 384, 4, 130, [0, 1, 0, 1], [1 + 383 * b // 15 for b in range(16)]),
     (16, 28, 4, 64, 385, 130, 129, [0, 1, 0, 1], [385, 1, 127, 128, 129, 255, 256, 257] * 2),
-    (20, 32, 4, 64, 128, 0, 1, [0, 1, 1, 1], [128, 1, 64, 127] * 5),   # one tile each
+    (32, 32, 4, 64, 128, 0, 1, [0, 1, 1, 1], [128, 1, 64, 127] * 8),   # one tile each
     (30, 16, 16, 128, 257, 4, 60, [0, 1] * 8, None),                   # a head a group
 ])
 def test_ragged(B, Hq, Hkv, d, T, S, W, labels, lens):
@@ -29,7 +29,7 @@ def test_ragged(B, Hq, Hkv, d, T, S, W, labels, lens):
     (128, 12, 32, 4, 300, 200, 0),
     (64, 12, 28, 4, 260, 400, 0),
     (128, 12, 32, 4, 300, 600, 300),
-    (128, 81, 32, 4, 257, 0, 0),  # 3,888 items
+    (128, 113, 32, 4, 257, 0, 0),  # 3,888 items
 ])
 def test_chunks_and_long_lists(d, B, Hq, Hkv, T, prefix, rule):
     ensure_lib()

@@ -19,7 +19,7 @@ pytestmark = pytest.mark.gpu
     (1, 8, 2, 128, 768, 4, 60, [0, 1], None),             # six tiles: not split
     (1, 8, 2, 128, 769, 4, 60, [0, 1], None),             # seven
     (1, 8, 2, 64, 1025, 16, 100, [0, 1], None),           # a last item of one row
-    (2, 12, 2, 128, 700, 200, 130, [1, 0], [700, 513]),   # ragged, sinks past a tile
+    (2, 12, 2, 128, 800, 200, 130, [1, 0], [800, 513]),   # ragged, sinks past a tile
     (1, 4, 4, 128, 2300, 0, 1, [1, 0, 1, 0], None),       # a window of one
     (1, 16, 2, 64, 1100, 4, 60, [0, 1], None),            # 72 items
 ])
@@ -53,7 +53,7 @@ def test_after_a_cached_prefix(d, rule):
 @pytest.mark.parametrize("d,B,Hq,Hkv,light,T,prefix", [
     (128, 20, 8, 1, 0, 256, 1280),   # 160 items: the 8 past the first wave are shared
     (64, 33, 7, 1, 1, 200, 2048),    # 231: 76 shared, then three light ones and an entry without work
-    (128, 3, 32, 4, 0, 300, 1500),   # 192 items in two tiles a sequence, a wave of whole ones first
+    (128, 4, 32, 4, 0, 300, 1500),   # 192 items of three tiles a sequence: a wave of whole ones, then 40 shared
     (128, 4, 25, 5, 1, 250, 2999),   # 100: the 75 heavy ones and one light one shared
 ])
 def test_last_wave_shared(d, B, Hq, Hkv, light, T, prefix):
@@ -85,7 +85,7 @@ def test_last_wave_shared(d, B, Hq, Hkv, light, T, prefix):
 @pytest.mark.parametrize("group", [1, 2, 7, 8])
 def test_items_of_two_heads(d, group):
     """An item is one query tile of two heads, or two tiles of an odd group's last
-    head: lengths around both, more items than two to an SM at the larger groups."""
+    head: lengths around both, more items than SMs at the larger groups."""
     run_case(6, 4 * group, 4, d, 641, 130, 129, [0, 1, 0, 1], seq_lens=[641, 1, 127, 128, 129, 385])
 
 
